@@ -169,6 +169,8 @@ template <typename T> class OpImpl : public purify_op {
   WorkItem* items = nullptr;
   T* deapod = nullptr;
   C* tw = nullptr;
+  C* tws = nullptr;  // stage twiddles of the half-length transforms (rows; columns from tws_col on)
+  size_t tws_col = 0;
   C* gridA = nullptr;
   C* gridP = nullptr;
   C* gridQ = nullptr;
@@ -256,7 +258,7 @@ template <typename T> class OpImpl : public purify_op {
 
   int partials_cap = 0;
   int size_partials() {
-    const int np = std::max({2 * n_items, row_inv_blocks(g), sara_partials_capacity(g.n, levels),
+    const int np = std::max({2 * n_items, row_inv_blocks<T>(g), sara_partials_capacity(g.n, levels),
                              vec_blocks(9 * N()), tv_partials(g.n), 1});
     if (2 * n_items > bpart_cap) {
       double* bnew = nullptr;
@@ -486,6 +488,9 @@ template <typename T> class OpImpl : public purify_op {
     int rc;
     if ((rc = alloc(&deapod, n))) return rc;
     if ((rc = alloc(&tw, g.K))) return rc;
+    std::vector<C> htws;
+    half_twiddles<T>(n, htws, &tws_col);
+    if ((rc = alloc(&tws, htws.size()))) return rc;
     if ((rc = alloc(&pos, M))) return rc;
     if (!light) {
       if ((rc = alloc(&uv_keep, 2 * size_t(M)))) return rc;
@@ -507,6 +512,7 @@ template <typename T> class OpImpl : public purify_op {
     }
     CK(cudaMemcpyAsync(deapod, hs.data(), n * sizeof(T), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(tw, htw.data(), g.K * sizeof(C), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(tws, htws.data(), htws.size() * sizeof(C), cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(err, 0, 2 * sizeof(int), s));
     CK(cudaMemsetAsync(sc, 0, kNumScalars * sizeof(double), s));
     if (!light) launch_check_finite<double>(uv, 2 * size_t(M), err + 1, s);
@@ -583,13 +589,24 @@ template <typename T> class OpImpl : public purify_op {
   // ---- operator building blocks (enqueue only)
   // F Z S in real form (the image is real): row pairs to half spectra, then
   // the half-spectrum columns to the full padded grid with their mirrors.
+  RowFwdArgs<T> row_fwd_args(const RowPro<T>& pro, const T* dea, C* B) const {
+    return RowFwdArgs<T>{g, pro, dea, B, tw, tws};
+  }
+  ColConvArgs<T> col_conv_args(C* B) const {
+    return ColConvArgs<T>{g, B, khat, khat + size_t(g.K / 2) * g.K, tw, tws + tws_col};
+  }
+  RowInvArgs<T> row_inv_args(const C* B, const T* dea, const RowEp<T>& ep_in) const {
+    RowEp<T> ep = ep_in;
+    if (!ep.err) ep.err = err;
+    return RowInvArgs<T>{g, B, dea, ep, tw, tws, row_inv_blocks<T>(g)};
+  }
   void fwd_grid(const RowPro<T>& pro, cudaStream_t s) {
     if (rec) {
-      record(R_RF, s).rf = RowFwdArgs<T>{g, pro, deapod, gridA, tw, row_pass_nseq(g)};
+      record(R_RF, s).rf = row_fwd_args(pro, deapod, gridA);
       record(R_CF, s).cf = ColFwdArgs<T>{g, gridA, gridP, tw, col_pass_width<T>()};
       return;
     }
-    PROF(KK_ROW_FWD, s, launch_row_fwd_h<T>(g, pro, deapod, gridA, tw, s));
+    PROF(KK_ROW_FWD, s, launch_row_fwd_h<T>(row_fwd_args(pro, deapod, gridA), s));
     PROF(KK_COL_FWD, s, launch_col_fwd_h<T>(g, gridA, gridP, tw, s));
   }
   void zero_q(cudaStream_t s) {
@@ -642,16 +659,11 @@ template <typename T> class OpImpl : public purify_op {
     PROF(KK_GRAM, s, launch_gram<T>(g, tmap, items, n_items, pos, kb, gridQ, err, s));
     col_inv(s);
   }
-  int row_ep(const RowEp<T>& ep_in, cudaStream_t s) {
-    RowEp<T> ep = ep_in;
-    if (!ep.err) ep.err = err;
-    if (rec) {
-      record(R_RI, s).ri = RowInvArgs<T>{g, gridA, deapod, ep, tw, row_pass_nseq(g), row_inv_blocks(g)};
-      return row_inv_blocks(g);
-    }
-    int np = 0;
-    PROF(KK_ROW_INV, s, np = launch_row_inv_h<T>(g, gridA, deapod, ep, tw, s));
-    return np;
+  int row_ep(const RowEp<T>& ep, cudaStream_t s) {
+    const RowInvArgs<T> a = row_inv_args(gridA, deapod, ep);
+    if (rec) record(R_RI, s).ri = a;
+    else PROF(KK_ROW_INV, s, launch_row_inv_h<T>(a, s));
+    return a.nblocks;
   }
 
   // Set-up of the convolution form of Re(Phi^H Phi): the PSF
@@ -709,29 +721,23 @@ template <typename T> class OpImpl : public purify_op {
   void normal_front(const RowPro<T>& pro, cudaStream_t s, C* B = nullptr) {
     if (!B) B = gridA;
     if (rec) {  // the batched solver takes the convolution form only
-      record(R_RF, s).rf = RowFwdArgs<T>{g, pro, nullptr, B, tw, row_pass_nseq(g)};
-      record(R_CC, s).cc = ColConvArgs<T>{g, B, khat, khat + size_t(g.K / 2) * g.K, tw, col_pass_width<T>()};
+      record(R_RF, s).rf = row_fwd_args(pro, nullptr, B);
+      record(R_CC, s).cc = col_conv_args(B);
       return;
     }
     if (toep) {
-      PROF(KK_ROW_FWD_H, s, launch_row_fwd_h<T>(g, pro, nullptr, B, tw, s));
-      PROF(KK_COL_CONV, s, launch_col_conv_h<T>(g, B, khat, tw, s));
+      PROF(KK_ROW_FWD_H, s, launch_row_fwd_h<T>(row_fwd_args(pro, nullptr, B), s));
+      PROF(KK_COL_CONV, s, launch_col_conv_h<T>(col_conv_args(B), s));
     } else {
       gram_front(pro, s);
     }
   }
-  int normal_back(const RowEp<T>& ep_in, cudaStream_t s, C* B = nullptr) {
-    RowEp<T> ep = ep_in;
-    if (!ep.err) ep.err = err;
-    if (!B) B = gridA;
-    if (rec) {
-      record(R_RI, s).ri = RowInvArgs<T>{g, B, nullptr, ep, tw, row_pass_nseq(g), row_inv_blocks(g)};
-      return row_inv_blocks(g);
-    }
-    int np = 0;
-    if (toep) PROF(KK_ROW_INV_H, s, np = launch_row_inv_h<T>(g, B, nullptr, ep, tw, s));
-    else PROF(KK_ROW_INV, s, np = launch_row_inv_h<T>(g, gridA, deapod, ep, tw, s));
-    return np;
+  int normal_back(const RowEp<T>& ep, cudaStream_t s, C* B = nullptr) {
+    if (!toep && !rec) return row_ep(ep, s);
+    const RowInvArgs<T> a = row_inv_args(B ? B : gridA, nullptr, ep);
+    if (rec) record(R_RI, s).ri = a;
+    else PROF(KK_ROW_INV_H, s, launch_row_inv_h<T>(a, s));
+    return a.nblocks;
   }
 
   // out = (nu2 Re Phi^H Phi + 2I) x

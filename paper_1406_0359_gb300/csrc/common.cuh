@@ -23,6 +23,24 @@ template <typename C> PD C cmul(C a, C b) {
   r.y = a.x * b.y + a.y * b.x;
   return r;
 }
+// FP32 pairs by one packed instruction (same rounding; half the issue slots
+// and code of two scalar ones).
+PD float2 cadd(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n"
+      " mov.b64 {%0, %1}, z;\n}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+PD float2 csub(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n sub.rn.f32x2 z, x, y;\n"
+      " mov.b64 {%0, %1}, z;\n}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
 template <typename C, typename T> PD C cscale(C a, T s) { a.x *= s; a.y *= s; return a; }
 template <typename C> PD C cmul_i(C a) { C r; r.x = -a.y; r.y = a.x; return r; }  // i * a
 

@@ -1,16 +1,13 @@
 // Oversampled 2D FFT passes of the NUFFT (operator F of Phi = G F Z S, Section 4).
 //
-// Each length-K transform (K = 2n, a power of two) is a Stockham sequence of
-// register radix-E stages (E = 8 or 16; one smaller stage last when log2 K
-// is not a multiple of log2 E).  A thread always holds the E elements
-// t + m K/E of its sequence: the first stage reads them straight from global
-// memory, the last writes its outputs straight to global memory, and the
-// stages in between exchange through shared memory (padded every 16
-// elements against bank conflicts).
+// The row passes and the convolution's column pass transform by halves (even
+// and odd frequencies apart, see "half-length transforms" below); the column
+// passes of Phi and Phi^H run length-K (K = 2n, a power of two) Stockham
+// sequences of register radix-16 stages with shared-memory exchanges.
 //
 // The image is real, so every pass works in real form: two image rows a, b
 // travel as one complex row x_a + i x_b, and only the half spectra (columns
-// 0..K/2 of the row transforms) are kept, n x K/2 complex values.
+// 0..K/2 of the row transforms) are kept, n x K/2 complex values, transposed.
 // Forward (Phi):   row pass over the n non-zero image rows (pairs), fused with
 //                  the deapodisation S and zero-padding Z; column pass over
 //                  the K/2 half-spectrum columns, writing each grid column
@@ -22,6 +19,9 @@
 //                  writing only the n rows the crop Z^T keeps; row pass
 //                  fused with the crop, the deapodisation and the solver
 //                  epilogues.
+#include <cmath>
+#include <vector>
+
 #include "internal.h"
 #include "solver_kernels.h"
 
@@ -118,6 +118,47 @@ template <typename C> struct Dft<16, C> {
   }
 };
 
+// cos / sin of 2 pi m / 32 with the sign of `dir`, for the fixed m of the radix-32 butterfly
+template <typename C> PD C w32(int m, int dir) {
+  typedef decltype(C().x) T;
+  constexpr double c[9] = {1.0,
+                           0.98078528040323044913,
+                           0.92387953251128675613,
+                           0.83146961230254523708,
+                           0.70710678118654752440,
+                           0.55557023301960222474,
+                           0.38268343236508977173,
+                           0.19509032201612826785,
+                           0.0};
+  const int q = (m >> 3) & 3, f = m & 7;  // quadrant, angle within it
+  const double a = c[f], b = c[8 - f];
+  const T re = T(q == 0 ? a : (q == 1 ? -b : (q == 2 ? -a : b)));
+  const T im = T(q == 0 ? b : (q == 1 ? a : (q == 2 ? -b : -a)));
+  return cmk<C>(re, dir < 0 ? -im : im);
+}
+template <typename C> struct Dft<32, C> {
+  // 32 = 4 x 8: 4-point DFTs on (n2, n2+8, n2+16, n2+24), twiddle W32^(n2 k1), 8-point DFTs
+  static PD void run(C* a, int o, int st, int dir) {
+#pragma unroll
+    for (int n2 = 0; n2 < 8; ++n2)
+      dft4(a[o + n2 * st], a[o + (n2 + 8) * st], a[o + (n2 + 16) * st], a[o + (n2 + 24) * st], dir);
+#pragma unroll
+    for (int n2 = 1; n2 < 8; ++n2)
+#pragma unroll
+      for (int k1 = 1; k1 < 4; ++k1)
+        a[o + (n2 + 8 * k1) * st] = cmul(a[o + (n2 + 8 * k1) * st], w32<C>(n2 * k1, dir));
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) Dft<8, C>::run(a, o + 8 * k1 * st, st, dir);
+    C t[32];  // X[k1 + 4 k2] = a[8 k1 + k2]
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1)
+#pragma unroll
+      for (int k2 = 0; k2 < 8; ++k2) t[k1 + 4 * k2] = a[o + (8 * k1 + k2) * st];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) a[o + k * st] = t[k];
+  }
+};
+
 PD int sidx(int e) { return e + (e >> 4); }  // padded shared index
 
 // Compile-time plan of a length-2^LOGN transform with E (8 or 16) elements
@@ -206,11 +247,7 @@ template <int LOGN, int E = 16> PD int last_pos(int t, int cnt) {
   return t + (cnt / R) * P::T + (cnt % R) * (P::N / R);
 }
 
-constexpr int kRowCta = 256;
-constexpr int kRowE = 8;  // elements per thread in the real-form row passes
-// ... unless a row of K / 8 threads would not fit one CTA (K = 4096): 16 there.
-template <int LOGN> constexpr int row_e() { return (1 << LOGN) / kRowE <= kRowCta ? kRowE : 16; }
-inline int row_e_host(int K) { return K / kRowE <= kRowCta ? kRowE : 16; }
+constexpr int kRowCta = 256;  // threads per CTA of the plain row transforms
 
 // Column passes read kColBytes contiguous bytes of each row: col_width
 // interleaved columns per CTA.
@@ -220,111 +257,322 @@ __host__ __device__ inline size_t padded(int N) { return size_t(N) + size_t(N) /
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
-// Row-pass epilogues (see RowEpMode): per output, its operands (EpOpd, from
-// the rows staged in shared memory) and the stores and partial sums of the
-// mode.
-template <typename T> struct EpOpd { T a, b; };
-template <typename T> struct EpAcc { Acc<T> a[5]; };
-template <int MODE, typename T>
-PD void row_ep_store(const RowEp<T>& ep, size_t idx, T val, EpOpd<T> opd, EpAcc<T>& part) {
-  if constexpr (MODE == EP_CG_AP) {
-    // A thread's 16 terms are summed by plain FMAs (their rounding errors are
-    // independent across the ~10^5 threads and average out); the per-thread
-    // sums are then merged compensated.
-    const T o = T(ep.nu2) * val + T(2) * opd.a;  // (A p)_i
-    ep.out[idx] = o;
-    part.a[0].s = fma(opd.a, o, part.a[0].s);
-    part.a[1].s = fma(opd.b, o, part.a[1].s);
-    part.a[2].s = fma(o, o, part.a[2].s);
-    part.a[3].s = fma(opd.b, opd.a, part.a[3].s);
-    part.a[4].s = fma(opd.b, opd.b, part.a[4].s);
-  } else if constexpr (MODE == EP_CG_R0) {
-    const T o = opd.a - T(ep.nu2) * val;
-    ep.out[idx] = o;
-    ep.out2[idx] = o;
-    part.a[0].add_prod(o, o);
-  } else if constexpr (MODE == EP_POWER) {
-    ep.out[idx] = val;
-    part.a[0].add_prod(val, val);
-  } else if constexpr (MODE == EP_XS_ADD) {
-    ep.out[idx] = opd.a + T(ep.nu) * val;
-  } else if constexpr (MODE == EP_QX) {
-    ep.out[idx] = T(ep.nu2) * val + T(2) * opd.a;
-  } else {
-    ep.out[idx] = val;
+// ------------------------------------------------- half-length transforms
+// An image row (or column) holds n values on the K = 2n grid, the rest zero,
+// and only n of the inverse transform's outputs are kept.  Splitting the
+// frequencies by parity turns either into two independent length-n
+// transforms: with the pixel's signed position p in [-n/2, n/2) taken modulo n
+// as the sequence index,
+//   Z(2m)     = sum_p z_p          exp(-2 pi i m p / n),
+//   Z(2m + 1) = sum_p z_p omega^p  exp(-2 pi i m p / n),  omega = exp(-2 pi i / K),
+// and the inverse's output at p is E(p) + conj(omega^p) O(p) from the two
+// length-n inverse transforms.  No zero is ever transformed, the two halves
+// meet only once (in the sum of the inverse), and because the mirror -k of a
+// frequency has k's parity, the separation of a row pair's half spectra stays
+// inside each half.
+//
+// One half is transformed by TT = n / E threads holding E elements each
+// (element j = t + TT m in register m, before and after every transform), in
+// radix-E stages with shared-memory exchanges between them: at n = 1024 one
+// warp, two radix-32 stages and one exchange, with no CTA barrier inside (the
+// length-2048 form of four radix-8 / three radix-16 stages spent its time on
+// barriers, exchanges and scattered twiddle gathers).  The twiddles of stage
+// st come from a table laid out [r - 1][k], so a warp's reads are contiguous.
+template <typename T, int LOGN, int E_> struct Half {
+  static constexpr int E = E_;
+  static constexpr int LE = E == 32 ? 5 : (E == 16 ? 4 : 3);
+  static constexpr int N = 1 << LOGN;
+  static constexpr int TT = N / E;
+  static constexpr int NST = (LOGN + LE - 1) / LE;
+  static constexpr int V = 16 / int(sizeof(T));  // reals per 16-byte vector
+  // elements of one half's exchange buffer (one pad element every E: the
+  // first exchange writes at a stride of E)
+  static constexpr int BUF = N + N / E;
+  __host__ __device__ static constexpr int radix(int st) {
+    return st + 1 < NST ? E : (1 << (LOGN - LE * (NST - 1)));
+  }
+  // row pairs of one row-pass CTA: at least a warp of threads, and enough
+  // rows to fill a 32-byte sector of a transposed column (4 rows FP32, 2 FP64)
+  static constexpr int PMIN = sizeof(T) == 4 ? 2 : 1;
+  static constexpr int PW = 32 / (2 * TT) > 1 ? 32 / (2 * TT) : 1;
+  static constexpr int PAIRS0 = PW > PMIN ? PW : PMIN;
+  static constexpr int PAIRS = PAIRS0 > N / 2 ? N / 2 : PAIRS0;
+  static constexpr int ROW_THREADS = 2 * TT * PAIRS;
+  // columns of one convolution CTA: at least a warp
+  static constexpr int COLS = PW;
+  static constexpr int COL_THREADS = 2 * TT * COLS;
+  // 512 threads' worth of CTAs per SM: 128 registers per thread
+  static constexpr int ROW_MINB = ROW_THREADS >= 512 ? 1 : (512 / ROW_THREADS > 16 ? 16 : 512 / ROW_THREADS);
+  static constexpr int COL_MINB = COL_THREADS >= 512 ? 1 : (512 / COL_THREADS > 16 ? 16 : 512 / COL_THREADS);
+};
+
+// Elements per thread.  Small images leave most of the chip idle, so more
+// threads with fewer elements win (n = 512: Phi^H Phi 11.1 us with 8 / 16
+// elements in the row / column passes against 14.0 with 32); at n = 1024 the
+// row passes measured the same with 16 and 32 and the column pass, whose 1024
+// columns fill the chip, is faster with one exchange per transform than with
+// two (22.2 against 22.8 us).  FP64 elements are twice as wide: 16 at most.
+template <typename T, int LOGN> struct RowHalf : Half<T, LOGN, LOGN <= 9 ? 8 : 16> {};
+template <typename T, int LOGN>
+struct ColHalf : Half<T, LOGN, LOGN <= 8 ? 8 : (LOGN <= 9 || sizeof(T) == 8 ? 16 : 32)> {};
+
+// Barrier of one half's threads: they share a warp, or are whole warps.
+template <int TT> PD void half_sync(int half) {
+  if constexpr (TT <= 32) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(half + 1), "n"(TT) : "memory");
+}
+
+// One stage: R-point DFTs over registers q + r Q (element j = t + q TT of each
+// is r N/R apart), twiddled by W(r k), k = j mod Ns.
+template <typename H, int R, int NS, int DIR, typename C>
+PD void half_stage(C (&v)[H::E], int t, const C* __restrict__ tab) {
+  constexpr int Q = H::E / R;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    if constexpr (NS > 1) {
+      const int k = (t + q * H::TT) & (NS - 1);
+#pragma unroll
+      for (int r = 1; r < R; ++r) {
+        C w = tab[(r - 1) * NS + k];
+        if (DIR > 0) w.y = -w.y;
+        v[q + r * Q] = cmul(v[q + r * Q], w);
+      }
+    }
+    Dft<R, C>::run(v, q, Q, DIR);
   }
 }
-// Image column of the m-th output of thread t of an inverse row pass (grid
-// column q maps to image column (q + K/4) mod K, kept when < n = K/2).
-template <int LOGN, int E = 16> PD int ep_col(int t, int m) {
-  constexpr int K = 1 << LOGN;
-  return (last_pos<LOGN, E>(t, m) + K / 4) & (K - 1);
+
+// All stages; s is the half's exchange buffer, free to be overwritten.  The
+// last stage leaves output j = t + TT m in register m, as the input was.
+template <typename H, int DIR, int ST = 0, int NS = 1, typename C>
+PD void half_fft(C (&v)[H::E], int t, C* s, int half, const C* __restrict__ tab) {
+  constexpr int R = H::radix(ST);
+  half_stage<H, R, NS, DIR>(v, t, tab);
+  if constexpr (ST + 1 < H::NST) {
+    constexpr int Q = H::E / R;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int j = t + q * H::TT, k = j & (NS - 1), base = (j - k) * R + k;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int e = base + r * NS;
+        s[e + (e >> H::LE)] = v[q + r * Q];
+      }
+    }
+    half_sync<H::TT>(half);
+#pragma unroll
+    for (int m = 0; m < H::E; ++m) {
+      const int e = t + m * H::TT;
+      v[m] = s[e + (e >> H::LE)];
+    }
+    half_sync<H::TT>(half);
+    half_fft<H, DIR, ST + 1, NS * R>(v, t, s, half, tab + (NS > 1 ? (R - 1) * NS : 0));
+  }
 }
 
-// Register slot m of the j-th of the E/2 grid columns of a thread that hold
-// image pixels: with K = 2n, grid column q = t + m K/E holds image column
-// i2 = (q + K/4) mod K, inside the image for m < E/4 and m >= 3E/4 only.
-template <int E> PD constexpr int kept_slot(int j) { return j < E / 4 ? j : j + E / 2; }
-
-// Forward row prologue (see RowProMode) of image rows row0[r] at the E/2
-// kept grid columns of thread t.  All loads precede the CG step's stores.
-template <int LOGN, int NR, int E, typename T>
-PD void row_prologue(const RowPro<T>& pro, const size_t (&row0)[NR], int t, T (&val)[NR][E / 2], int (&i2)[E / 2]) {
-  constexpr int K = 1 << LOGN, TT = K / E;
+// omega^p (DIR -1) or its conjugate (DIR +1) at element j = t + TT m, from the
+// table tw[j] = exp(-2 pi i j / K); positions past n/2 are p = j - n: a sign.
+template <typename H, int DIR, typename C> PD void half_omega(C (&v)[H::E], int t, const C* __restrict__ tw) {
 #pragma unroll
-  for (int j = 0; j < E / 2; ++j) i2[j] = (t + kept_slot<E>(j) * TT + K / 4) & (K - 1);
+  for (int m = 0; m < H::E; ++m) {
+    C w = tw[t + m * H::TT];
+    if (DIR > 0) w.y = -w.y;
+    if (m >= H::E / 2) w = cneg(w);
+    v[m] = cmul(v[m], w);
+  }
+}
+
+// 16-byte vectors of reals; `al` says the address is 16-byte aligned (a
+// caller's array need not be).
+template <typename T> struct V16;
+template <> struct V16<float> { typedef float4 type; };
+template <> struct V16<double> { typedef double2 type; };
+template <typename T, int V> PD void vload(T (&d)[V], const T* p, bool al) {
+  if (al) {
+    const typename V16<T>::type x = *reinterpret_cast<const typename V16<T>::type*>(p);
+    const T* e = reinterpret_cast<const T*>(&x);
+#pragma unroll
+    for (int k = 0; k < V; ++k) d[k] = e[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < V; ++k) d[k] = p[k];
+  }
+}
+template <typename T, int V> PD void vstore(T* p, const T (&d)[V], bool al) {
+  if (al) {
+    typename V16<T>::type x;
+    T* e = reinterpret_cast<T*>(&x);
+#pragma unroll
+    for (int k = 0; k < V; ++k) e[k] = d[k];
+    *reinterpret_cast<typename V16<T>::type*>(p) = x;
+  } else {
+#pragma unroll
+    for (int k = 0; k < V; ++k) p[k] = d[k];
+  }
+}
+PD bool aligned16(const void* p) { return (reinterpret_cast<size_t>(p) & 15) == 0; }
+
+// V consecutive complex values in shared memory, by 16-byte accesses.
+template <typename C, int V> PD void cload(C (&d)[V], const C* p) {
+  constexpr int W = 16 / int(sizeof(C));
+  typedef typename V16<decltype(C().x)>::type X;
+#pragma unroll
+  for (int k = 0; k < V; k += W) {
+    const X x = *reinterpret_cast<const X*>(p + k);
+    const C* e = reinterpret_cast<const C*>(&x);
+#pragma unroll
+    for (int q = 0; q < W; ++q) d[k + q] = e[q];
+  }
+}
+template <typename C, int V> PD void cstore(C* p, const C (&d)[V]) {
+  constexpr int W = 16 / int(sizeof(C));
+  typedef typename V16<decltype(C().x)>::type X;
+#pragma unroll
+  for (int k = 0; k < V; k += W) {
+    X x;
+    C* e = reinterpret_cast<C*>(&x);
+#pragma unroll
+    for (int q = 0; q < W; ++q) e[q] = d[k + q];
+    *reinterpret_cast<X*>(p + k) = x;
+  }
+}
+
+// 32-byte global accesses (one sector): 4 complex floats or 2 complex doubles.
+PD void ld32(float2 (&d)[4], const float2* p) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(d[0].x), "=f"(d[0].y), "=f"(d[1].x), "=f"(d[1].y), "=f"(d[2].x), "=f"(d[2].y), "=f"(d[3].x),
+                 "=f"(d[3].y)
+               : "l"(p));
+}
+PD void ld32(double2 (&d)[2], const double2* p) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(d[0].x), "=d"(d[0].y), "=d"(d[1].x), "=d"(d[1].y)
+               : "l"(p));
+}
+PD void st32(float2* p, const float2 (&d)[4]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(d[0].x), "f"(d[0].y),
+               "f"(d[1].x), "f"(d[1].y), "f"(d[2].x), "f"(d[2].y), "f"(d[3].x), "f"(d[3].y)
+               : "memory");
+}
+PD void st32(double2* p, const double2 (&d)[2]) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(d[0].x), "d"(d[0].y), "d"(d[1].x),
+               "d"(d[1].y)
+               : "memory");
+}
+
+// Element (column c, row i) of the half-spectrum buffer B: stored transposed,
+// each column's n rows contiguous, the even columns before the odd ones --
+// the column passes read and write whole lines, and the row passes whole
+// 32-byte sectors (2 PAIRS rows of a column).
+PD size_t half_at(int c, int i, int n) { return (size_t(c & 1) * (n / 2) + (c >> 1)) * n + i; }
+
+// Row-pass epilogues (see RowEpMode): the outputs of V consecutive pixels
+// from their transform values and operands (a, b: see ep_staged), and the
+// mode's partial sums.
+template <typename T> struct EpAcc { Acc<T> a[5]; };
+template <int MODE, int V, typename T>
+PD void row_ep_store(const RowEp<T>& ep, size_t idx, bool al, const T (&val)[V], const T (&a)[V], const T (&b)[V],
+                     EpAcc<T>& part, Acc<T> (&sq)[V]) {
+  T o[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    if constexpr (MODE == EP_CG_AP) {
+      // (A p)_i; a short run of terms is summed by plain FMAs (their rounding
+      // errors are independent across the ~10^5 runs and average out) and
+      // then merged compensated.
+      o[k] = T(ep.nu2) * val[k] + T(2) * a[k];
+      part.a[0].s = fma(a[k], o[k], part.a[0].s);
+      part.a[1].s = fma(b[k], o[k], part.a[1].s);
+      part.a[2].s = fma(o[k], o[k], part.a[2].s);
+      part.a[3].s = fma(b[k], a[k], part.a[3].s);
+      part.a[4].s = fma(b[k], b[k], part.a[4].s);
+    } else if constexpr (MODE == EP_CG_R0) {
+      o[k] = (a[k] - T(2) * b[k]) - T(ep.nu2) * val[k];
+      sq[k].add_prod(o[k], o[k]);
+    } else if constexpr (MODE == EP_POWER) {
+      o[k] = val[k];
+      sq[k].add_prod(val[k], val[k]);
+    } else if constexpr (MODE == EP_XS_ADD) {
+      o[k] = a[k] + T(ep.nu) * val[k];
+    } else if constexpr (MODE == EP_QX) {
+      o[k] = T(ep.nu2) * val[k] + T(2) * a[k];
+    } else {
+      o[k] = val[k];
+    }
+  }
+  vstore(ep.out + idx, o, al);
+  if constexpr (MODE == EP_CG_R0) vstore(ep.out2 + idx, o, al);
+}
+
+// Forward row prologue (see RowProMode) of V consecutive pixels of U chunks
+// of a row pair (pixel offsets ia of row a; row b is n further on).  All loads
+// precede the CG step's stores.
+template <int U, int V, typename T>
+PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al, T (&va)[U][V], T (&vb)[U][V]) {
   if (pro.mode == PRO_CG_STEP) {
     // x += alpha p, r -= alpha Ap, p = r + beta p (alpha, beta of the previous step)
     const T alpha = T(pro.scalars[S_ALPHA]), beta = T(pro.scalars[S_BETA]);
-    T xv[NR][E / 2], rv[NR][E / 2], av[NR][E / 2];
+    T xv[2 * U][V], rv[2 * U][V], pv[2 * U][V], av[2 * U][V];
 #pragma unroll
-    for (int r = 0; r < NR; ++r)
+    for (int u = 0; u < 2 * U; ++u) {
+      const size_t i = ia[u >> 1] + size_t(u & 1) * n;
+      vload(xv[u], pro.xu + i, true);
+      vload(rv[u], pro.r + i, true);
+      vload(pv[u], pro.p + i, true);
+      vload(av[u], pro.ap + i, true);
+    }
 #pragma unroll
-      for (int j = 0; j < E / 2; ++j) {
-        const size_t idx = row0[r] + i2[j];
-        xv[r][j] = pro.xu[idx];
-        rv[r][j] = pro.r[idx];
-        val[r][j] = pro.p[idx];
-        av[r][j] = pro.ap[idx];
+    for (int u = 0; u < 2 * U; ++u) {
+      const size_t i = ia[u >> 1] + size_t(u & 1) * n;
+      T xn[V], rn[V], pn[V];
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        rn[k] = fma(-alpha, av[u][k], rv[u][k]);
+        xn[k] = fma(alpha, pv[u][k], xv[u][k]);
+        pn[k] = fma(beta, pv[u][k], rn[k]);
+        if (u & 1) vb[u >> 1][k] = pn[k];
+        else va[u >> 1][k] = pn[k];
       }
-#pragma unroll
-    for (int r = 0; r < NR; ++r)
-#pragma unroll
-      for (int j = 0; j < E / 2; ++j) {
-        const size_t idx = row0[r] + i2[j];
-        const T pv = val[r][j];
-        const T rn = fma(-alpha, av[r][j], rv[r][j]);
-        pro.xu[idx] = fma(alpha, pv, xv[r][j]);
-        pro.r[idx] = rn;
-        val[r][j] = fma(beta, pv, rn);
-        pro.p[idx] = val[r][j];
-      }
+      vstore(pro.xu + i, xn, true);
+      vstore(pro.r + i, rn, true);
+      vstore(pro.p + i, pn, true);
+    }
   } else if (pro.mode == PRO_CG_START) {
     // r = b - A x_hat, p = r (b in pro.x, A x_hat in pro.ap)
-    T bv[NR][E / 2], av[NR][E / 2];
+    T bv[2 * U][V], av[2 * U][V];
 #pragma unroll
-    for (int r = 0; r < NR; ++r)
+    for (int u = 0; u < 2 * U; ++u) {
+      const size_t i = ia[u >> 1] + size_t(u & 1) * n;
+      vload(bv[u], pro.x + i, true);
+      vload(av[u], pro.ap + i, true);
+    }
 #pragma unroll
-      for (int j = 0; j < E / 2; ++j) {
-        const size_t idx = row0[r] + i2[j];
-        bv[r][j] = pro.x[idx];
-        av[r][j] = pro.ap[idx];
+    for (int u = 0; u < 2 * U; ++u) {
+      const size_t i = ia[u >> 1] + size_t(u & 1) * n;
+      T rn[V];
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        rn[k] = bv[u][k] - av[u][k];
+        if (u & 1) vb[u >> 1][k] = rn[k];
+        else va[u >> 1][k] = rn[k];
       }
-#pragma unroll
-    for (int r = 0; r < NR; ++r)
-#pragma unroll
-      for (int j = 0; j < E / 2; ++j) {
-        const size_t idx = row0[r] + i2[j];
-        val[r][j] = bv[r][j] - av[r][j];
-        pro.r[idx] = val[r][j];
-        pro.p[idx] = val[r][j];
-      }
+      vstore(pro.r + i, rn, true);
+      vstore(pro.p + i, rn, true);
+    }
   } else {
     const T scl = pro.mode == PRO_SCALE ? T(pro.scalars[pro.idx]) : T(1);
 #pragma unroll
-    for (int r = 0; r < NR; ++r)
+    for (int u = 0; u < U; ++u) {
+      vload(va[u], pro.x + ia[u], al);
+      vload(vb[u], pro.x + ia[u] + n, al);
+    }
 #pragma unroll
-      for (int j = 0; j < E / 2; ++j) val[r][j] = pro.x[row0[r] + i2[j]] * scl;
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        va[u][k] *= scl;
+        vb[u][k] *= scl;
+      }
   }
 }
 
@@ -429,8 +677,184 @@ PD void row_ep_finish(const RowEp<T>& ep, EpAcc<T> part, double* red /*[5*32]*/,
   }
 }
 
-// Operand arrays an epilogue reads (staged in shared memory by the real-form
-// inverse row pass): CG_AP p, r; CG_R0 b, p; QX p; XS_ADD b.
+// ----------------------------------------------------------------- kernels
+template <typename T, int LOGN> struct ColThreads {
+  static constexpr int value = (kColBytes / int(sizeof(typename cplx_t<T>::type))) * ((1 << LOGN) / 16);
+};
+
+// The image is real, so two rows a, b travel as one complex row z = x_a + i x_b,
+// whose transform Z separates as X_a(k) = (Z(k) + conj Z(-k)) / 2 and
+// X_b(k) = (Z(k) - conj Z(-k)) / (2i), and only the half spectrum k in [0, K/2]
+// is kept: n complex values, entry 0 carrying the two real ones,
+// X(0) + i X(K/2).  They are stored transposed (half_at).
+
+// Forward row pass of the real form: PAIRS row pairs per CTA, zero-padded to K
+// columns, to their half spectra.  Per pair two halves of TT threads.  Latency
+// and L1 bound (one wave, an L2-resident set; shared-memory exchanges and
+// 32-byte stores): n = 1024 with the CG update as prologue 8.8 us, against
+// 11.5 us for 2048-point transforms on 256 threads.
+template <typename T, int LOGN, typename Src>
+__global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN>::ROW_MINB) k_row_fwd_h(Src src) {
+  typedef typename cplx_t<T>::type C;
+  typedef RowHalf<T, LOGN> H;
+  constexpr int n = H::N, V = H::V, E = H::E, TT = H::TT, NT = H::ROW_THREADS;
+  decltype(auto) a = src.get();
+  const RowPro<T>& pro = a.pro;
+  const T* __restrict__ deapod = a.deapod;
+  C* __restrict__ B = a.B;
+  const C* __restrict__ tw = a.tw;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  C* zb = reinterpret_cast<C*>(sm_raw);      // [PAIRS][n]: the packed rows
+  C* bufs = zb + H::PAIRS * n;               // [PAIRS][2][BUF]
+  const int r0 = int(blockIdx.x) * 2 * H::PAIRS;
+  {
+    constexpr int CH = H::PAIRS * n / V;     // chunks of V pixels of a row pair
+    constexpr int IT = CH / NT, U = IT % 2 == 0 ? 2 : 1;
+    static_assert(CH % NT == 0, "E is a multiple of 2 V");
+    const bool al = aligned16(pro.x);
+    for (int it = 0; it < IT; it += U) {
+      size_t ia[U];
+      int at[U];
+      T va[U][V], vb[U][V];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int ch = int(threadIdx.x) + (it + u) * NT;
+        const int pr = ch / (n / V), i = (ch - pr * (n / V)) * V;
+        at[u] = pr * n + i;
+        ia[u] = size_t(r0 + 2 * pr) * n + i;
+      }
+      row_prologue<U, V>(pro, ia, n, al, va, vb);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (deapod) {  // S: deapodisation of both rows (the Phi form; the convolution form has none)
+          const int row = r0 + 2 * (at[u] / n), i = at[u] & (n - 1);
+          const T da = deapod[row], db = deapod[row + 1];
+          T dc[V];
+          vload(dc, deapod + i, true);
+#pragma unroll
+          for (int k = 0; k < V; ++k) {
+            va[u][k] *= da * dc[k];
+            vb[u][k] *= db * dc[k];
+          }
+        }
+        C z[V];
+#pragma unroll
+        for (int k = 0; k < V; ++k) z[k] = cmk<C>(va[u][k], vb[u][k]);
+        cstore(zb + at[u], z);
+      }
+    }
+  }
+  __syncthreads();
+  const int half = threadIdx.x / TT, t = threadIdx.x - half * TT;
+  const int pr = half >> 1, odd = half & 1;
+  C* s = bufs + size_t(half) * H::BUF;
+  C v[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) v[m] = zb[pr * n + t + ((m + E / 2) & (E - 1)) * TT];  // pixel of position j mod n
+  if (odd) half_omega<H, -1>(v, t, tw);
+  half_fft<H, -1>(v, t, s, half, a.tws);
+#pragma unroll
+  for (int m = 0; m < E; ++m) s[t + m * TT] = v[m];
+  __syncthreads();
+  // separate the pairs: column c = 2m + odd from elements m and -m of its half
+  constexpr int PC = sizeof(T) == 4 ? 2 : 1;  // pairs per 32-byte store
+  static_assert(H::PAIRS % PC == 0, "whole sectors");
+  for (int w = threadIdx.x; w < n * (H::PAIRS / PC); w += NT) {
+    const int cp = w & (n - 1), pc = w / n;  // column in storage order
+    const int o = cp >= n / 2, m = cp - o * (n / 2), mm = o ? n - 1 - m : (n - m) & (n - 1);
+    C out[2 * PC];
+#pragma unroll
+    for (int q = 0; q < PC; ++q) {
+      const C* hs = bufs + size_t((pc * PC + q) * 2 + o) * H::BUF;
+      const C zk = hs[m];
+      if (cp == 0) {
+        const C zh = hs[n / 2];
+        out[2 * q] = cmk<C>(zk.x, zh.x);
+        out[2 * q + 1] = cmk<C>(zk.y, zh.y);
+      } else {
+        const C zm = hs[mm];  // Z(-k)
+        out[2 * q] = cmk<C>(T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y));
+        out[2 * q + 1] = cmk<C>(T(0.5) * (zk.y + zm.y), T(0.5) * (zm.x - zk.x));
+      }
+    }
+    st32(B + size_t(cp) * n + r0 + pc * 2 * PC, out);
+  }
+}
+
+// Column pass of the convolution form (Section 3: Phi^H Phi precomputed): the
+// forward FFT of each half-spectrum column over the K grid rows (n non-zero),
+// the product with the PSF's real spectrum, and the inverse FFT's n kept rows,
+// all in one thread's registers (the forward transform ends in the order in
+// which the inverse begins).  Column 0 holds two real-row columns,
+// c0 = X(., 0) + i X(., K/2): its transform P splits into the even part
+// (P(q) + conj P(-q)) / 2 (column 0's) and (P(q) - conj P(-q)) / 2 (i times
+// column K/2's), each multiplied by its own spectrum column.
+// One column (two warps at n = 1024) per CTA, so that 1024 small CTAs spread
+// evenly: 11.4 us against 22.3 us for 256 CTAs of four 2048-point columns.
+template <typename T, int LOGN, typename Src>
+__global__ void __launch_bounds__(ColHalf<T, LOGN>::COL_THREADS, ColHalf<T, LOGN>::COL_MINB) k_col_conv_h(Src src) {
+  typedef typename cplx_t<T>::type C;
+  typedef ColHalf<T, LOGN> H;
+  constexpr int n = H::N, E = H::E, TT = H::TT;
+  decltype(auto) a = src.get();
+  const T* __restrict__ khat = a.khat;
+  const C* __restrict__ tw = a.tw;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  C* bufs = reinterpret_cast<C*>(sm_raw);
+  const int half = threadIdx.x / TT, t = threadIdx.x - half * TT;
+  const int col = int(blockIdx.x) * H::COLS + (half >> 1), odd = half & 1;
+  C* s = bufs + size_t(half) * H::BUF;
+  C* __restrict__ Bc = a.B + size_t(col) * n;
+  C v[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) v[m] = Bc[t + ((m + E / 2) & (E - 1)) * TT];
+  if (odd) half_omega<H, -1>(v, t, tw);
+  half_fft<H, -1>(v, t, s, half, a.tws);
+  const T* kc = khat + (size_t(col) * 2 + odd) * n;
+  if (blockIdx.x == 0) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) s[t + m * TT] = v[m];
+    __syncthreads();
+    const T* kn = a.knyq + odd * n;
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int q = t + m * TT;
+      const T h0 = kc[q];
+      if (col == 0) {
+        const T hn = kn[q];
+        const C P = v[m], Pm = s[odd ? n - 1 - q : (n - q) & (n - 1)];
+        const T evx = T(0.5) * (P.x + Pm.x), evy = T(0.5) * (P.y - Pm.y);
+        const T odx = T(0.5) * (P.x - Pm.x), ody = T(0.5) * (P.y + Pm.y);
+        v[m] = cmk<C>(h0 * evx + hn * odx, h0 * evy + hn * ody);
+      } else {
+        v[m] = cscale(v[m], h0);
+      }
+    }
+    __syncthreads();
+  } else {
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = cscale(v[m], kc[t + m * TT]);
+  }
+  half_fft<H, 1>(v, t, s, half, a.tws);
+  if (odd) half_omega<H, 1>(v, t, tw);
+  // the halves' sum: each half finishes half of the rows and hands over the rest
+#pragma unroll
+  for (int m = 0; m < E / 2; ++m) {
+    if (odd) s[t + m * TT] = v[m];
+    else s[t + (m + E / 2) * TT] = v[m + E / 2];
+  }
+  __syncthreads();
+  const C* so = bufs + size_t(half ^ 1) * H::BUF;
+#pragma unroll
+  for (int m = 0; m < E / 2; ++m) {
+    const int me = m + (odd ? E / 2 : 0);
+    const C mine = odd ? v[m + E / 2] : v[m];
+    Bc[t + ((me + E / 2) & (E - 1)) * TT] = cadd(mine, so[t + me * TT]);
+  }
+}
+
+// Operand arrays an epilogue reads (staged in shared memory by the inverse row
+// pass): CG_AP p, r; CG_R0 b, p; QX p; XS_ADD b.
 template <typename T> PD int ep_staged(const RowEp<T>& ep, const T** src) {
   switch (ep.mode) {
     case EP_CG_AP: src[0] = ep.p; src[1] = ep.r; return 2;
@@ -440,268 +864,165 @@ template <typename T> PD int ep_staged(const RowEp<T>& ep, const T** src) {
     default: return 0;
   }
 }
-// Epilogue of both rows of a real-form sequence with the operands in shared
-// memory (ops[k][row][n]).
-template <int LOGN, int MODE, int E, typename T>
-PD EpAcc<T> row_ep_staged_mode(const RowEp<T>& ep, const T (&val)[2][E], int t, const size_t (&row0)[2],
-                               const T* ops) {
-  constexpr int n = (1 << LOGN) / 2;
-  EpAcc<T> part;
+// Sum of the halves, deapodisation (S^T after the crop: the Phi^H form) and
+// epilogue of the CTA's rows, V pixels of a row pair at a time; the operands
+// lie in shared memory (ops[pair][k][row][n]).
+template <int LOGN, int MODE, typename T>
+PD EpAcc<T> row_ep_rows(const RowEp<T>& ep, const typename cplx_t<T>::type* bufs, const T* ops, const T* deapod,
+                        int r0) {
+  typedef typename cplx_t<T>::type C;
+  typedef RowHalf<T, LOGN> H;
+  constexpr int n = H::N, V = H::V, NT = H::ROW_THREADS;
+  constexpr int NOP = MODE == EP_CG_AP || MODE == EP_CG_R0 ? 2 : (MODE == EP_QX || MODE == EP_XS_ADD ? 1 : 0);
+  const bool al = MODE != EP_STORE || aligned16(ep.out);  // only EP_STORE writes a caller's array
+  EpAcc<T> part, run;
+  Acc<T> sq[V];  // compensated sums of squares, V independent chains
+  int terms = 0;
+  for (int ch = threadIdx.x; ch < H::PAIRS * n / V; ch += NT) {
+    const int pr = ch / (n / V), i = (ch - pr * (n / V)) * V;
+    const C* he = bufs + size_t(2 * pr) * H::BUF + i;
+    const C* ho = he + H::BUF;
+    T val[2][V];
+    C ze[V], zo[V];
+    cload(ze, he);
+    cload(zo, ho);
 #pragma unroll
-  for (int m = 0; m < E; ++m) {
-    const int i2 = ep_col<LOGN, E>(t, m);
-    if (i2 < n) {
+    for (int k = 0; k < V; ++k) {
+      const C z = cadd(ze[k], zo[k]);
+      val[0][k] = z.x;
+      val[1][k] = z.y;
+    }
+    const int row = r0 + 2 * pr;
+    if (deapod) {
+      const T da = deapod[row], db = deapod[row + 1];
+      T dc[V];
+      vload(dc, deapod + i, true);
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const T o0 = ops[r * n + i2], o1 = ops[(2 + r) * n + i2];
-        EpOpd<T> opd{T(0), T(0)};
-        if constexpr (MODE == EP_CG_AP) opd = EpOpd<T>{o0, o1};
-        else if constexpr (MODE == EP_CG_R0) opd.a = o0 - T(2) * o1;
-        else if constexpr (MODE == EP_QX || MODE == EP_XS_ADD) opd.a = o0;
-        row_ep_store<MODE>(ep, row0[r] + i2, val[r][m], opd, part);
+      for (int k = 0; k < V; ++k) {
+        val[0][k] *= da * dc[k];
+        val[1][k] *= db * dc[k];
       }
     }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      T o0[V] = {}, o1[V] = {};
+      if constexpr (NOP > 0) vload(o0, ops + (size_t(2 * pr) * 2 + r) * n + i, true);
+      if constexpr (NOP > 1) vload(o1, ops + (size_t(2 * pr + 1) * 2 + r) * n + i, true);
+      row_ep_store<MODE>(ep, size_t(row + r) * n + i, al, val[r], o0, o1, part, sq);
+    }
+    if constexpr (MODE == EP_CG_AP) {  // plain runs of 16 terms
+      terms += 2 * V;
+      if (terms >= 16 || V < 4) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          run.a[k].add(part.a[k].s);
+          part.a[k] = Acc<T>();
+        }
+        terms = 0;
+      }
+    }
+  }
+  if constexpr (MODE == EP_CG_AP) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) acc_merge(run.a[k], part.a[k]);
+    return run;
+  }
+  if constexpr (MODE == EP_CG_R0 || MODE == EP_POWER) {
+#pragma unroll
+    for (int k = 0; k < V; ++k) acc_merge(part.a[0], sq[k]);
   }
   return part;
 }
-template <int LOGN, int E, typename T>
-PD EpAcc<T> row_ep_staged(const RowEp<T>& ep, const T (&val)[2][E], int t, const size_t (&row0)[2], const T* ops) {
+template <int LOGN, typename T>
+PD EpAcc<T> row_ep_all(const RowEp<T>& ep, const typename cplx_t<T>::type* bufs, const T* ops, const T* deapod, int r0) {
   switch (ep.mode) {
-    case EP_CG_AP: return row_ep_staged_mode<LOGN, EP_CG_AP>(ep, val, t, row0, ops);
-    case EP_CG_R0: return row_ep_staged_mode<LOGN, EP_CG_R0>(ep, val, t, row0, ops);
-    case EP_POWER: return row_ep_staged_mode<LOGN, EP_POWER>(ep, val, t, row0, ops);
-    case EP_XS_ADD: return row_ep_staged_mode<LOGN, EP_XS_ADD>(ep, val, t, row0, ops);
-    case EP_QX: return row_ep_staged_mode<LOGN, EP_QX>(ep, val, t, row0, ops);
-    default: return row_ep_staged_mode<LOGN, EP_STORE>(ep, val, t, row0, ops);
+    case EP_CG_AP: return row_ep_rows<LOGN, EP_CG_AP>(ep, bufs, ops, deapod, r0);
+    case EP_CG_R0: return row_ep_rows<LOGN, EP_CG_R0>(ep, bufs, ops, deapod, r0);
+    case EP_POWER: return row_ep_rows<LOGN, EP_POWER>(ep, bufs, ops, deapod, r0);
+    case EP_XS_ADD: return row_ep_rows<LOGN, EP_XS_ADD>(ep, bufs, ops, deapod, r0);
+    case EP_QX: return row_ep_rows<LOGN, EP_QX>(ep, bufs, ops, deapod, r0);
+    default: return row_ep_rows<LOGN, EP_STORE>(ep, bufs, ops, deapod, r0);
   }
 }
 
-// ----------------------------------------------------------------- kernels
-template <typename T, int LOGN> struct ColThreads {
-  static constexpr int value = (kColBytes / int(sizeof(typename cplx_t<T>::type))) * ((1 << LOGN) / 16);
-};
-
-// Composite operator by convolution (Section 3: precompute Phi^H Phi), in its
-// real form.  The image is real and the PSF spectrum real and even, so only
-// the half spectrum k2 in [0, K/2] of each image row is carried: two rows a, b
-// travel as one complex row z = x_a + i x_b, whose transform Z separates as
-// X_a(k) = (Z(k) + conj Z(-k)) / 2 and X_b(k) = (Z(k) - conj Z(-k)) / (2i).
-// A half-spectrum row holds K/2 complex values; its entry 0 carries the two
-// real ones, X(0) + i X(K/2).  Half-spectrum rows are stored n x K/2 in A.
-
-// Forward row pass of the real form: rows 2 pr and 2 pr + 1 of the prologue's
-// image, zero-padded to K columns, to their half spectra.
-template <typename T, int LOGN, int E, typename Src>
-__global__ void __launch_bounds__(kRowCta) k_row_fwd_h(Src src) {
-  typedef typename cplx_t<T>::type C;
-  decltype(auto) a = src.get();
-  const Geometry& g = a.g;
-  const RowPro<T>& pro = a.pro;
-  const T* __restrict__ deapod = a.deapod;
-  C* __restrict__ B = a.B;
-  const C* __restrict__ tw = a.tw;
-  const int nseq = a.nseq;
-  constexpr int TT = Plan<LOGN, E>::T;
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int K = g.K, n = g.n, H = K / 2;
-  const int seq = threadIdx.x / TT, t = threadIdx.x - seq * TT;
-  const int ia = 2 * (blockIdx.x * nseq + seq), ib = ia + 1;
-  C* s = reinterpret_cast<C*>(sm_raw) + seq * padded(K);
-  const size_t row0[2] = {size_t(ia) * n, size_t(ib) * n};
-  T val[2][E / 2];
-  int i2[E / 2];
-  row_prologue<LOGN, 2, E>(pro, row0, t, val, i2);
-  C v[E];
-#pragma unroll
-  for (int m = 0; m < E; ++m) v[m] = cz<C>();
-  if (deapod) {  // S: deapodisation of both rows (the Phi form; the convolution form has none)
-    const T da = deapod[ia], db = deapod[ib];
-#pragma unroll
-    for (int j = 0; j < E / 2; ++j) {
-      const T dc = deapod[i2[j]];
-      v[kept_slot<E>(j)] = cmk<C>(val[0][j] * da * dc, val[1][j] * db * dc);
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < E / 2; ++j) v[kept_slot<E>(j)] = cmk<C>(val[0][j], val[1][j]);
-  }
-  auto to_smem = [&](int q, C x) { s[sidx(q)] = x; };
-  run_stages<LOGN, 0, E>(v, t, 1, s, 1, tw, -1, to_smem);
-  __syncthreads();
-  C* oa = B + size_t(ia) * H;
-  C* ob = oa + H;
-#pragma unroll
-  for (int m = 0; m < E / 2; ++m) {
-    const int k = t + m * TT;
-    const C zk = s[sidx(k)];
-    if (k == 0) {
-      const C zh = s[sidx(H)];
-      oa[0] = cmk<C>(zk.x, zh.x);
-      ob[0] = cmk<C>(zk.y, zh.y);
-    } else {
-      const C zm = s[sidx(K - k)];  // Z(-k)
-      oa[k] = cmk<C>(T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y));
-      ob[k] = cmk<C>(T(0.5) * (zk.y + zm.y), T(0.5) * (zm.x - zk.x));
-    }
-  }
-}
-
-// Column pass of the real form: cw half-spectrum columns per CTA, forward
-// FFT over the K rows (n non-zero), multiply by the PSF spectrum, inverse FFT,
-// keep the n rows the crop retains.  Column 0 holds two real-row columns,
-// c0 = X(., 0) + i X(., K/2): its transform P splits into the even part
-// (P(q) + conj P(-q)) / 2 (column 0's) and (P(q) - conj P(-q)) / 2 (i times
-// column K/2's), each multiplied by its own spectrum column.
-// One CTA per SM and the full register file per thread: the radix-16
-// stages then run spill-free, which measured faster (22.6 against 24.8 us per
-// launch at K = 2048) than two spilling CTAs per SM, despite the second wave.
+// Inverse row pass of the real form: the half spectra of rows a and b rebuilt
+// into Z = Y_a + i Y_b over all K frequencies (Y(K - k) = conj Y(k)), one
+// inverse transform by halves, Re -> row a, Im -> row b, crop and row
+// epilogue.  Bound as the forward pass: n = 1024 with the CG epilogue 9.8 us,
+// against 14.0 us for 2048-point transforms.
 template <typename T, int LOGN, typename Src>
-__global__ void __launch_bounds__(ColThreads<T, LOGN>::value, 1)
-    k_col_conv_h(Src src) {
+__global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN>::ROW_MINB) k_row_inv_h(Src src) {
   typedef typename cplx_t<T>::type C;
+  typedef RowHalf<T, LOGN> H;
+  constexpr int n = H::N, E = H::E, TT = H::TT, NT = H::ROW_THREADS;
   decltype(auto) a = src.get();
-  const Geometry& g = a.g;
-  C* __restrict__ B = a.B;
-  const T* __restrict__ khat = a.khat;
-  const T* __restrict__ knyq = a.knyq;
-  const C* __restrict__ tw = a.tw;
-  const int cw = a.cw;
-  constexpr int TT = Plan<LOGN>::T;
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int K = g.K, n = g.n, half = n / 2, H = K / 2;
-  const int cc = threadIdx.x % cw, t = threadIdx.x / cw;
-  const int c = blockIdx.x * cw + cc;
-  C* s = reinterpret_cast<C*>(sm_raw) + cc;  // cw interleaved columns
-  auto load = [&](int m) -> C {
-    const int i1 = (t + m * TT + half) & (K - 1);
-    return i1 < n ? B[size_t(i1) * H + c] : cz<C>();
-  };
-  auto to_smem = [&](int q, C v) { s[sidx(q) * cw] = v; };
-  fft_seq<LOGN>(t, s, cw, tw, -1, load, to_smem);
-  __syncthreads();
-  if (blockIdx.x == 0) {
-    // column 0 (this CTA's first): the pairs (q, -q), q = 0..K/2, in place,
-    // spread over all the CTA's threads with their spectrum values loaded
-    // first; ev(-q) = conj ev(q), od(-q) = -conj od(q)
-    C* s0 = reinterpret_cast<C*>(sm_raw);
-    const int nt = blockDim.x;
-    for (int q0 = 0; q0 <= H; q0 += 4 * nt) {
-      T h0[4], hn[4], h0m[4], hnm[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int q = q0 + u * nt + int(threadIdx.x), qm = (K - q) & (K - 1);
-        if (q <= H) {
-          h0[u] = khat[size_t(q) * cw];
-          hn[u] = knyq[q];
-          h0m[u] = khat[size_t(qm) * cw];
-          hnm[u] = knyq[qm];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int q = q0 + u * nt + int(threadIdx.x), qm = (K - q) & (K - 1);
-        if (q <= H) {
-          const C P = s0[sidx(q) * cw], Pm = s0[sidx(qm) * cw];
-          const T evx = T(0.5) * (P.x + Pm.x), evy = T(0.5) * (P.y - Pm.y);
-          const T odx = T(0.5) * (P.x - Pm.x), ody = T(0.5) * (P.y + Pm.y);
-          s0[sidx(q) * cw] = cmk<C>(h0[u] * evx + hn[u] * odx, h0[u] * evy + hn[u] * ody);
-          if (qm != q) s0[sidx(qm) * cw] = cmk<C>(h0m[u] * evx - hnm[u] * odx, hnm[u] * ody - h0m[u] * evy);
-        }
-      }
-    }
-  }
-  __syncthreads();
-  C v[16];
-  const T* kc = khat + (size_t(blockIdx.x) * K) * cw + cc;
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const int q = t + m * TT;
-    v[m] = cscale(s[sidx(q) * cw], c ? kc[size_t(q) * cw] : T(1));
-  }
-  __syncthreads();
-  auto store = [&](int q, C x) {
-    const int i1 = (q + half) & (K - 1);
-    if (i1 < n) B[size_t(i1) * H + c] = x;
-  };
-  run_stages<LOGN, 0>(v, t, 1, s, cw, tw, +1, store);
-}
-
-// Inverse row pass of the real form: the half spectra of rows a = 2 pr and
-// b = 2 pr + 1 rebuilt into Z = Y_a + i Y_b over all K frequencies
-// (Y(K - k) = conj Y(k)), one inverse FFT, Re -> row a, Im -> row b, crop and
-// row epilogue.
-template <typename T, int LOGN, int E, typename Src>
-__global__ void __launch_bounds__(kRowCta, 2) k_row_inv_h(Src src) {
-  typedef typename cplx_t<T>::type C;
-  decltype(auto) a = src.get();
-  const Geometry& g = a.g;
   const C* __restrict__ B = a.B;
-  const T* __restrict__ deapod = a.deapod;
   const RowEp<T>& ep = a.ep;
   const C* __restrict__ tw = a.tw;
-  const int nseq = a.nseq;
-  constexpr int TT = Plan<LOGN, E>::T;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ double red[5 * 32];
   __shared__ __align__(8) uint64_t bar;
-  const int K = g.K, n = g.n, H = K / 2;
-  const int seq = threadIdx.x / TT, t = threadIdx.x - seq * TT;
-  const int ia = 2 * (blockIdx.x * nseq + seq), ib = ia + 1;
-  C* s = reinterpret_cast<C*>(sm_raw) + seq * padded(K);
-  // The epilogue's operand rows (ops[seq][k][row][n]) arrive by bulk copies
+  C* bufs = reinterpret_cast<C*>(sm_raw);  // [PAIRS][2][BUF]
+  const int r0 = int(blockIdx.x) * 2 * H::PAIRS;
+  // The epilogue's operand rows (ops[pair][k][row][n]) arrive by bulk copies
   // while the transform runs.
-  T* ops_all = reinterpret_cast<T*>(sm_raw + align16(nseq * padded(K) * sizeof(C)));
+  T* ops = reinterpret_cast<T*>(sm_raw + align16(size_t(H::PAIRS) * 2 * H::BUF * sizeof(C)));
   const T* opd[2] = {nullptr, nullptr};
   const int nop = ep_staged(ep, opd);
   if (nop > 0 && threadIdx.x == 0) {
     mbar_init(&bar, 1);
     fence_barrier_init();
-    const uint32_t row_bytes = uint32_t(n * sizeof(T));
-    mbar_arrive_expect_tx(&bar, uint32_t(nseq * nop * 2) * row_bytes);
-    for (int q = 0; q < nseq; ++q) {
-      const int r0 = 2 * (blockIdx.x * nseq + q);
+    const uint32_t pair_bytes = uint32_t(2 * n * sizeof(T));  // rows a and b are contiguous
+    mbar_arrive_expect_tx(&bar, uint32_t(H::PAIRS * nop) * pair_bytes);
+    for (int q = 0; q < H::PAIRS; ++q)
       for (int k = 0; k < nop; ++k)
-        for (int r = 0; r < 2; ++r)
-          bulk_load(ops_all + ((size_t(q) * 2 + k) * 2 + r) * n, opd[k] + size_t(r0 + r) * n, row_bytes, &bar);
-    }
+        bulk_load(ops + (size_t(q) * 2 + k) * 2 * n, opd[k] + size_t(r0 + 2 * q) * n, pair_bytes, &bar);
   }
-  __syncthreads();
-  const C* ba = B + size_t(ia) * H;
-  const C* bb = ba + H;
-  // frequency q = t + m K/E: entry q for m < E/2, entry K - q (entry 0 for
-  // q = K/2) above; thread 0 unpacks entry 0 into Y(0) and Y(K/2)
-  auto load = [&](int m) -> C {
-    const int q = t + m * TT;
-    const int e = m < E / 2 ? q : ((K - q) & (H - 1));
-    const C a = ba[e], b = bb[e];
-    if (t == 0 && (m == 0 || m == E / 2)) return m == 0 ? cmk<C>(a.x, b.x) : cmk<C>(a.y, b.y);
-    return m < E / 2 ? cmk<C>(a.x - b.y, a.y + b.x) : cmk<C>(a.x + b.y, b.x - a.y);
-  };
-  T val[2][E];
-  int cnt = 0;
-  auto stash = [&](int, C v) {  // sink order, see last_pos
-    val[0][cnt] = v.x;
-    val[1][cnt] = v.y;
-    ++cnt;
-  };
-  fft_seq<LOGN, E>(t, s, 1, tw, +1, load, stash);
-  if (deapod) {  // S^T after the crop (the Phi^H form)
-    const T da = deapod[ia], db = deapod[ib];
+  // the halves' spectra: column c = 2m + odd gives elements m and -m of its half
+  constexpr int PC = sizeof(T) == 4 ? 2 : 1;
+  constexpr int LT = n * (H::PAIRS / PC) / NT, LU = LT % 4 == 0 ? 4 : (LT % 2 == 0 ? 2 : 1);  // LU loads in flight
+  for (int l = 0; l < LT; l += LU) {
+    C ins[LU][2 * PC];
 #pragma unroll
-    for (int m = 0; m < E; ++m) {
-      const int i2 = ep_col<LOGN, E>(t, m);
-      if (i2 < n) {
-        const T dc = deapod[i2];
-        val[0][m] *= da * dc;
-        val[1][m] *= db * dc;
+    for (int u = 0; u < LU; ++u) {
+      const int w = int(threadIdx.x) + (l + u) * NT;
+      ld32(ins[u], B + size_t(w & (n - 1)) * n + r0 + (w / n) * 2 * PC);
+    }
+#pragma unroll
+    for (int u = 0; u < LU; ++u)
+#pragma unroll
+    for (int q = 0; q < PC; ++q) {
+      const int w = int(threadIdx.x) + (l + u) * NT;
+      const int cp = w & (n - 1), pc = w / n;
+      const int o = cp >= n / 2, m = cp - o * (n / 2), mm = o ? n - 1 - m : (n - m) & (n - 1);
+      const C (&in)[2 * PC] = ins[u];
+      C* hs = bufs + size_t((pc * PC + q) * 2 + o) * H::BUF;
+      const C ya = in[2 * q], yb = in[2 * q + 1];
+      if (cp == 0) {
+        hs[0] = cmk<C>(ya.x, yb.x);
+        hs[n / 2] = cmk<C>(ya.y, yb.y);
+      } else {
+        hs[m] = cmk<C>(ya.x - yb.y, ya.y + yb.x);
+        hs[mm] = cmk<C>(ya.x + yb.y, yb.x - ya.y);
       }
     }
   }
-  const size_t row0[2] = {size_t(ia) * n, size_t(ib) * n};
+  __syncthreads();
+  const int half = threadIdx.x / TT, t = threadIdx.x - half * TT, odd = half & 1;
+  C* s = bufs + size_t(half) * H::BUF;
+  C v[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) v[m] = s[t + m * TT];
+  half_sync<TT>(half);
+  half_fft<H, 1>(v, t, s, half, a.tws);
+  if (odd) half_omega<H, 1>(v, t, tw);
+#pragma unroll
+  for (int m = 0; m < E; ++m) s[t + ((m + E / 2) & (E - 1)) * TT] = v[m];  // at its pixel
   bool ok = true;
   if (nop > 0) ok = mbar_wait_bounded(&bar, 0, ep.err);
+  __syncthreads();
   EpAcc<T> part;
-  if (ok) part = row_ep_staged<LOGN>(ep, val, t, row0, ops_all + size_t(seq) * 4 * n);
+  if (ok) part = row_ep_all<LOGN>(ep, bufs, ops, a.deapod, r0);
   row_ep_finish(ep, part, red, int(blockIdx.x), a.nblocks);
 }
 
@@ -741,7 +1062,7 @@ __global__ void __launch_bounds__(ColThreads<T, LOGN>::value, 1)
   C* s = reinterpret_cast<C*>(sm_raw) + cc;
   auto load = [&](int m) -> C {
     const int i1 = (t + m * TT + half) & (K - 1);
-    return i1 < n ? B[size_t(i1) * H + c] : cz<C>();
+    return i1 < n ? B[half_at(c, i1, n)] : cz<C>();
   };
   auto to_smem = [&](int q, C v) { s[sidx(q) * cw] = v; };
   fft_seq<LOGN>(t, s, cw, tw, -1, load, to_smem);
@@ -811,7 +1132,7 @@ __global__ void __launch_bounds__(ColThreads<T, LOGN>::value, ColThreads<T, LOGN
   };
   auto store = [&](int q, C v) {
     const int i1 = (q + half) & (K - 1);
-    if (i1 < n) B[size_t(i1) * H + c] = v;
+    if (i1 < n) B[half_at(c, i1, n)] = v;
   };
   fft_seq<LOGN>(t, s, cw, tw, +1, load, store);
 }
@@ -862,17 +1183,6 @@ __global__ void __launch_bounds__(ColThreads<T, LOGN>::value) k_cols_plain(typen
 }  // namespace
 
 
-// Row pairs per CTA of the real-form row passes (E elements per thread).
-inline int row_pair_nseq(const Geometry& g, int E) {
-  int s = kRowCta / (g.K / E);
-  if (s < 1) s = 1;
-  if (s > g.n / 2) s = g.n / 2;
-  return s;
-}
-
-// CTAs of one inverse row pass (its epilogue's partial sums).
-int row_inv_blocks(const Geometry& g) { return g.n / 2 / row_pair_nseq(g, row_e_host(g.K)); }
-int row_pass_nseq(const Geometry& g) { return row_pair_nseq(g, row_e_host(g.K)); }
 template <typename T> int col_pass_width() { return col_width<T>(); }
 template int col_pass_width<float>();
 template int col_pass_width<double>();
@@ -900,18 +1210,19 @@ template int col_pass_width<double>();
     default: break;                                       \
   }
 
+// L = log2 K; the passes of half transforms are templated on log2 n = L - 1
 template <typename T, int L> cudaError_t configure_one() {
-  cudaError_t e = raise_smem_limit(k_row_fwd_h<T, L, row_e<L>(), ArgVal<RowFwdArgs<T>>>);
-  if (e == cudaSuccess) e = raise_smem_limit(k_col_conv_h<T, L, ArgVal<ColConvArgs<T>>>);
+  cudaError_t e = raise_smem_limit(k_row_fwd_h<T, L - 1, ArgVal<RowFwdArgs<T>>>);
+  if (e == cudaSuccess) e = raise_smem_limit(k_col_conv_h<T, L - 1, ArgVal<ColConvArgs<T>>>);
   if (e == cudaSuccess) e = raise_smem_limit(k_col_fwd_h<T, L, ArgVal<ColFwdArgs<T>>>);
   if (e == cudaSuccess) e = raise_smem_limit(k_col_inv_h<T, L, ArgVal<ColInvArgs<T>>>);
-  if (e == cudaSuccess) e = raise_smem_limit(k_row_inv_h<T, L, row_e<L>(), ArgVal<RowInvArgs<T>>>);
+  if (e == cudaSuccess) e = raise_smem_limit(k_row_inv_h<T, L - 1, ArgVal<RowInvArgs<T>>>);
   if constexpr (L >= 7 && L <= 11) {
-    if (e == cudaSuccess) e = raise_smem_limit(k_row_fwd_h<T, L, row_e<L>(), ArgTab<RowFwdArgs<T>>>);
-    if (e == cudaSuccess) e = raise_smem_limit(k_col_conv_h<T, L, ArgTab<ColConvArgs<T>>>);
+    if (e == cudaSuccess) e = raise_smem_limit(k_row_fwd_h<T, L - 1, ArgTab<RowFwdArgs<T>>>);
+    if (e == cudaSuccess) e = raise_smem_limit(k_col_conv_h<T, L - 1, ArgTab<ColConvArgs<T>>>);
     if (e == cudaSuccess) e = raise_smem_limit(k_col_fwd_h<T, L, ArgTab<ColFwdArgs<T>>>);
     if (e == cudaSuccess) e = raise_smem_limit(k_col_inv_h<T, L, ArgTab<ColInvArgs<T>>>);
-    if (e == cudaSuccess) e = raise_smem_limit(k_row_inv_h<T, L, row_e<L>(), ArgTab<RowInvArgs<T>>>);
+    if (e == cudaSuccess) e = raise_smem_limit(k_row_inv_h<T, L - 1, ArgTab<RowInvArgs<T>>>);
   }
   if (e == cudaSuccess) e = raise_smem_limit(k_rows_plain<T, L>);
   if (e == cudaSuccess) e = raise_smem_limit(k_cols_plain<T, L>);
@@ -942,17 +1253,17 @@ __global__ void k_embed_psf(const T* __restrict__ psf, int n, typename cplx_t<T>
   X[idx] = cmk<C>(psf[size_t(i1) * K + i2], T(0));
 }
 
-// Real part of the spectrum, columns [0, K/2) in launch_col_conv_h's layout
-// [column block][row][cw], column K/2 after them.
+// Real part of the spectrum in launch_col_conv_h's layout: per column (storage
+// order of half_at) its even grid rows, then its odd ones; column K/2 after them.
 template <typename T>
-__global__ void k_spectrum_layout(const typename cplx_t<T>::type* __restrict__ X, int K, int cw, double scale,
+__global__ void k_spectrum_layout(const typename cplx_t<T>::type* __restrict__ X, int K, double scale,
                                   T* __restrict__ khat) {
   const size_t idx = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= size_t(K) * K) return;
-  const int q = int(idx / K), c = int(idx % K), H = K / 2;
-  const T v = T(double(X[idx].x) * scale);
-  if (c < H) khat[(size_t(c / cw) * K + q) * cw + (c % cw)] = v;
-  else if (c == H) khat[size_t(H) * K + q] = v;
+  const int q = int(idx / K), c = int(idx % K), n = K / 2;
+  if (c > n) return;
+  const size_t col = c == n ? size_t(n) : size_t(c & 1) * (n / 2) + (c >> 1);
+  khat[(col * 2 + (q & 1)) * n + (q >> 1)] = T(double(X[idx].x) * scale);
 }
 
 template <typename T>
@@ -963,37 +1274,70 @@ void build_psf_spectrum(const T* psf, int n, T* khat, typename cplx_t<T>::type* 
   const int tb = 256;
   k_embed_psf<T><<<int((tot + tb - 1) / tb), tb, 0, s>>>(psf, n, X);
   launch_fft2_plain<T>(K, X, tw, -1, s);
-  k_spectrum_layout<T><<<int((tot + tb - 1) / tb), tb, 0, s>>>(X, K, col_width<T>(), 1.0 / (double(K) * K), khat);
+  k_spectrum_layout<T><<<int((tot + tb - 1) / tb), tb, 0, s>>>(X, K, 1.0 / (double(K) * K), khat);
 }
 
-// Launch shapes of the real-form passes for grid side K (image side n = K/2).
-inline int row_pass_ctas(const Geometry& g) { return g.n / 2 / row_pair_nseq(g, row_e_host(g.K)); }
-template <typename T> inline size_t row_fwd_smem(const Geometry& g) {
-  return row_pair_nseq(g, row_e_host(g.K)) * padded(g.K) * sizeof(typename cplx_t<T>::type);
+// Launch shapes of the passes of half transforms.
+template <typename T, int LOGN> struct HalfShape {
+  typedef RowHalf<T, LOGN> H;
+  typedef ColHalf<T, LOGN> HC;
+  typedef typename cplx_t<T>::type C;
+  static constexpr int row_ctas = H::N / 2 / H::PAIRS;
+  static constexpr int col_ctas = HC::N / HC::COLS;
+  static size_t fwd_smem() { return size_t(H::PAIRS) * (H::N + 2 * H::BUF) * sizeof(C); }
+  static size_t inv_smem(bool operands) {
+    return align16(size_t(H::PAIRS) * 2 * H::BUF * sizeof(C)) + (operands ? size_t(H::PAIRS) * 4 * H::N * sizeof(T) : 0);
+  }
+  static size_t conv_smem() { return size_t(HC::COLS) * 2 * HC::BUF * sizeof(C); }
+};
+// CTAs of one inverse row pass (its epilogue's partial sums).
+template <typename T> int row_inv_blocks(const Geometry& g) {
+  int b = 0;
+  PURIFY_LOGN_SWITCH(g.K, (b = HalfShape<T, L - 1>::row_ctas));
+  return b;
 }
-template <typename T> inline size_t row_inv_smem(const Geometry& g) {
-  const int nseq = row_pair_nseq(g, row_e_host(g.K));
-  return align16(nseq * padded(g.K) * sizeof(typename cplx_t<T>::type)) + size_t(nseq) * 4 * g.n * sizeof(T);
+template int row_inv_blocks<float>(const Geometry&);
+template int row_inv_blocks<double>(const Geometry&);
+// Twiddles of the half transforms of length n: per stage after the first,
+// W(r k) = exp(-2 pi i r k / (Ns R)) as [r - 1][k], k < Ns; the row passes'
+// table, then the convolution's from element *col_at on.
+template <typename H, typename C> static void half_twiddles_of(std::vector<C>& out) {
+  int ns = H::radix(0);
+  for (int st = 1; st < H::NST; ++st) {
+    const int R = H::radix(st);
+    for (int r = 1; r < R; ++r)
+      for (int k = 0; k < ns; ++k) {
+        const double a = -2.0 * M_PI * double(r) * k / (double(ns) * R);
+        C w;
+        w.x = decltype(w.x)(std::cos(a));
+        w.y = decltype(w.y)(std::sin(a));
+        out.push_back(w);
+      }
+    ns *= R;
+  }
 }
+template <typename T> void half_twiddles(int n, std::vector<typename cplx_t<T>::type>& out, size_t* col_at) {
+  out.clear();
+  PURIFY_LOGN_SWITCH(2 * n, (half_twiddles_of<RowHalf<T, L - 1>>(out)));
+  *col_at = out.size();
+  PURIFY_LOGN_SWITCH(2 * n, (half_twiddles_of<ColHalf<T, L - 1>>(out)));
+}
+template void half_twiddles<float>(int, std::vector<float2>&, size_t*);
+template void half_twiddles<double>(int, std::vector<double2>&, size_t*);
 template <typename T> inline size_t col_smem(const Geometry& g) {
   return col_width<T>() * padded(g.K) * sizeof(typename cplx_t<T>::type);
 }
 
-template <typename T>
-void launch_row_fwd_h(const Geometry& g, const RowPro<T>& pro, const T* deapod, typename cplx_t<T>::type* B,
-                      const typename cplx_t<T>::type* tw, cudaStream_t s) {
-  const int nseq = row_pair_nseq(g, row_e_host(g.K));
-  ArgVal<RowFwdArgs<T>> src{RowFwdArgs<T>{g, pro, deapod, B, tw, nseq}};
-  PURIFY_LOGN_SWITCH(g.K, (k_row_fwd_h<T, L, row_e<L>()><<<row_pass_ctas(g), nseq * Plan<L, row_e<L>()>::T,
-                                                           row_fwd_smem<T>(g), s>>>(src)));
+template <typename T> void launch_row_fwd_h(const RowFwdArgs<T>& a, cudaStream_t s) {
+  ArgVal<RowFwdArgs<T>> src{a};
+  PURIFY_LOGN_SWITCH(a.g.K, (k_row_fwd_h<T, L - 1><<<HalfShape<T, L - 1>::row_ctas, RowHalf<T, L - 1>::ROW_THREADS,
+                                                     HalfShape<T, L - 1>::fwd_smem(), s>>>(src)));
 }
 
-template <typename T>
-void launch_col_conv_h(const Geometry& g, typename cplx_t<T>::type* B, const T* khat,
-                       const typename cplx_t<T>::type* tw, cudaStream_t s) {
-  const int cw = col_width<T>();
-  ArgVal<ColConvArgs<T>> src{ColConvArgs<T>{g, B, khat, khat + size_t(g.K / 2) * g.K, tw, cw}};
-  PURIFY_LOGN_SWITCH(g.K, (k_col_conv_h<T, L><<<g.K / 2 / cw, cw * Plan<L>::T, col_smem<T>(g), s>>>(src)));
+template <typename T> void launch_col_conv_h(const ColConvArgs<T>& a, cudaStream_t s) {
+  ArgVal<ColConvArgs<T>> src{a};
+  PURIFY_LOGN_SWITCH(a.g.K, (k_col_conv_h<T, L - 1><<<HalfShape<T, L - 1>::col_ctas, ColHalf<T, L - 1>::COL_THREADS,
+                                                      HalfShape<T, L - 1>::conv_smem(), s>>>(src)));
 }
 
 template <typename T>
@@ -1012,31 +1356,28 @@ void launch_col_inv_h(const Geometry& g, const typename cplx_t<T>::type* Q, type
   PURIFY_LOGN_SWITCH(g.K, (k_col_inv_h<T, L><<<g.K / 2 / cw, cw * Plan<L>::T, col_smem<T>(g), s>>>(src)));
 }
 
-template <typename T>
-int launch_row_inv_h(const Geometry& g, const typename cplx_t<T>::type* B, const T* deapod, const RowEp<T>& ep,
-                     const typename cplx_t<T>::type* tw, cudaStream_t s) {
-  const int nseq = row_pair_nseq(g, row_e_host(g.K));
-  const int nb = row_pass_ctas(g);
-  ArgVal<RowInvArgs<T>> src{RowInvArgs<T>{g, B, deapod, ep, tw, nseq, nb}};
-  PURIFY_LOGN_SWITCH(g.K, (k_row_inv_h<T, L, row_e<L>()><<<nb, nseq * Plan<L, row_e<L>()>::T, row_inv_smem<T>(g),
-                                                           s>>>(src)));
-  return nb;
+template <typename T> void launch_row_inv_h(const RowInvArgs<T>& a, cudaStream_t s) {
+  ArgVal<RowInvArgs<T>> src{a};
+  const bool operands = a.ep.mode != EP_STORE && a.ep.mode != EP_POWER;
+  PURIFY_LOGN_SWITCH(a.g.K, (k_row_inv_h<T, L - 1><<<HalfShape<T, L - 1>::row_ctas, RowHalf<T, L - 1>::ROW_THREADS,
+                                                     HalfShape<T, L - 1>::inv_smem(operands), s>>>(src)));
 }
 
 // Batched passes: `count` instances of one grid side (g gives the shared
 // shape), arguments in a device table, instance = blockIdx.y.
 template <typename T>
 void launch_row_fwd_h_batch(const Geometry& g, const RowFwdArgs<T>* tab, int count, cudaStream_t s) {
-  const int nseq = row_pair_nseq(g, row_e_host(g.K));
   ArgTab<RowFwdArgs<T>> src{tab};
-  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_row_fwd_h<T, L, row_e<L>()><<<dim3(row_pass_ctas(g), count),
-                                                           nseq * Plan<L, row_e<L>()>::T, row_fwd_smem<T>(g), s>>>(src)));
+  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_row_fwd_h<T, L - 1><<<dim3(HalfShape<T, L - 1>::row_ctas, count),
+                                                         RowHalf<T, L - 1>::ROW_THREADS, HalfShape<T, L - 1>::fwd_smem(),
+                                                         s>>>(src)));
 }
 template <typename T>
 void launch_col_conv_h_batch(const Geometry& g, const ColConvArgs<T>* tab, int count, cudaStream_t s) {
-  const int cw = col_width<T>();
   ArgTab<ColConvArgs<T>> src{tab};
-  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_col_conv_h<T, L><<<dim3(g.K / 2 / cw, count), cw * Plan<L>::T, col_smem<T>(g), s>>>(src)));
+  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_col_conv_h<T, L - 1><<<dim3(HalfShape<T, L - 1>::col_ctas, count),
+                                                          ColHalf<T, L - 1>::COL_THREADS,
+                                                          HalfShape<T, L - 1>::conv_smem(), s>>>(src)));
 }
 template <typename T>
 void launch_col_fwd_h_batch(const Geometry& g, const ColFwdArgs<T>* tab, int count, cudaStream_t s) {
@@ -1052,10 +1393,10 @@ void launch_col_inv_h_batch(const Geometry& g, const ColInvArgs<T>* tab, int cou
 }
 template <typename T>
 void launch_row_inv_h_batch(const Geometry& g, const RowInvArgs<T>* tab, int count, cudaStream_t s) {
-  const int nseq = row_pair_nseq(g, row_e_host(g.K));
   ArgTab<RowInvArgs<T>> src{tab};
-  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_row_inv_h<T, L, row_e<L>()><<<dim3(row_pass_ctas(g), count),
-                                                           nseq * Plan<L, row_e<L>()>::T, row_inv_smem<T>(g), s>>>(src)));
+  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_row_inv_h<T, L - 1><<<dim3(HalfShape<T, L - 1>::row_ctas, count),
+                                                         RowHalf<T, L - 1>::ROW_THREADS,
+                                                         HalfShape<T, L - 1>::inv_smem(true), s>>>(src)));
 }
 
 template <typename T>
@@ -1073,12 +1414,9 @@ void launch_fft2_plain(int K, typename cplx_t<T>::type* X, const typename cplx_t
 }
 
 #define INST(T)                                                                                              \
-  template void launch_row_fwd_h<T>(const Geometry&, const RowPro<T>&, const T*, cplx_t<T>::type*,             \
-                                    const cplx_t<T>::type*, cudaStream_t);                                     \
-  template void launch_col_conv_h<T>(const Geometry&, cplx_t<T>::type*, const T*, const cplx_t<T>::type*,       \
-                                     cudaStream_t);                                                            \
-  template int launch_row_inv_h<T>(const Geometry&, const cplx_t<T>::type*, const T*, const RowEp<T>&,          \
-                                   const cplx_t<T>::type*, cudaStream_t);                                      \
+  template void launch_row_fwd_h<T>(const RowFwdArgs<T>&, cudaStream_t);                                     \
+  template void launch_col_conv_h<T>(const ColConvArgs<T>&, cudaStream_t);                                   \
+  template void launch_row_inv_h<T>(const RowInvArgs<T>&, cudaStream_t);                                     \
   template void launch_fft2_plain<T>(int, cplx_t<T>::type*, const cplx_t<T>::type*, int, cudaStream_t);     \
   template void launch_col_fwd_h<T>(const Geometry&, const cplx_t<T>::type*, cplx_t<T>::type*,                \
                                     const cplx_t<T>::type*, cudaStream_t);                                     \

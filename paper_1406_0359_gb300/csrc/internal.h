@@ -138,8 +138,8 @@ template <typename T> struct RowFwdArgs {
   RowPro<T> pro;
   const T* deapod;
   typename cplx_t<T>::type* B;
-  const typename cplx_t<T>::type* tw;
-  int nseq;
+  const typename cplx_t<T>::type* tw;   // exp(-2 pi i j / K)
+  const typename cplx_t<T>::type* tws;  // stage twiddles (half_twiddles)
 };
 template <typename T> struct ColConvArgs {
   Geometry g;
@@ -147,7 +147,7 @@ template <typename T> struct ColConvArgs {
   const T* khat;
   const T* knyq;
   const typename cplx_t<T>::type* tw;
-  int cw;
+  const typename cplx_t<T>::type* tws;
 };
 template <typename T> struct RowInvArgs {
   Geometry g;
@@ -155,7 +155,7 @@ template <typename T> struct RowInvArgs {
   const T* deapod;
   RowEp<T> ep;
   const typename cplx_t<T>::type* tw;
-  int nseq;
+  const typename cplx_t<T>::type* tws;
   int nblocks;  // CTAs of the instance (its epilogue partials, its ticket)
 };
 template <typename T> struct ColFwdArgs {
@@ -217,23 +217,21 @@ template <typename T> cudaError_t configure_nufft();
 template <typename T> cudaError_t configure_sara();
 
 // CTAs of one inverse row pass (the partial sums its epilogue writes).
-int row_inv_blocks(const Geometry& g);
-// Row pairs per CTA of the row passes; interleaved columns per CTA of the
-// column passes.
-int row_pass_nseq(const Geometry& g);
+template <typename T> int row_inv_blocks(const Geometry& g);
+// Stage twiddles of the row passes and the convolution's column pass for
+// image side n (one table per operator).
+template <typename T> void half_twiddles(int n, std::vector<typename cplx_t<T>::type>& out, size_t* col_at);
+// Interleaved columns per CTA of the column passes of Phi and Phi^H.
 template <typename T> int col_pass_width();
 // Composite operator Phi^H Phi as a convolution, in real form: the image
-// rows' half spectra (n x K/2 complex in B, entry 0 = X(0) + i X(K/2)).
-// Forward row pass (prologue, zero-padding, row FFT of row pairs):
-// deapod: S applied to both rows (Phi), or null (the convolution form).
-template <typename T>
-void launch_row_fwd_h(const Geometry& g, const RowPro<T>& pro, const T* deapod, typename cplx_t<T>::type* B,
-                      const typename cplx_t<T>::type* tw, cudaStream_t s);
+// rows' half spectra (n x K/2 complex in B, stored transposed; entry 0 =
+// X(0) + i X(K/2)).  Forward row pass (prologue, zero-padding, row FFT of row
+// pairs); deapod: S applied to both rows (Phi), or null (the convolution form).
+template <typename T> void launch_row_fwd_h(const RowFwdArgs<T>& a, cudaStream_t s);
 // Column pass: forward column FFT, multiply by the real PSF spectrum khat
-// ([K/2/cw][K][cw], then column K/2 as K values), inverse FFT, crop (in place).
-template <typename T>
-void launch_col_conv_h(const Geometry& g, typename cplx_t<T>::type* B, const T* khat,
-                       const typename cplx_t<T>::type* tw, cudaStream_t s);
+// (per column its even grid rows, then its odd ones; column K/2 at knyq),
+// inverse FFT, crop (in place).
+template <typename T> void launch_col_conv_h(const ColConvArgs<T>& a, cudaStream_t s);
 // Real-form column passes of Phi (half-spectrum rows B -> the full padded
 // grid, mirrored columns included) and Phi^H (padded accumulator Q -> the
 // half-spectrum rows of its Hermitian part).
@@ -243,11 +241,9 @@ void launch_col_fwd_h(const Geometry& g, const typename cplx_t<T>::type* B, type
 template <typename T>
 void launch_col_inv_h(const Geometry& g, const typename cplx_t<T>::type* Q, typename cplx_t<T>::type* B,
                       const typename cplx_t<T>::type* tw, cudaStream_t s);
-// Inverse row pass with the row epilogue (deapod: S^T, or null); returns the
-// number of partial sums.
-template <typename T>
-int launch_row_inv_h(const Geometry& g, const typename cplx_t<T>::type* B, const T* deapod, const RowEp<T>& ep,
-                     const typename cplx_t<T>::type* tw, cudaStream_t s);
+// Inverse row pass with the row epilogue (deapod: S^T, or null); its epilogue
+// writes row_inv_blocks partial sums.
+template <typename T> void launch_row_inv_h(const RowInvArgs<T>& a, cudaStream_t s);
 // Batched real-form passes: `count` instances of the grid side g.K (image
 // sides 64..1024), one launch, arguments from a device table (instance =
 // blockIdx.y); every instance has g's launch shape.
@@ -259,7 +255,7 @@ template <typename T> void launch_row_inv_h_batch(const Geometry& g, const RowIn
 // Real spectrum of the convolution kernel from the PSF image (2n x 2n real,
 // pixel offsets [-n, n)^2): circulant embedding on the K = 2n grid, forward
 // FFT, scaled by 1/K^2, columns [0, K/2] stored in launch_col_conv_h's layout
-// (K/2 * K + K values).  X: K x K scratch.
+// ((K/2 + 1) K values).  X: K x K scratch.
 template <typename T>
 void build_psf_spectrum(const T* psf, int n, T* khat, typename cplx_t<T>::type* X,
                         const typename cplx_t<T>::type* tw, cudaStream_t s);
