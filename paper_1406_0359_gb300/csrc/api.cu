@@ -411,7 +411,8 @@ template <typename T> class OpImpl : public purify_op {
     if (nbases) *nbases = sara.nbases;
     return m;
   }
-  size_t grid_bytes() const { return size_t(g.KP) * g.KP * sizeof(C); }
+  size_t grid_cells() const { return size_t(g.KP) * g.KC; }
+  size_t grid_bytes() const { return grid_cells() * sizeof(C); }
 
   // light: gridding-only operator (Phi^H; no forward grid, no uv copy), as
   // the PSF set-up of the convolution form needs.
@@ -432,10 +433,10 @@ template <typename T> class OpImpl : public purify_op {
     g.n = n;
     g.K = 2 * n;
     g.KP = g.K + kJ;
+    g.KC = n + kJ;
     g.pad_lo = kJ / 2 - 1;
     g.TB = tile > 0 ? tile : 8;
-    if (g.TB > g.K) g.TB = g.K;
-    g.ntile1d = g.K / g.TB;
+    g.ntv = n / g.TB;
     g.M = M;
     levels = L;
     // default work-item length by M (what purify_autotune usually picks:
@@ -498,8 +499,8 @@ template <typename T> class OpImpl : public purify_op {
     }
     if (!refine && (rc = alloc(&perm, M))) return rc;
     if ((rc = alloc(&gridA, size_t(n) * (g.K / 2)))) return rc;  // half-spectrum rows
-    if (!light && (rc = alloc(&gridP, size_t(g.KP) * g.KP))) return rc;
-    if ((rc = alloc(&gridQ, size_t(g.KP) * g.KP))) return rc;
+    if (!light && (rc = alloc(&gridP, grid_cells()))) return rc;
+    if ((rc = alloc(&gridQ, grid_cells()))) return rc;
     if ((rc = alloc(&sc, kNumScalars))) return rc;
     if ((rc = alloc(&err, 2))) return rc;  // [0] timed-out wait, [1] non-finite input
     sara.n = n;
@@ -546,9 +547,9 @@ template <typename T> class OpImpl : public purify_op {
     }
     const int cw = int(sizeof(C) / 8);
     const int PW = g.TB + kJ;
-    cuuint64_t dims[2] = {cuuint64_t(g.KP) * cw, cuuint64_t(g.KP)};
-    cuuint64_t strides[1] = {cuuint64_t(g.KP) * sizeof(C)};
-    cuuint32_t box[2] = {cuuint32_t((PW + 2) * cw), cuuint32_t(PW)};  // PW rows of PW + 2 (bank spread)
+    cuuint64_t dims[2] = {cuuint64_t(g.KC) * cw, cuuint64_t(g.KP)};
+    cuuint64_t strides[1] = {cuuint64_t(g.KC) * sizeof(C)};
+    cuuint32_t box[2] = {cuuint32_t(degrid_patch_pitch<T>(g.TB) * cw), cuuint32_t(PW)};
     cuuint32_t estr[2] = {1, 1};
     CUresult cr = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, gridP, dims, strides, box, estr,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -588,7 +589,7 @@ template <typename T> class OpImpl : public purify_op {
 
   // ---- operator building blocks (enqueue only)
   // F Z S in real form (the image is real): row pairs to half spectra, then
-  // the half-spectrum columns to the full padded grid with their mirrors.
+  // the half-spectrum columns to the padded half grid.
   RowFwdArgs<T> row_fwd_args(const RowPro<T>& pro, const T* dea, C* B) const {
     return RowFwdArgs<T>{g, pro, dea, B, tw, tws};
   }
@@ -603,11 +604,11 @@ template <typename T> class OpImpl : public purify_op {
   void fwd_grid(const RowPro<T>& pro, cudaStream_t s) {
     if (rec) {
       record(R_RF, s).rf = row_fwd_args(pro, deapod, gridA);
-      record(R_CF, s).cf = ColFwdArgs<T>{g, gridA, gridP, tw, col_pass_width<T>()};
+      record(R_CF, s).cf = ColFwdArgs<T>{g, gridA, gridP, tw, tws + tws_col};
       return;
     }
     PROF(KK_ROW_FWD, s, launch_row_fwd_h<T>(row_fwd_args(pro, deapod, gridA), s));
-    PROF(KK_COL_FWD, s, launch_col_fwd_h<T>(g, gridA, gridP, tw, s));
+    PROF(KK_COL_FWD, s, launch_col_fwd_h<T>(ColFwdArgs<T>{g, gridA, gridP, tw, tws + tws_col}, s));
   }
   void zero_q(cudaStream_t s) {
     if (rec) {
@@ -620,10 +621,10 @@ template <typename T> class OpImpl : public purify_op {
   // Hermitian part (the row pass follows in row_ep / normal_back).
   void col_inv(cudaStream_t s) {
     if (rec) {
-      record(R_CI, s).ci = ColInvArgs<T>{g, gridQ, gridA, tw, col_pass_width<T>()};
+      record(R_CI, s).ci = ColInvArgs<T>{g, gridQ, gridA, tw, tws + tws_col};
       return;
     }
-    PROF(KK_COL_INV, s, launch_col_inv_h<T>(g, gridQ, gridA, tw, s));
+    PROF(KK_COL_INV, s, launch_col_inv_h<T>(ColInvArgs<T>{g, gridQ, gridA, tw, tws + tws_col}, s));
   }
   void degrid(const DegridEp<C>& ep, cudaStream_t s) {
     if (rec) {
@@ -1287,6 +1288,7 @@ template <typename T> class OpImpl : public purify_op {
     const size_t tv = prior == 1 ? 2 * N() : 0;  // the TV prox's warm-started dual
     return int64_t(sizeof(StateHeader)) + int64_t((3 * N() + 2 * D() + 2 * size_t(g.M) + tv) * sizeof(T));
   }
+  static constexpr int kStateZ3 = 5;
   // (device array, element count) pairs in checkpoint order; returns their number.
   int state_arrays(T* (&a)[7], size_t (&len)[7]) const {
     T* arr[7] = {xh, xs, z1, z2, w, reinterpret_cast<T*>(z3), tvq};
@@ -1296,6 +1298,31 @@ template <typename T> class OpImpl : public purify_op {
       len[k] = l[k];
     }
     return prior == 1 ? 7 : 6;
+  }
+  // z_3 between the operator's sorted order and a checkpoint's (the whole
+  // grid's sorted order, which holds no mirror images): `to_file` fills tmp
+  // from z_3, otherwise z_3 from tmp.
+  int checkpoint_z3(C* tmp, bool to_file) {
+    const size_t M = size_t(g.M);
+    int *order = nullptr, *blk = nullptr;
+    C* caller = nullptr;
+    cudaError_t e = setup_alloc(&order, M * sizeof(int), own);
+    if (e == cudaSuccess) e = setup_alloc(&caller, M * sizeof(C), own);
+    if (e == cudaSuccess && nblocks > 1) e = setup_alloc(&blk, M * sizeof(int), own);
+    int rc = map_err(e, __LINE__);
+    if (!rc && blk) launch_slot_blocks(items, n_items, perm, blk, own);
+    if (!rc) rc = sort_order_plain(uv_keep, g.M, g, order, own, blk);
+    if (!rc && to_file) {
+      launch_scatter<C>(z3, perm, M, caller, own);
+      launch_gather<C>(caller, order, M, tmp, own);
+    } else if (!rc) {
+      launch_scatter<C>(tmp, order, M, caller, own);
+      launch_gather<C>(caller, perm, M, z3, own);
+    }
+    for (void* t : {static_cast<void*>(order), static_cast<void*>(blk), static_cast<void*>(caller)})
+      if (t) cudaFreeAsync(t, own);
+    if (!rc) rc = map_err(cudaStreamSynchronize(own), __LINE__);
+    return rc;
   }
   int save_state(void* host, int64_t bytes) override {
     if (!run.active || !host || bytes < state_bytes()) return PURIFY_ERR_INVALID;
@@ -1324,11 +1351,16 @@ template <typename T> class OpImpl : public purify_op {
     T* a[7];
     size_t len[7];
     const int na = state_arrays(a, len);
-    for (int k = 0; k < na; ++k) {
-      CK(cudaMemcpy(dst, a[k], len[k] * sizeof(T), cudaMemcpyDeviceToHost));
+    C* z3f = nullptr;
+    CK(setup_alloc(&z3f, size_t(g.M) * sizeof(C), own));
+    int rc = checkpoint_z3(z3f, true);
+    for (int k = 0; k < na && !rc; ++k) {
+      const T* from = k == kStateZ3 ? reinterpret_cast<const T*>(z3f) : a[k];
+      rc = map_err(cudaMemcpy(dst, from, len[k] * sizeof(T), cudaMemcpyDeviceToHost), __LINE__);
       dst += len[k] * sizeof(T);
     }
-    return PURIFY_OK;
+    cudaFreeAsync(z3f, own);
+    return rc;
   }
   int load_state(const void* host, int64_t bytes) override {
     if (!run.active || !host || bytes < state_bytes()) return PURIFY_ERR_INVALID;
@@ -1345,10 +1377,18 @@ template <typename T> class OpImpl : public purify_op {
     T* a[7];
     size_t len[7];
     const int na = state_arrays(a, len);
-    for (int k = 0; k < na; ++k) {
-      CK(cudaMemcpy(a[k], src, len[k] * sizeof(T), cudaMemcpyHostToDevice));
+    C* z3f = nullptr;
+    CK(setup_alloc(&z3f, size_t(g.M) * sizeof(C), own));
+    CK(cudaStreamSynchronize(own));
+    int rcl = PURIFY_OK;
+    for (int k = 0; k < na && !rcl; ++k) {
+      T* to = k == kStateZ3 ? reinterpret_cast<T*>(z3f) : a[k];
+      rcl = map_err(cudaMemcpy(to, src, len[k] * sizeof(T), cudaMemcpyHostToDevice), __LINE__);
       src += len[k] * sizeof(T);
     }
+    if (!rcl) rcl = checkpoint_z3(z3f, false);
+    cudaFreeAsync(z3f, own);
+    if (rcl) return rcl;
     run.round = h.round;
     run.t = h.t;
     run.total = h.total;

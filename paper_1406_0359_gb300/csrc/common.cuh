@@ -44,6 +44,14 @@ PD float2 csub(float2 a, float2 b) {
 template <typename C, typename T> PD C cscale(C a, T s) { a.x *= s; a.y *= s; return a; }
 template <typename C> PD C cmul_i(C a) { C r; r.x = -a.y; r.y = a.x; return r; }  // i * a
 
+// Entry p of an operator's permutation: the caller's index m, or ~m for a
+// visibility kept as its mirror image, whose value is conjugated.
+PD int perm_index(int p) { return p < 0 ? ~p : p; }
+template <typename C> PD C perm_value(int p, C v) {
+  if (p < 0) v.y = -v.y;
+  return v;
+}
+
 // Device error flag values (first writer wins).
 enum : int { DEV_OK = 0, DEV_TIMEOUT = 1 };
 

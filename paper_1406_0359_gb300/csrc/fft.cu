@@ -1,24 +1,22 @@
 // Oversampled 2D FFT passes of the NUFFT (operator F of Phi = G F Z S, Section 4).
 //
-// The row passes and the convolution's column pass transform by halves (even
-// and odd frequencies apart, see "half-length transforms" below); the column
-// passes of Phi and Phi^H run length-K (K = 2n, a power of two) Stockham
-// sequences of register radix-16 stages with shared-memory exchanges.
+// All passes transform by halves (even and odd frequencies apart, see
+// "half-length transforms" below); only the set-up of the PSF spectrum runs
+// plain length-K transforms (K = 2n, a power of two).
 //
 // The image is real, so every pass works in real form: two image rows a, b
 // travel as one complex row x_a + i x_b, and only the half spectra (columns
 // 0..K/2 of the row transforms) are kept, n x K/2 complex values, transposed.
 // Forward (Phi):   row pass over the n non-zero image rows (pairs), fused with
 //                  the deapodisation S and zero-padding Z; column pass over
-//                  the K/2 half-spectrum columns, writing each grid column
-//                  and its conjugate mirror into the padded grid (with its
-//                  periodic J-wide halo) that degridding stages by TMA.
-// Adjoint (Phi^H): column pass reading the padded gridding accumulator,
-//                  folding its halo back onto the torus and taking its
-//                  Hermitian part (Re of the image is all Phi^H keeps),
-//                  writing only the n rows the crop Z^T keeps; row pass
-//                  fused with the crop, the deapodisation and the solver
-//                  epilogues.
+//                  the half-spectrum columns into the padded half grid
+//                  (columns 0..n; periodic and mirrored J-wide halo) that
+//                  degridding stages by TMA.
+// Adjoint (Phi^H): column pass reading the padded gridding accumulator (half
+//                  grid), folding its halo and taking the Hermitian part
+//                  (Re of the image is all Phi^H keeps), writing only the n
+//                  rows the crop Z^T keeps; row pass fused with the crop, the
+//                  deapodisation and the solver epilogues.
 #include <cmath>
 #include <vector>
 
@@ -379,6 +377,27 @@ template <typename H, int DIR, typename C> PD void half_omega(C (&v)[H::E], int 
     if (DIR > 0) w.y = -w.y;
     if (m >= H::E / 2) w = cneg(w);
     v[m] = cmul(v[m], w);
+  }
+}
+
+// The sum of a column's two inverse halves into its n rows at Bc: each half
+// finishes half of the rows and hands over the rest through its buffer.
+template <typename H, typename C>
+PD void half_join(const C (&v)[H::E], int t, int odd, C* bufs, int half, C* Bc) {
+  constexpr int E = H::E, TT = H::TT;
+  C* s = bufs + size_t(half) * H::BUF;
+#pragma unroll
+  for (int m = 0; m < E / 2; ++m) {
+    if (odd) s[t + m * TT] = v[m];
+    else s[t + (m + E / 2) * TT] = v[m + E / 2];
+  }
+  __syncthreads();
+  const C* so = bufs + size_t(half ^ 1) * H::BUF;
+#pragma unroll
+  for (int m = 0; m < E / 2; ++m) {
+    const int me = m + (odd ? E / 2 : 0);
+    const C mine = odd ? v[m + E / 2] : v[m];
+    Bc[t + ((me + E / 2) & (E - 1)) * TT] = cadd(mine, so[t + me * TT]);
   }
 }
 
@@ -837,20 +856,7 @@ __global__ void __launch_bounds__(ColHalf<T, LOGN>::COL_THREADS, ColHalf<T, LOGN
   }
   half_fft<H, 1>(v, t, s, half, a.tws);
   if (odd) half_omega<H, 1>(v, t, tw);
-  // the halves' sum: each half finishes half of the rows and hands over the rest
-#pragma unroll
-  for (int m = 0; m < E / 2; ++m) {
-    if (odd) s[t + m * TT] = v[m];
-    else s[t + (m + E / 2) * TT] = v[m + E / 2];
-  }
-  __syncthreads();
-  const C* so = bufs + size_t(half ^ 1) * H::BUF;
-#pragma unroll
-  for (int m = 0; m < E / 2; ++m) {
-    const int me = m + (odd ? E / 2 : 0);
-    const C mine = odd ? v[m + E / 2] : v[m];
-    Bc[t + ((me + E / 2) & (E - 1)) * TT] = cadd(mine, so[t + me * TT]);
-  }
+  half_join<H>(v, t, odd, bufs, half, Bc);
 }
 
 // Operand arrays an epilogue reads (staged in shared memory by the inverse row
@@ -1026,115 +1032,165 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
   row_ep_finish(ep, part, red, int(blockIdx.x), a.nblocks);
 }
 
-// Real-form column passes of Phi and Phi^H on the padded grid (K + J per side,
-// periodic halo of J cells).  Grid cell (q, c) sits at padded row/column
-// q + pad_lo and also, near the edges, at its periodic image.
-PD int halo_images(int q, int K, int pl, int (&at)[2]) {
-  const int jhi = kJ - pl;  // grid indices < jhi repeat past the end
+// Real-form column passes of Phi and Phi^H on the padded half grid (K + J rows,
+// columns 0..n, a halo of J cells on both axes): grid cell (q, c) sits at row
+// q + pad_lo, column c + pad_lo; rows near the edges also at their periodic
+// image, and the halo's columns -c and 2n - c hold conj G(-q, c).  A CTA takes
+// COLS columns, c = COLS u + 1 + k, so that COLS cells of a grid row start on
+// a 32-byte sector; the last CTA's last column is the packed one, which holds
+// columns 0 and n.
+template <typename T, int LOGN>
+struct GridHalf : Half<T, LOGN, LOGN <= 8 ? 8 : (LOGN <= 9 || sizeof(T) == 8 ? 16 : 32)> {
+  typedef Half<T, LOGN, LOGN <= 8 ? 8 : (LOGN <= 9 || sizeof(T) == 8 ? 16 : 32)> Base;
+  static constexpr int COLS = kColBytes / int(sizeof(typename cplx_t<T>::type));
+  static constexpr int NT = COLS * 2 * Base::TT;
+  static constexpr int MINB = NT >= 512 ? 1 : 512 / NT;
+};
+
+// Padded rows of grid row q (its periodic image too, near the edges).
+PD int halo_rows(int q, int K, int pl, int (&at)[2]) {
   at[0] = q + pl;
-  at[1] = q >= K - pl ? q + pl - K : (q < jhi ? q + pl + K : -1);
-  return at[1] >= 0 ? 2 : 1;
+  at[1] = q >= K - pl ? q + pl - K : q + pl + K;
+  return q >= K - pl || q < kJ - pl ? 2 : 1;
 }
 
-// Phi: cw half-spectrum columns c per CTA.  For the image rows' half spectra
-// X(., c), c < K/2, the column FFT gives grid column c, and column K - c is
-// its conjugate mirror, G(q, K - c) = conj G(-q, c) (a real image).  Column 0
-// carries X(., 0) + i X(., K/2): its transform P gives grid column 0 as
-// (P(q) + conj P(-q)) / 2 and column K/2 as -i (P(q) - conj P(-q)) / 2.
-// One CTA per SM, spill-free (measured 22.3 against 24.6 us at K = 2048 for
-// two spilling CTAs per SM; the adjoint pass below measured slower that way,
-// 39.4 against 36.4 us, and keeps two).
+// Phi: the column FFT of the image rows' half spectra X(., c) gives grid
+// column c.  The packed column X(., 0) + i X(., n) transforms to P; column 0
+// is (P(q) + conj P(-q)) / 2 and column n is -i (P(q) - conj P(-q)) / 2.
+// Bound by its writes (a half grid of 17 MB at n = 1024) and latency: 15.2 us
+// against 19.9 us for the whole grid by 2048-point transforms.
 template <typename T, int LOGN, typename Src>
-__global__ void __launch_bounds__(ColThreads<T, LOGN>::value, 1)
-    k_col_fwd_h(Src src) {
+__global__ void __launch_bounds__(GridHalf<T, LOGN>::NT, GridHalf<T, LOGN>::MINB) k_col_fwd_h(Src src) {
   typedef typename cplx_t<T>::type C;
+  typedef GridHalf<T, LOGN> H;
+  constexpr int n = H::N, K = 2 * n, E = H::E, TT = H::TT, NC = H::COLS;
   decltype(auto) a = src.get();
-  const Geometry& g = a.g;
-  const C* __restrict__ B = a.B;
   C* __restrict__ Pg = a.Pg;
-  const C* __restrict__ tw = a.tw;
-  const int cw = a.cw;
-  constexpr int TT = Plan<LOGN>::T;
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int K = g.K, n = g.n, half = n / 2, H = K / 2, pl = g.pad_lo, KP = g.KP;
-  const int cc = threadIdx.x % cw, t = threadIdx.x / cw;
-  const int c = blockIdx.x * cw + cc;
-  C* s = reinterpret_cast<C*>(sm_raw) + cc;
-  auto load = [&](int m) -> C {
-    const int i1 = (t + m * TT + half) & (K - 1);
-    return i1 < n ? B[half_at(c, i1, n)] : cz<C>();
-  };
-  auto to_smem = [&](int q, C v) { s[sidx(q) * cw] = v; };
-  fft_seq<LOGN>(t, s, cw, tw, -1, load, to_smem);
+  C* bufs = reinterpret_cast<C*>(sm_raw);
+  const int pl = a.g.pad_lo, KC = a.g.KC;
+  const int half = threadIdx.x / TT, t = threadIdx.x - half * TT, odd = half & 1;
+  const int c0 = NC * int(blockIdx.x) + 1;
+  const bool packed = c0 + NC - 1 == n;  // this CTA's last column
+  C* s = bufs + size_t(half) * H::BUF;
+  {
+    const int c = c0 + (half >> 1);
+    const C* __restrict__ Bc = a.B + (c == n ? size_t(0) : half_at(c, 0, n));
+    C v[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = Bc[t + ((m + E / 2) & (E - 1)) * TT];
+    if (odd) half_omega<H, -1>(v, t, a.tw);
+    half_fft<H, -1>(v, t, s, half, a.tws);
+#pragma unroll
+    for (int m = 0; m < E; ++m) s[t + m * TT] = v[m];
+  }
   __syncthreads();
-  auto put = [&](int q, int col, C v) {
-    int rows[2], cols[2];
-    const int nr = halo_images(q, K, pl, rows), nc = halo_images(col, K, pl, cols);
-    for (int a = 0; a < nr; ++a)
-      for (int b = 0; b < nc; ++b) Pg[size_t(rows[a]) * KP + cols[b]] = v;
-  };
-#pragma unroll 4
-  for (int m = 0; m < 16; ++m) {
-    const int q = t + m * TT, qm = (K - q) & (K - 1);
-    const C P = s[sidx(q) * cw];
-    if (c != 0) {
-      put(q, c, P);
-      put(qm, K - c, cmk<C>(P.x, -P.y));
-    } else {
-      const C Pm = s[sidx(qm) * cw];
-      put(q, 0, cmk<C>(T(0.5) * (P.x + Pm.x), T(0.5) * (P.y - Pm.y)));
-      // -i (P - conj Pm) / 2
-      put(q, H, cmk<C>(T(0.5) * (P.y + Pm.y), T(0.5) * (Pm.x - P.x)));
+  for (int q = threadIdx.x; q < K; q += H::NT) {
+    const int o = q & 1, m = q >> 1;
+    C out[NC], col0 = cz<C>();
+#pragma unroll
+    for (int k = 0; k < NC; ++k) out[k] = bufs[size_t(2 * k + o) * H::BUF + m];
+    if (packed) {
+      const C P = out[NC - 1], Pm = bufs[size_t(2 * (NC - 1) + o) * H::BUF + (o ? n - 1 - m : (n - m) & (n - 1))];
+      col0 = cmk<C>(T(0.5) * (P.x + Pm.x), T(0.5) * (P.y - Pm.y));
+      out[NC - 1] = cmk<C>(T(0.5) * (P.y + Pm.y), T(0.5) * (Pm.x - P.x));
+    }
+    int at[2], am[2];
+    const int nr = halo_rows(q, K, pl, at), nm = halo_rows((K - q) & (K - 1), K, pl, am);
+    for (int r = 0; r < nr; ++r) {
+      st32(Pg + size_t(at[r]) * KC + c0 + pl, out);
+      if (packed) Pg[size_t(at[r]) * KC + pl] = col0;
+    }
+    if (c0 <= pl || c0 + NC > n - pl) {  // columns whose mirror image lies in the halo
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const int c = c0 + k;
+        const C w = cmk<C>(out[k].x, -out[k].y);
+        for (int r = 0; r < nm; ++r) {
+          if (c <= pl) Pg[size_t(am[r]) * KC + pl - c] = w;
+          if (c < n && c >= n - pl) Pg[size_t(am[r]) * KC + 2 * n - c + pl] = w;
+        }
+      }
     }
   }
 }
 
 // Phi^H: Re of the inverse transform of the gridded accumulator Q is the
-// inverse transform of its Hermitian part Qh(q, c) = (Q(q, c) + conj Q(-q, -c)) / 2,
-// so only columns c <= K/2 are transformed: cw half-spectrum columns per
-// CTA (halo folded on load), inverse column FFT, the n cropped rows into the
-// half-spectrum rows B; column 0 packs the two Hermitian columns 0 and K/2 as
-// Qh(., 0) + i Qh(., K/2), whose transforms are real.
+// inverse transform of its Hermitian part Qh(q, c) = (Q(q, c) + conj Q(-q, -c)) / 2.
+// Away from the halo's columns the second term is empty (every visibility was
+// gridded in the lower half), so a column is read once, its row halo folded,
+// then transformed (inverse, by halves), the n cropped rows into the
+// half-spectrum rows B; the packed column is Qh(., 0) + i Qh(., n), whose
+// transforms are real.  18.6 us against 34.4 us for the whole grid (n = 1024),
+// where every element waited for two dependent, folded reads.
 template <typename T, int LOGN, typename Src>
-__global__ void __launch_bounds__(ColThreads<T, LOGN>::value, ColThreads<T, LOGN>::value <= 512 ? 2 : 1)
-    k_col_inv_h(Src src) {
+__global__ void __launch_bounds__(GridHalf<T, LOGN>::NT, GridHalf<T, LOGN>::MINB) k_col_inv_h(Src src) {
   typedef typename cplx_t<T>::type C;
+  typedef GridHalf<T, LOGN> H;
+  constexpr int n = H::N, K = 2 * n, E = H::E, TT = H::TT, NC = H::COLS;
   decltype(auto) a = src.get();
-  const Geometry& g = a.g;
   const C* __restrict__ Q = a.Q;
-  C* __restrict__ B = a.B;
-  const C* __restrict__ tw = a.tw;
-  const int cw = a.cw;
-  constexpr int TT = Plan<LOGN>::T;
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int K = g.K, n = g.n, half = n / 2, H = K / 2, pl = g.pad_lo, KP = g.KP;
-  const int cc = threadIdx.x % cw, t = threadIdx.x / cw;
-  const int c = blockIdx.x * cw + cc;
-  C* s = reinterpret_cast<C*>(sm_raw) + cc;
-  auto fold = [&](int q, int col) -> C {
-    int rows[2], cols[2];
-    const int nr = halo_images(q, K, pl, rows), nc = halo_images(col, K, pl, cols);
-    C v = cz<C>();
-    for (int a = 0; a < nr; ++a)
-      for (int b = 0; b < nc; ++b) v = cadd(v, Q[size_t(rows[a]) * KP + cols[b]]);
+  C* bufs = reinterpret_cast<C*>(sm_raw);
+  const int pl = a.g.pad_lo, KC = a.g.KC;
+  const int half = threadIdx.x / TT, t = threadIdx.x - half * TT, odd = half & 1;
+  const int c0 = NC * int(blockIdx.x) + 1;
+  const bool packed = c0 + NC - 1 == n;
+  auto fold = [&](int q, int c) -> C {  // one cell with its row images
+    int at[2];
+    const int nr = halo_rows(q & (K - 1), K, pl, at);
+    C v = Q[size_t(at[0]) * KC + c + pl];
+    if (nr > 1) v = cadd(v, Q[size_t(at[1]) * KC + c + pl]);
     return v;
   };
-  auto load = [&](int m) -> C {
-    const int q = t + m * TT, qm = (K - q) & (K - 1);
-    if (c != 0) {
-      const C a = fold(q, c), b = fold(qm, K - c);
-      return cmk<C>(T(0.5) * (a.x + b.x), T(0.5) * (a.y - b.y));
+  constexpr int IT = K / H::NT, U = IT % 4 == 0 ? 4 : (IT % 2 == 0 ? 2 : 1);  // U sector loads in flight
+  static_assert(K % H::NT == 0, "E is a multiple of COLS");
+  for (int it = 0; it < IT; it += U) {
+    C in[U][NC];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      ld32(in[u], Q + size_t(int(threadIdx.x) + (it + u) * H::NT + pl) * KC + c0 + pl);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int q = int(threadIdx.x) + (it + u) * H::NT, o = q & 1, m = q >> 1;
+      int at[2];
+      if (halo_rows(q, K, pl, at) > 1) {
+        C im[NC];
+        ld32(im, Q + size_t(at[1]) * KC + c0 + pl);
+#pragma unroll
+        for (int k = 0; k < NC; ++k) in[u][k] = cadd(in[u][k], im[k]);
+      }
+      if (c0 <= pl || c0 + NC > n - pl) {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+          const int c = c0 + k;
+          if (c <= pl || c >= n - pl) {  // the mirror image's column: -c, or 2n - c (c itself for c = n)
+            const C w = fold(K - q, c <= pl ? -c : 2 * n - c);
+            in[u][k] = cmk<C>(in[u][k].x + w.x, in[u][k].y - w.y);
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < NC; ++k) in[u][k] = cscale(in[u][k], T(0.5));
+      if (packed) {
+        const C a0 = fold(q, 0), b0 = fold(K - q, 0);
+        const C h0 = cmk<C>(T(0.5) * (a0.x + b0.x), T(0.5) * (a0.y - b0.y)), hn = in[u][NC - 1];
+        in[u][NC - 1] = cmk<C>(h0.x - hn.y, h0.y + hn.x);  // h0 + i hn
+      }
+#pragma unroll
+      for (int k = 0; k < NC; ++k) bufs[size_t(2 * k + o) * H::BUF + m] = in[u][k];
     }
-    const C a0 = fold(q, 0), b0 = fold(qm, 0), aH = fold(q, H), bH = fold(qm, H);
-    const C h0 = cmk<C>(T(0.5) * (a0.x + b0.x), T(0.5) * (a0.y - b0.y));
-    const C hH = cmk<C>(T(0.5) * (aH.x + bH.x), T(0.5) * (aH.y - bH.y));
-    return cmk<C>(h0.x - hH.y, h0.y + hH.x);  // h0 + i hH
-  };
-  auto store = [&](int q, C v) {
-    const int i1 = (q + half) & (K - 1);
-    if (i1 < n) B[half_at(c, i1, n)] = v;
-  };
-  fft_seq<LOGN>(t, s, cw, tw, +1, load, store);
+  }
+  __syncthreads();
+  C* s = bufs + size_t(half) * H::BUF;
+  C v[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) v[m] = s[t + m * TT];
+  half_sync<TT>(half);
+  half_fft<H, 1>(v, t, s, half, a.tws);
+  if (odd) half_omega<H, 1>(v, t, a.tw);
+  const int c = c0 + (half >> 1);
+  half_join<H>(v, t, odd, bufs, half, a.B + (c == n ? size_t(0) : half_at(c, 0, n)));
 }
 
 // Plain in-place transforms of a K x K complex array (set-up of the PSF spectrum).
@@ -1183,10 +1239,6 @@ __global__ void __launch_bounds__(ColThreads<T, LOGN>::value) k_cols_plain(typen
 }  // namespace
 
 
-template <typename T> int col_pass_width() { return col_width<T>(); }
-template int col_pass_width<float>();
-template int col_pass_width<double>();
-
 #define PURIFY_LOGN_SWITCH(K, BODY)     \
   switch (K) {                          \
     case 32: { constexpr int L = 5; BODY; } break;   \
@@ -1214,14 +1266,14 @@ template int col_pass_width<double>();
 template <typename T, int L> cudaError_t configure_one() {
   cudaError_t e = raise_smem_limit(k_row_fwd_h<T, L - 1, ArgVal<RowFwdArgs<T>>>);
   if (e == cudaSuccess) e = raise_smem_limit(k_col_conv_h<T, L - 1, ArgVal<ColConvArgs<T>>>);
-  if (e == cudaSuccess) e = raise_smem_limit(k_col_fwd_h<T, L, ArgVal<ColFwdArgs<T>>>);
-  if (e == cudaSuccess) e = raise_smem_limit(k_col_inv_h<T, L, ArgVal<ColInvArgs<T>>>);
+  if (e == cudaSuccess) e = raise_smem_limit(k_col_fwd_h<T, L - 1, ArgVal<ColFwdArgs<T>>>);
+  if (e == cudaSuccess) e = raise_smem_limit(k_col_inv_h<T, L - 1, ArgVal<ColInvArgs<T>>>);
   if (e == cudaSuccess) e = raise_smem_limit(k_row_inv_h<T, L - 1, ArgVal<RowInvArgs<T>>>);
   if constexpr (L >= 7 && L <= 11) {
     if (e == cudaSuccess) e = raise_smem_limit(k_row_fwd_h<T, L - 1, ArgTab<RowFwdArgs<T>>>);
     if (e == cudaSuccess) e = raise_smem_limit(k_col_conv_h<T, L - 1, ArgTab<ColConvArgs<T>>>);
-    if (e == cudaSuccess) e = raise_smem_limit(k_col_fwd_h<T, L, ArgTab<ColFwdArgs<T>>>);
-    if (e == cudaSuccess) e = raise_smem_limit(k_col_inv_h<T, L, ArgTab<ColInvArgs<T>>>);
+    if (e == cudaSuccess) e = raise_smem_limit(k_col_fwd_h<T, L - 1, ArgTab<ColFwdArgs<T>>>);
+    if (e == cudaSuccess) e = raise_smem_limit(k_col_inv_h<T, L - 1, ArgTab<ColInvArgs<T>>>);
     if (e == cudaSuccess) e = raise_smem_limit(k_row_inv_h<T, L - 1, ArgTab<RowInvArgs<T>>>);
   }
   if (e == cudaSuccess) e = raise_smem_limit(k_rows_plain<T, L>);
@@ -1288,6 +1340,9 @@ template <typename T, int LOGN> struct HalfShape {
   static size_t inv_smem(bool operands) {
     return align16(size_t(H::PAIRS) * 2 * H::BUF * sizeof(C)) + (operands ? size_t(H::PAIRS) * 4 * H::N * sizeof(T) : 0);
   }
+  typedef GridHalf<T, LOGN> HG;
+  static constexpr int grid_ctas = H::N / HG::COLS;
+  static size_t grid_smem() { return size_t(HG::COLS) * 2 * HG::BUF * sizeof(C); }
   static size_t conv_smem() { return size_t(HC::COLS) * 2 * HC::BUF * sizeof(C); }
 };
 // CTAs of one inverse row pass (its epilogue's partial sums).
@@ -1300,7 +1355,7 @@ template int row_inv_blocks<float>(const Geometry&);
 template int row_inv_blocks<double>(const Geometry&);
 // Twiddles of the half transforms of length n: per stage after the first,
 // W(r k) = exp(-2 pi i r k / (Ns R)) as [r - 1][k], k < Ns; the row passes'
-// table, then the convolution's from element *col_at on.
+// table, then the column passes' from element *col_at on.
 template <typename H, typename C> static void half_twiddles_of(std::vector<C>& out) {
   int ns = H::radix(0);
   for (int st = 1; st < H::NST; ++st) {
@@ -1324,10 +1379,6 @@ template <typename T> void half_twiddles(int n, std::vector<typename cplx_t<T>::
 }
 template void half_twiddles<float>(int, std::vector<float2>&, size_t*);
 template void half_twiddles<double>(int, std::vector<double2>&, size_t*);
-template <typename T> inline size_t col_smem(const Geometry& g) {
-  return col_width<T>() * padded(g.K) * sizeof(typename cplx_t<T>::type);
-}
-
 template <typename T> void launch_row_fwd_h(const RowFwdArgs<T>& a, cudaStream_t s) {
   ArgVal<RowFwdArgs<T>> src{a};
   PURIFY_LOGN_SWITCH(a.g.K, (k_row_fwd_h<T, L - 1><<<HalfShape<T, L - 1>::row_ctas, RowHalf<T, L - 1>::ROW_THREADS,
@@ -1340,20 +1391,16 @@ template <typename T> void launch_col_conv_h(const ColConvArgs<T>& a, cudaStream
                                                       HalfShape<T, L - 1>::conv_smem(), s>>>(src)));
 }
 
-template <typename T>
-void launch_col_fwd_h(const Geometry& g, const typename cplx_t<T>::type* B, typename cplx_t<T>::type* Pg,
-                      const typename cplx_t<T>::type* tw, cudaStream_t s) {
-  const int cw = col_width<T>();
-  ArgVal<ColFwdArgs<T>> src{ColFwdArgs<T>{g, B, Pg, tw, cw}};
-  PURIFY_LOGN_SWITCH(g.K, (k_col_fwd_h<T, L><<<g.K / 2 / cw, cw * Plan<L>::T, col_smem<T>(g), s>>>(src)));
+template <typename T> void launch_col_fwd_h(const ColFwdArgs<T>& a, cudaStream_t s) {
+  ArgVal<ColFwdArgs<T>> src{a};
+  PURIFY_LOGN_SWITCH(a.g.K, (k_col_fwd_h<T, L - 1><<<HalfShape<T, L - 1>::grid_ctas, GridHalf<T, L - 1>::NT,
+                                                     HalfShape<T, L - 1>::grid_smem(), s>>>(src)));
 }
 
-template <typename T>
-void launch_col_inv_h(const Geometry& g, const typename cplx_t<T>::type* Q, typename cplx_t<T>::type* B,
-                      const typename cplx_t<T>::type* tw, cudaStream_t s) {
-  const int cw = col_width<T>();
-  ArgVal<ColInvArgs<T>> src{ColInvArgs<T>{g, Q, B, tw, cw}};
-  PURIFY_LOGN_SWITCH(g.K, (k_col_inv_h<T, L><<<g.K / 2 / cw, cw * Plan<L>::T, col_smem<T>(g), s>>>(src)));
+template <typename T> void launch_col_inv_h(const ColInvArgs<T>& a, cudaStream_t s) {
+  ArgVal<ColInvArgs<T>> src{a};
+  PURIFY_LOGN_SWITCH(a.g.K, (k_col_inv_h<T, L - 1><<<HalfShape<T, L - 1>::grid_ctas, GridHalf<T, L - 1>::NT,
+                                                     HalfShape<T, L - 1>::grid_smem(), s>>>(src)));
 }
 
 template <typename T> void launch_row_inv_h(const RowInvArgs<T>& a, cudaStream_t s) {
@@ -1381,15 +1428,17 @@ void launch_col_conv_h_batch(const Geometry& g, const ColConvArgs<T>* tab, int c
 }
 template <typename T>
 void launch_col_fwd_h_batch(const Geometry& g, const ColFwdArgs<T>* tab, int count, cudaStream_t s) {
-  const int cw = col_width<T>();
   ArgTab<ColFwdArgs<T>> src{tab};
-  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_col_fwd_h<T, L><<<dim3(g.K / 2 / cw, count), cw * Plan<L>::T, col_smem<T>(g), s>>>(src)));
+  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_col_fwd_h<T, L - 1><<<dim3(HalfShape<T, L - 1>::grid_ctas, count),
+                                                         GridHalf<T, L - 1>::NT, HalfShape<T, L - 1>::grid_smem(),
+                                                         s>>>(src)));
 }
 template <typename T>
 void launch_col_inv_h_batch(const Geometry& g, const ColInvArgs<T>* tab, int count, cudaStream_t s) {
-  const int cw = col_width<T>();
   ArgTab<ColInvArgs<T>> src{tab};
-  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_col_inv_h<T, L><<<dim3(g.K / 2 / cw, count), cw * Plan<L>::T, col_smem<T>(g), s>>>(src)));
+  PURIFY_LOGN_SWITCH_BATCH(g.K, (k_col_inv_h<T, L - 1><<<dim3(HalfShape<T, L - 1>::grid_ctas, count),
+                                                         GridHalf<T, L - 1>::NT, HalfShape<T, L - 1>::grid_smem(),
+                                                         s>>>(src)));
 }
 template <typename T>
 void launch_row_inv_h_batch(const Geometry& g, const RowInvArgs<T>* tab, int count, cudaStream_t s) {
@@ -1418,10 +1467,8 @@ void launch_fft2_plain(int K, typename cplx_t<T>::type* X, const typename cplx_t
   template void launch_col_conv_h<T>(const ColConvArgs<T>&, cudaStream_t);                                   \
   template void launch_row_inv_h<T>(const RowInvArgs<T>&, cudaStream_t);                                     \
   template void launch_fft2_plain<T>(int, cplx_t<T>::type*, const cplx_t<T>::type*, int, cudaStream_t);     \
-  template void launch_col_fwd_h<T>(const Geometry&, const cplx_t<T>::type*, cplx_t<T>::type*,                \
-                                    const cplx_t<T>::type*, cudaStream_t);                                     \
-  template void launch_col_inv_h<T>(const Geometry&, const cplx_t<T>::type*, cplx_t<T>::type*,                \
-                                    const cplx_t<T>::type*, cudaStream_t);                                     \
+  template void launch_col_fwd_h<T>(const ColFwdArgs<T>&, cudaStream_t);                                     \
+  template void launch_col_inv_h<T>(const ColInvArgs<T>&, cudaStream_t);                                     \
   template void build_psf_spectrum<T>(const T*, int, T*, cplx_t<T>::type*, const cplx_t<T>::type*, cudaStream_t); \
   template void launch_row_fwd_h_batch<T>(const Geometry&, const RowFwdArgs<T>*, int, cudaStream_t);         \
   template void launch_col_conv_h_batch<T>(const Geometry&, const ColConvArgs<T>*, int, cudaStream_t);       \

@@ -2,16 +2,18 @@
 //
 // HBM layout of one operator (T = float or double, C = complex<T>):
 //   pos    [M]        visibility positions in uv-tile order (Pos<T>)
-//   perm   [M]        sorted slot -> caller's visibility index
+//   perm   [M]        sorted slot -> caller's visibility index m, or ~m where the
+//                     visibility is kept as its mirror image (see Geometry)
 //   items  [n_items]  work items: (tile, first slot, end slot), <= chunk slots each
 //   gridA  [n][K/2]   half-spectrum rows: the row FFTs of image row pairs
 //                     x_a + i x_b split into the half spectra of rows a and b
 //                     (entry 0 = X(0) + i X(K/2)), after the forward row pass
 //                     or before the inverse one
-//   gridP  [KP][KP]   forward oversampled grid with a J-wide periodic halo,
+//   gridP  [KP][KC]   forward oversampled grid, columns 0..n with a J-wide halo,
 //                     read in (TB+J)^2 patches by TMA for degridding
-//   gridQ  [KP][KP]   gridding accumulator with the same halo (folded on read)
-// with K = 2n the oversampled grid side and KP = K + J its padded side.
+//   gridQ  [KP][KC]   gridding accumulator with the same halo (folded on read)
+// with K = 2n the oversampled grid side, KP = K + J padded rows and KC = n + J
+// padded columns.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -45,8 +47,15 @@ template <> struct Pos<double> { double u, v; };
 
 struct WorkItem { int tile, begin, end, pad; };  // pad: visibility block of the item
 
+// The image is real, so y(-u, -v) = conj y(u, v): a visibility whose grid
+// column lies in the upper half [n, K) is kept as its mirror image -- cell and
+// offset reflected on both axes, value conjugated on the way in and out (perm)
+// -- and only the grid's columns 0..n (and a J-wide halo) exist.  Half the
+// grid is written, zeroed, gathered and folded, and its tiles hold twice the
+// visibilities.  The reflected cell is K - 1 - cell with offset 1 - f, whose
+// taps are exactly the mirror images of the original ones.
 struct Geometry {
-  int n, K, KP, pad_lo, TB, ntile1d;
+  int n, K, KP, KC, pad_lo, TB, ntv;  // ntv: uv tiles along the second axis (n / TB); K / TB along the first
   int64_t M;
 };
 
@@ -163,14 +172,14 @@ template <typename T> struct ColFwdArgs {
   const typename cplx_t<T>::type* B;
   typename cplx_t<T>::type* Pg;
   const typename cplx_t<T>::type* tw;
-  int cw;
+  const typename cplx_t<T>::type* tws;
 };
 template <typename T> struct ColInvArgs {
   Geometry g;
   const typename cplx_t<T>::type* Q;
   typename cplx_t<T>::type* B;
   const typename cplx_t<T>::type* tw;
-  int cw;
+  const typename cplx_t<T>::type* tws;
 };
 
 // Arguments of the warp-per-item degridding / gridding (one operator; a batch
@@ -218,11 +227,9 @@ template <typename T> cudaError_t configure_sara();
 
 // CTAs of one inverse row pass (the partial sums its epilogue writes).
 template <typename T> int row_inv_blocks(const Geometry& g);
-// Stage twiddles of the row passes and the convolution's column pass for
-// image side n (one table per operator).
+// Stage twiddles of the row passes and (from element *col_at on) the column
+// passes for image side n.
 template <typename T> void half_twiddles(int n, std::vector<typename cplx_t<T>::type>& out, size_t* col_at);
-// Interleaved columns per CTA of the column passes of Phi and Phi^H.
-template <typename T> int col_pass_width();
 // Composite operator Phi^H Phi as a convolution, in real form: the image
 // rows' half spectra (n x K/2 complex in B, stored transposed; entry 0 =
 // X(0) + i X(K/2)).  Forward row pass (prologue, zero-padding, row FFT of row
@@ -232,15 +239,11 @@ template <typename T> void launch_row_fwd_h(const RowFwdArgs<T>& a, cudaStream_t
 // (per column its even grid rows, then its odd ones; column K/2 at knyq),
 // inverse FFT, crop (in place).
 template <typename T> void launch_col_conv_h(const ColConvArgs<T>& a, cudaStream_t s);
-// Real-form column passes of Phi (half-spectrum rows B -> the full padded
-// grid, mirrored columns included) and Phi^H (padded accumulator Q -> the
-// half-spectrum rows of its Hermitian part).
-template <typename T>
-void launch_col_fwd_h(const Geometry& g, const typename cplx_t<T>::type* B, typename cplx_t<T>::type* Pg,
-                      const typename cplx_t<T>::type* tw, cudaStream_t s);
-template <typename T>
-void launch_col_inv_h(const Geometry& g, const typename cplx_t<T>::type* Q, typename cplx_t<T>::type* B,
-                      const typename cplx_t<T>::type* tw, cudaStream_t s);
+// Real-form column passes of Phi (half-spectrum rows B -> the padded half grid
+// with its halo) and Phi^H (padded accumulator Q -> the half-spectrum rows of
+// its Hermitian part).
+template <typename T> void launch_col_fwd_h(const ColFwdArgs<T>& a, cudaStream_t s);
+template <typename T> void launch_col_inv_h(const ColInvArgs<T>& a, cudaStream_t s);
 // Inverse row pass with the row epilogue (deapod: S^T, or null); its epilogue
 // writes row_inv_blocks partial sums.
 template <typename T> void launch_row_inv_h(const RowInvArgs<T>& a, cudaStream_t s);
@@ -264,6 +267,8 @@ template <typename T>
 void launch_fft2_plain(int K, typename cplx_t<T>::type* X, const typename cplx_t<T>::type* tw, int dir,
                        cudaStream_t s);
 
+// Row pitch of degridding's staged patch, in cells (the TMA box's width).
+template <typename T> int degrid_patch_pitch(int TB);
 template <typename T>
 void launch_degrid(const Geometry& g, const CUtensorMap& map, const WorkItem* items, int n_items,
                    const Pos<T>* pos, const int* perm, const KbPoly<T>& kb, const DegridEp<typename cplx_t<T>::type>& ep,
@@ -300,6 +305,12 @@ template <typename U> cudaError_t setup_alloc(U** p, size_t bytes, cudaStream_t 
 // item lies in one block (its `pad` field).
 // Positions for the grid of twice the resolution of a binning of the Kc grid
 // (fine tiles TB = 2 x the coarse tiles): the coarse items and order serve.
+// Order of the visibilities by (block, tile, cell) on the whole grid, without
+// mirror images: the order of z_3 in a checkpoint (blocks: per visibility in
+// caller order, or null).  order[s] = caller's index; synchronises s.
+int sort_order_plain(const double* uv, int64_t M, const Geometry& g, int* order, cudaStream_t s, const int* blocks);
+// Block of every visibility in caller order, from the work items.
+void launch_slot_blocks(const WorkItem* items, int n_items, const int* perm, int* blocks, cudaStream_t s);
 template <typename T>
 void launch_encode_x2(const double* uv, const int* perm, int64_t M, int Kc, int TB, Pos<T>* pos, cudaStream_t s);
 // items_pool: allocate the work list from this pool on `s` (else cudaMalloc).

@@ -81,14 +81,14 @@ template <> PD void atomic_add_global<double2>(double2* p, double2 v) {
 // columns are read past the grid's edge on the last tile column, where the
 // tensor copy fills zeros, and never used).
 template <typename C>
-PD bool stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu, int tv, int TB, int PW, int* err) {
+PD bool stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu, int tv, int TB, int PW, int PP, int* err) {
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     fence_barrier_init();
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    mbar_arrive_expect_tx(bar, uint32_t(PW * (PW + 2) * sizeof(C)));
+    mbar_arrive_expect_tx(bar, uint32_t(PW * PP * sizeof(C)));
     const int cw = int(sizeof(C) / 8);
     tma_load_2d(patch, map, tv * TB * cw, tu * TB, bar);
   }
@@ -158,7 +158,7 @@ template <> PD void stage_store_grid<double>(double* st, const double (&wu)[kJ],
 
 template <typename T> __host__ __device__ inline size_t tile_patch_bytes(int TB) {
   const size_t PW = size_t(TB + kJ);
-  return PW * (PW + 2) * sizeof(typename cplx_t<T>::type);
+  return PW * (sizeof(T) == 4 ? 24 : PW + 2) * sizeof(typename cplx_t<T>::type);
 }
 template <typename T> __host__ __device__ inline size_t tile_acc_bytes(int TB) {
   const size_t PW = size_t(TB + kJ);
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kThreads) k_tile(Geometry g, const __grid_cons
   __shared__ __align__(8) uint64_t bar;
   __shared__ double red[32];
   const WorkItem it = items[blockIdx.x];
-  const int tu = it.tile / g.ntile1d, tv = it.tile - tu * g.ntile1d;
+  const int tu = it.tile / g.ntv, tv = it.tile - tu * g.ntv;
   const int PW = g.TB + kJ, PA = PW + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned char* cur = sm_raw;
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kThreads) k_tile(Geometry g, const __grid_cons
   }
   T* stage = reinterpret_cast<T*>(cur);
   if (kGather) {
-    if (!stage_patch(patch, &bar, &map, tu, tv, g.TB, PW, err)) return;
+    if (!stage_patch(patch, &bar, &map, tu, tv, g.TB, PW, sizeof(T) == 4 ? 24 : PW + 2, err)) return;
   } else {
     __syncthreads();
   }
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kThreads) k_tile(Geometry g, const __grid_cons
       kb_eval(kb, fv, wv);
       if (MODE == TM_GRID) {
         if (gpro.mode == GP_PERM) {
-          u = gpro.y[perm[i]];
+          u = perm_value(perm[i], gpro.y[perm_index(perm[i])]);
         } else if (gpro.mode == GP_SORTED) {
           u = gpro.y[i];
         } else {  // GP_BALL
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kThreads) k_tile(Geometry g, const __grid_cons
       const T* sj = wst + j * kStage;
       const int cell = *reinterpret_cast<const int*>(sj + 2 * kJ + 2);
       if (cell != cell_cur) {  // warp-uniform
-        const int ro = ((cell >> 8) + ta) * (PW + 2) + (cell & 255) + tb;
+        const int ro = ((cell >> 8) + ta) * (sizeof(T) == 4 ? 24 : PW + 2) + (cell & 255) + tb;
         if (kScatter && cell_cur >= 0) {
           C* row = wacc + ((cell_cur >> 8) + ta) * PA + (cell_cur & 255) + tb;
           row[0] = cadd(row[0], s0);
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kThreads) k_tile(Geometry g, const __grid_cons
     __syncwarp();
     if (MODE == TM_DEGRID && valid) {
       if (dep.mode == DG_STORE_PERM) {
-        dep.y[perm[i]] = mine;
+        dep.y[perm_index(perm[i])] = perm_value(perm[i], mine);
       } else if (dep.mode == DG_STORE_SORTED) {
         dep.y[i] = mine;
       } else {  // DG_BALL
@@ -353,11 +353,9 @@ __global__ void __launch_bounds__(kThreads) k_tile(Geometry g, const __grid_cons
     C v = cz<C>();
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) v = cadd(v, acc[w * PW * PA + r * PA + c]);
-    if (v.x != 0 || v.y != 0) atomic_add_global(Q + size_t(tu * g.TB + r) * g.KP + (tv * g.TB + c), v);
+    if (v.x != 0 || v.y != 0) atomic_add_global(Q + size_t(tu * g.TB + r) * g.KC + (tv * g.TB + c), v);
   }
 }
-
-constexpr int kDgStage = 2 * kJ + 4;  // wu[J], wv[J], result re, im, cell, pad
 
 // ---------------------------------------------------------------------------
 // Warp-per-item forms of degridding and gridding (the ball block and the
@@ -367,18 +365,25 @@ constexpr int kDgStage = 2 * kJ + 4;  // wu[J], wv[J], result re, im, cell, pad
 // largest first so the hardware's CTA scheduling balances the load.
 constexpr int kWItems = kThreads / 32;  // items (warps) per CTA
 
+// Row pitch (cells) of the staged patch.  A warp's lanes read cells of one
+// grid row after another; FP32 cells are 8 bytes and served per half-warp (16
+// cells), so at a pitch of 8 mod 16 the 8 cells of two neighbouring tile rows
+// fall on disjoint banks (a tile of 16 is a half-warp wide by itself).  FP64
+// cells are served per quarter-warp; two more columns spread their rows.
+template <typename T> __host__ __device__ constexpr int patch_pitch(int TB) {
+  return sizeof(T) == 4 ? 24 : TB + kJ + 2;
+}
 template <typename T> __host__ __device__ inline size_t warp_patch_elems(int TB) {
-  const size_t PW = size_t(TB + kJ);
-  return PW * (PW + 2);
+  return size_t(TB + kJ) * patch_pitch<T>(TB);
 }
 
 template <typename C>
-PD bool warp_stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu, int tv, int TB, int PW, int lane,
-                         int* err) {
+PD bool warp_stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu, int tv, int TB, uint32_t bytes,
+                         int lane, int* err) {
   if (lane == 0) {
     mbar_init(bar, 1);
     fence_barrier_init();
-    mbar_arrive_expect_tx(bar, uint32_t(PW * (PW + 2) * sizeof(C)));
+    mbar_arrive_expect_tx(bar, bytes);
     const int cw = int(sizeof(C) / 8);
     tma_load_2d(patch, map, tv * TB * cw, tu * TB, bar);
   }
@@ -387,117 +392,93 @@ PD bool warp_stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu
   return __all_sync(0xffffffffu, ok) != 0;
 }
 
+// Degridding: one lane per visibility, its kernel weights in registers, its
+// J x J cells gathered from the warp's staged patch; visibilities are sorted by
+// cell, so a warp's lanes read neighbouring cells.  Bound by the shared-memory
+// pipe: 64 cells of 8 bytes at 128 bytes a clock are 4 cycles per visibility
+// (two for pairs of lanes in one cell, which share a read).  The form with
+// four lanes per visibility staged every weight through shared memory and
+// summed by shuffles, 7.8 cycles: 141 us a launch against 84 (1024^2,
+// M = 4,194,304).
 template <typename T, typename Src>
 __global__ void __launch_bounds__(kThreads) k_degrid_w(Src src, KbPoly<T> kb, const __grid_constant__ CUtensorMap map0) {
   typedef typename cplx_t<T>::type C;
   decltype(auto) a = src.get();
   const Geometry& g = a.g;
-  const WorkItem* __restrict__ items = a.items;
   const int n_items = a.n_items;
   const Pos<T>* __restrict__ pos = a.pos;
   const int* __restrict__ perm = a.perm;
   const DegridEp<C>& dep = a.dep;
-  int* err = a.err;
   const CUtensorMap* map = Src::kTable ? a.map : &map0;
   extern __shared__ __align__(128) unsigned char sm_raw[];
   __shared__ __align__(8) uint64_t bars[kWItems];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int item = blockIdx.x * kWItems + warp;
   if (item >= n_items) return;
-  const WorkItem it = items[item];
-  const int tu = it.tile / g.ntile1d, tv = it.tile - tu * g.ntile1d;
-  const int PW = g.TB + kJ, PP = PW + 2;
+  const WorkItem it = a.items[item];
+  const int tu = it.tile / g.ntv, tv = it.tile - tu * g.ntv;
+  const int PP = patch_pitch<T>(g.TB);
   const size_t pe = warp_patch_elems<T>(g.TB);
   C* patch = reinterpret_cast<C*>(sm_raw) + warp * pe;
-  T* wst = reinterpret_cast<T*>(reinterpret_cast<C*>(sm_raw) + kWItems * pe) + warp * 32 * kDgStage;
   if (Src::kTable && lane == 0) tensormap_acquire(map);
-  if (!warp_stage_patch(patch, &bars[warp], map, tu, tv, g.TB, PW, lane, err)) return;
-  const int grp = lane >> 2, k = lane & 3;
+  int i = it.begin + lane;
+  Pos<T> p = pos[min(i, it.end - 1)];  // the first positions arrive beside the patch
+  if (!warp_stage_patch(patch, &bars[warp], map, tu, tv, g.TB, uint32_t(pe * sizeof(C)), lane, a.err)) return;
+  const bool ball = dep.mode == DG_BALL;
   Acc<T> p0, p1;
-  for (int base = it.begin; base < it.end; base += 32) {
-    const int i = base + lane;
+  for (; i - lane < it.end; i += 32) {
     const bool valid = i < it.end;
-    const int nv = min(32, it.end - base);
-    {
-      T wu[kJ], wv[kJ];
-      int cu = 0, cv = 0;
-      if (valid) {
-        T fu, fv;
-        decode(pos[i], cu, fu, cv, fv);
-        kb_eval(kb, fu, wu);
-        kb_eval(kb, fv, wv);
-      } else {
-#pragma unroll
-        for (int a = 0; a < kJ; ++a) wu[a] = wv[a] = T(0);
-      }
-      stage_store(wst + lane * kDgStage, wu, wv, T(0), T(0), cu * 256 + cv);
+    const int is = min(i, it.end - 1);
+    // the epilogue's operands and the next positions are on their way while the taps are summed
+    C z = cz<C>(), yv = cz<C>();
+    int pm = 0;
+    if (ball) {
+      z = dep.z[is];
+      yv = dep.ys[is];
+    } else if (dep.mode == DG_STORE_PERM) {
+      pm = perm[is];
     }
-    __syncwarp();
+    const Pos<T> cur = p;
+    p = pos[min(i + 32, it.end - 1)];
+    int cu, cv;
+    T fu, fv, wu[kJ], wv[kJ];
+    decode(cur, cu, fu, cv, fv);
+    kb_eval(kb, fu, wu);
+    kb_eval(kb, fv, wv);
+    const C* row = patch + cu * PP + cv;
+    C acc = cz<C>();
 #pragma unroll
-    for (int s4 = 0; s4 < 4; ++s4) {
-      const int j = s4 * 8 + grp;
-      C part = cz<C>();
-      if (j < nv) {
-        const T* sj = wst + j * kDgStage;
-        const int cell = *reinterpret_cast<const int*>(sj + 2 * kJ + 2);
-        const T wa0 = sj[2 * k], wa1 = sj[2 * k + 1];
-        T wv[kJ];
-        if constexpr (sizeof(T) == 4) {
-          const float4 w0 = *reinterpret_cast<const float4*>(sj + kJ);
-          const float4 w1 = *reinterpret_cast<const float4*>(sj + kJ + 4);
-          wv[0] = w0.x; wv[1] = w0.y; wv[2] = w0.z; wv[3] = w0.w;
-          wv[4] = w1.x; wv[5] = w1.y; wv[6] = w1.z; wv[7] = w1.w;
-        } else {
+    for (int r = 0; r < kJ; ++r) {
+      C h = cz<C>();
 #pragma unroll
-          for (int b = 0; b < kJ; ++b) wv[b] = sj[kJ + b];
-        }
-        const C* r0 = patch + ((cell >> 8) + 2 * k) * PP + (cell & 255);
-        const C* r1 = r0 + PP;
-        T hx0 = 0, hy0 = 0, hx1 = 0, hy1 = 0;
-#pragma unroll
-        for (int b = 0; b < kJ; ++b) {
-          const C g0 = r0[b], g1 = r1[b];
-          hx0 = fma(wv[b], g0.x, hx0);
-          hy0 = fma(wv[b], g0.y, hy0);
-          hx1 = fma(wv[b], g1.x, hx1);
-          hy1 = fma(wv[b], g1.y, hy1);
-        }
-        part = cmk<C>(fma(wa0, hx0, wa1 * hx1), fma(wa0, hy0, wa1 * hy1));
+      for (int b = 0; b < kJ; ++b) {
+        const C c = row[b];
+        h.x = fma(wv[b], c.x, h.x);
+        h.y = fma(wv[b], c.y, h.y);
       }
-      part.x += __shfl_xor_sync(0xffffffffu, part.x, 1);
-      part.y += __shfl_xor_sync(0xffffffffu, part.y, 1);
-      part.x += __shfl_xor_sync(0xffffffffu, part.x, 2);
-      part.y += __shfl_xor_sync(0xffffffffu, part.y, 2);
-      if (k == 0 && j < nv) {
-        T* sj = wst + j * kDgStage;
-        sj[2 * kJ] = part.x;
-        sj[2 * kJ + 1] = part.y;
-      }
+      acc.x = fma(wu[r], h.x, acc.x);
+      acc.y = fma(wu[r], h.y, acc.y);
+      row += PP;
     }
-    __syncwarp();
-    if (valid) {
-      const T* st = wst + lane * kDgStage;
-      const C acc_v = cmk<C>(st[2 * kJ], st[2 * kJ + 1]);
-      if (dep.mode == DG_STORE_PERM) {
-        dep.y[perm[i]] = acc_v;
-      } else if (dep.mode == DG_STORE_SORTED) {
-        dep.y[i] = acc_v;
-      } else {  // DG_BALL
-        const C z = dep.z[i], yv = dep.ys[i];
-        const T nu = T(dep.nu);
-        const C v = cmk<C>(fma(nu, acc_v.x, z.x), fma(nu, acc_v.y, z.y));
-        dep.z[i] = v;
-        const T dx = fma(-nu, yv.x, v.x), dy = fma(-nu, yv.y, v.y);
-        p0.add_prod(dx, dx);
-        p0.add_prod(dy, dy);
-        const T ex = acc_v.x - yv.x, ey = acc_v.y - yv.y;
-        p1.add_prod(ex, ex);
-        p1.add_prod(ey, ey);
-      }
+    if (!valid) continue;
+    if (ball) {
+      const T nu = T(dep.nu);
+      const C v = cmk<C>(fma(nu, acc.x, z.x), fma(nu, acc.y, z.y));
+      dep.z[i] = v;
+      const T dx = fma(-nu, yv.x, v.x), dy = fma(-nu, yv.y, v.y);
+      p0.add_prod(dx, dx);
+      p0.add_prod(dy, dy);
+      const T ex = acc.x - yv.x, ey = acc.y - yv.y;
+      p1.add_prod(ex, ex);
+      p1.add_prod(ey, ey);
+    } else if (dep.mode == DG_STORE_PERM) {
+      dep.y[perm_index(pm)] = perm_value(pm, acc);
+    } else {
+      dep.y[i] = acc;
     }
-    __syncwarp();
   }
-  if (dep.mode == DG_BALL) {
+  __syncwarp();
+  if (ball) {
     warp_merge(p0);
     warp_merge(p1);
     if (lane == 0) {
@@ -542,7 +523,7 @@ __global__ void __launch_bounds__(kThreads) k_grid_w(Src src, KbPoly<T> kb) {
   const int item = blockIdx.x * kWItems + warp;
   if (item >= n_items) return;
   const WorkItem it = items[item];
-  const int tu = it.tile / g.ntile1d, tv = it.tile - tu * g.ntile1d;
+  const int tu = it.tile / g.ntv, tv = it.tile - tu * g.ntv;
   const int PW = g.TB + kJ;
   // per warp: a PW x PW patch of cells (row stride PS), then the staging rows
   const int PS = grid_row_stride<T>(PW);
@@ -572,7 +553,7 @@ __global__ void __launch_bounds__(kThreads) k_grid_w(Src src, KbPoly<T> kb) {
         kb_eval(kb, fu, wu);
         kb_eval(kb, fv, wv);
         if (gpro.mode == GP_PERM) {
-          u = gpro.y[perm[i]];
+          u = perm_value(perm[i], gpro.y[perm_index(perm[i])]);
         } else if (gpro.mode == GP_SORTED) {
           u = gpro.y[i];
         } else {  // GP_BALL
@@ -634,7 +615,7 @@ __global__ void __launch_bounds__(kThreads) k_grid_w(Src src, KbPoly<T> kb) {
     const int r = e / PW, c = e - r * PW;
     const GCell<T> kc = wacc[r * PS + c];
     const C v = cmk<C>(kc.x, kc.y);
-    if (v.x != 0 || v.y != 0) atomic_add_global(Q + size_t(tu * g.TB + r) * g.KP + (tv * g.TB + c), v);
+    if (v.x != 0 || v.y != 0) atomic_add_global(Q + size_t(tu * g.TB + r) * g.KC + (tv * g.TB + c), v);
   }
 }
 
@@ -651,23 +632,36 @@ PD void grid_cell(double u, int K, int& cell, double& f) {
   if (c < 0) c += K;
   cell = int(c);
 }
+// Cell and offset of both axes, reflected into the half grid when the column
+// cell is in [K/2, K) (and fold is set); returns whether it was.
+PD bool grid_cells(const double* uv, int64_t m, int K, bool fold, int (&cell)[2], double (&f)[2]) {
+  grid_cell(uv[2 * m], K, cell[0], f[0]);
+  grid_cell(uv[2 * m + 1], K, cell[1], f[1]);
+  const bool mirror = fold && cell[1] >= K / 2;
+  if (mirror)
+    for (int a = 0; a < 2; ++a) {
+      cell[a] = K - 1 - cell[a];
+      f[a] = 1.0 - f[a];
+    }
+  return mirror;
+}
 
 // Sort key: tile id, then the cell inside the tile (row-major), so that a
 // tile's visibilities come grouped by grid cell.
 // With visibility blocks (Eq. 4) the block index leads the key, so that every
 // work item lies in one block.
 __global__ void k_bin_keys(const double* __restrict__ uv, const int* __restrict__ blocks, int64_t M, int K, int TB,
-                           int lb, int ntile1d, int tbits, uint32_t* __restrict__ keys, int* __restrict__ vals) {
+                           int lb, int ntv, int tbits, bool fold, uint32_t* __restrict__ keys,
+                           int* __restrict__ vals) {
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m >= M) return;
-  int cu, cv;
-  double fu, fv;
-  grid_cell(uv[2 * m], K, cu, fu);
-  grid_cell(uv[2 * m + 1], K, cv, fv);
-  const uint32_t tile = uint32_t((cu / TB) * ntile1d + (cv / TB));
+  int c[2];
+  double f[2];
+  const bool mirror = grid_cells(uv, m, K, fold, c, f);
+  const uint32_t tile = uint32_t((c[0] / TB) * ntv + (c[1] / TB));
   const uint32_t blk = blocks ? uint32_t(blocks[m]) : 0u;
-  keys[m] = (blk << (tbits + 2 * lb)) | (tile << (2 * lb)) | (uint32_t(cu % TB) << lb) | uint32_t(cv % TB);
-  vals[m] = int(m);
+  keys[m] = (blk << (tbits + 2 * lb)) | (tile << (2 * lb)) | (uint32_t(c[0] % TB) << lb) | uint32_t(c[1] % TB);
+  vals[m] = mirror ? ~int(m) : int(m);
 }
 
 constexpr int kSortThreads = 256;
@@ -899,15 +893,14 @@ __global__ void k_encode<float>(const double* __restrict__ uv, const int* __rest
                                 Pos<float>* __restrict__ pos) {
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= M) return;
-  const int64_t m = perm[i];
+  int cell[2];
+  double f[2];
+  grid_cells(uv, perm_index(perm[i]), K, true, cell, f);
   uint32_t e[2];
   for (int a = 0; a < 2; ++a) {
-    int cell;
-    double f;
-    grid_cell(uv[2 * m + a], K, cell, f);
-    uint32_t q = uint32_t(f * 16777216.0);
+    uint32_t q = uint32_t(f[a] * 16777216.0 + 0.5);
     if (q > 0xFFFFFFu) q = 0xFFFFFFu;
-    e[a] = (uint32_t(cell % TB) << 24) | q;
+    e[a] = (uint32_t(cell[a] % TB) << 24) | q;
   }
   Pos<float> p;
   p.u = e[0];
@@ -919,16 +912,14 @@ __global__ void k_encode<double>(const double* __restrict__ uv, const int* __res
                                  Pos<double>* __restrict__ pos) {
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= M) return;
-  const int64_t m = perm[i];
-  int cu, cv;
-  double fu, fv;
-  grid_cell(uv[2 * m], K, cu, fu);
-  grid_cell(uv[2 * m + 1], K, cv, fv);
+  int c[2];
+  double f[2];
+  grid_cells(uv, perm_index(perm[i]), K, true, c, f);
   Pos<double> p;
-  // cell + f may round up to the next integer when f is within an ulp of 1:
-  // keep the sum inside the cell
-  p.u = fmin(double(cu % TB) + fu, nextafter(double(cu % TB + 1), 0.0));
-  p.v = fmin(double(cv % TB) + fv, nextafter(double(cv % TB + 1), 0.0));
+  // cell + f may round up to the next integer when f is within an ulp of 1
+  // (and a mirrored f may be 1): keep the sum inside the cell
+  p.u = fmin(double(c[0] % TB) + f[0], nextafter(double(c[0] % TB + 1), 0.0));
+  p.v = fmin(double(c[1] % TB) + f[1], nextafter(double(c[1] % TB + 1), 0.0));
   pos[i] = p;
 }
 
@@ -941,23 +932,20 @@ __global__ void k_encode_x2(const double* __restrict__ uv, const int* __restrict
                             Pos<T>* __restrict__ pos) {
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= M) return;
-  const int64_t m = perm[i];
   int cell[2];
   double fr[2];
+  grid_cells(uv, perm_index(perm[i]), Kc, true, cell, fr);
   for (int a = 0; a < 2; ++a) {
-    int cc;
-    double fc;
-    grid_cell(uv[2 * m + a], Kc, cc, fc);
-    const double t2 = 2.0 * fc;  // exact
+    const double t2 = 2.0 * fr[a];  // exact
     const double up = t2 >= 1.0 ? 1.0 : 0.0;
-    cell[a] = (2 * cc + int(up)) % TB;
+    cell[a] = (2 * cell[a] + int(up)) % TB;
     fr[a] = t2 - up;
   }
   Pos<T> p;
   if constexpr (sizeof(T) == 4) {
     uint32_t e[2];
     for (int a = 0; a < 2; ++a) {
-      uint32_t q = uint32_t(fr[a] * 16777216.0);
+      uint32_t q = uint32_t(fr[a] * 16777216.0 + 0.5);
       if (q > 0xFFFFFFu) q = 0xFFFFFFu;
       e[a] = (uint32_t(cell[a]) << 24) | q;
     }
@@ -986,6 +974,10 @@ template cudaError_t configure_nufft<double>();
 
 cudaError_t set_wait_spins_nufft(uint32_t spins) { return set_module_wait_spins(spins); }
 
+template <typename T> int degrid_patch_pitch(int TB) { return patch_pitch<T>(TB); }
+template int degrid_patch_pitch<float>(int);
+template int degrid_patch_pitch<double>(int);
+
 size_t tile_smem_bytes(int precision_bytes, int TB, int mode) {
   if (precision_bytes == 4) {
     size_t b = tile_stage_bytes<float>();
@@ -1004,7 +996,7 @@ void launch_degrid(const Geometry& g, const CUtensorMap& map, const WorkItem* it
                    const int* perm, const KbPoly<T>& kb, const DegridEp<typename cplx_t<T>::type>& ep, int* err,
                    cudaStream_t s) {
   if (n_items <= 0) return;
-  const size_t sm = kWItems * (warp_patch_elems<T>(g.TB) * sizeof(typename cplx_t<T>::type) + 32 * kDgStage * sizeof(T));
+  const size_t sm = kWItems * warp_patch_elems<T>(g.TB) * sizeof(typename cplx_t<T>::type);
   ArgVal<DegridArgs<T>> src{DegridArgs<T>{g, nullptr, items, n_items, pos, perm, ep, err}};
   k_degrid_w<T><<<(n_items + kWItems - 1) / kWItems, kThreads, sm, s>>>(src, kb, map);
 }
@@ -1013,7 +1005,7 @@ template <typename T>
 void launch_degrid_batch(const DegridArgs<T>* tab, int count, int max_items, int max_tb, const KbPoly<T>& kb,
                          cudaStream_t s) {
   if (max_items <= 0 || count <= 0) return;
-  const size_t sm = kWItems * (warp_patch_elems<T>(max_tb) * sizeof(typename cplx_t<T>::type) + 32 * kDgStage * sizeof(T));
+  const size_t sm = kWItems * warp_patch_elems<T>(max_tb) * sizeof(typename cplx_t<T>::type);
   CUtensorMap unused;
   std::memset(&unused, 0, sizeof(unused));
   ArgTab<DegridArgs<T>> src{tab};
@@ -1057,20 +1049,76 @@ void launch_encode_x2(const double* uv, const int* perm, int64_t M, int Kc, int 
   k_encode_x2<T><<<int((M + tb - 1) / tb), tb, 0, s>>>(uv, perm, M, Kc, TB, pos);
 }
 
+// Fields of a binning key: block, tile, cell row and column inside the tile.
+struct KeyBits { int lb, tbits, bits; };
+static KeyBits key_bits(int TB, int tiles_per_block, int R) {
+  KeyBits k{0, 0, 0};
+  while ((1 << k.lb) < TB) ++k.lb;
+  while ((1 << k.tbits) < tiles_per_block) ++k.tbits;
+  int rbits = 0;
+  while ((1 << rbits) < (R > 1 ? R : 1)) ++rbits;
+  k.bits = 2 * k.lb + k.tbits + rbits;
+  return k;
+}
+
+// Stable radix sort of (key, value) pairs by the low `bits` bits; the sorted
+// values end in `vals`, the sorted keys at `keys` (which may move to `k1`).
+static cudaError_t sort_pairs(uint32_t*& keys, uint32_t* k1, int* vals, int* v1, int64_t M, int bits, int nblocks,
+                              int* hist, int* bsum, cudaStream_t s) {
+  uint32_t* kout = k1;
+  int* vin = vals;
+  int* vout = v1;
+  for (int shift = 0; shift < bits; shift += 8) {
+    k_radix_hist<<<nblocks, kSortThreads, 0, s>>>(keys, M, shift, nblocks, hist);
+    launch_scan(hist, int64_t(256) * nblocks, nullptr, bsum, s);
+    k_radix_scatter<<<nblocks, kSortThreads, 0, s>>>(keys, vin, M, shift, nblocks, hist, kout, vout);
+    std::swap(keys, kout);
+    std::swap(vin, vout);
+  }
+  if (vin != vals) return cudaMemcpyAsync(vals, vin, M * sizeof(int), cudaMemcpyDeviceToDevice, s);
+  return cudaGetLastError();
+}
+
+int sort_order_plain(const double* uv, int64_t M, const Geometry& g, int* order, cudaStream_t s, const int* blocks) {
+  const int nt = g.K / g.TB;
+  const KeyBits kb = key_bits(g.TB, nt * nt, blocks ? 64 : 1);
+  const int nblocks = int((M + kSortTile - 1) / kSortTile), tb = 256;
+  uint32_t *k0 = nullptr, *k1 = nullptr;
+  int *v1 = nullptr, *hist = nullptr, *bsum = nullptr;
+  cudaError_t e = setup_alloc(&k0, M * sizeof(uint32_t), s);
+  if (e == cudaSuccess) e = setup_alloc(&k1, M * sizeof(uint32_t), s);
+  if (e == cudaSuccess) e = setup_alloc(&v1, M * sizeof(int), s);
+  if (e == cudaSuccess) e = setup_alloc(&hist, size_t(256) * nblocks * sizeof(int), s);
+  if (e == cudaSuccess) e = setup_alloc(&bsum, 1024 * sizeof(int), s);
+  if (e == cudaSuccess) {
+    k_bin_keys<<<int((M + tb - 1) / tb), tb, 0, s>>>(uv, blocks, M, g.K, g.TB, kb.lb, nt, kb.tbits, false, k0, order);
+    uint32_t* kin = k0;
+    e = sort_pairs(kin, k1, order, v1, M, kb.bits, nblocks, hist, bsum, s);
+  }
+  for (void* t : {static_cast<void*>(k0), static_cast<void*>(k1), static_cast<void*>(v1), static_cast<void*>(hist),
+                  static_cast<void*>(bsum)})
+    if (t) cudaFreeAsync(t, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  return e == cudaSuccess ? 0 : (e == cudaErrorMemoryAllocation ? -2 : -3);
+}
+
+__global__ void k_slot_blocks(const WorkItem* __restrict__ items, const int* __restrict__ perm,
+                              int* __restrict__ blocks) {
+  const WorkItem it = items[blockIdx.x];
+  for (int i = it.begin + int(threadIdx.x); i < it.end; i += blockDim.x) blocks[perm_index(perm[i])] = it.pad;
+}
+void launch_slot_blocks(const WorkItem* items, int n_items, const int* perm, int* blocks, cudaStream_t s) {
+  if (n_items > 0) k_slot_blocks<<<n_items, 128, 0, s>>>(items, perm, blocks);
+}
+
 template <typename T>
 int build_bins(const double* uv, int64_t M, const Geometry& g, int chunk, Pos<T>* pos, int* perm,
                WorkItem** items_out, int* n_items_out, cudaStream_t s, const int* blocks, int R,
                cudaMemPool_t items_pool) {
-  const int tiles_per_block = g.ntile1d * g.ntile1d;
+  const int tiles_per_block = (g.K / g.TB) * g.ntv;
   const int ntiles = tiles_per_block * (R > 1 ? R : 1);  // bins
-  int lb = 0;
-  while ((1 << lb) < g.TB) ++lb;
-  int tbits = 0;
-  while ((1 << tbits) < tiles_per_block) ++tbits;
-  int rbits = 0;
-  while ((1 << rbits) < (R > 1 ? R : 1)) ++rbits;
-  const int bits = 2 * lb + tbits + rbits;
-  const int passes = (bits + 7) / 8;
+  const KeyBits kb = key_bits(g.TB, tiles_per_block, R);
+  const int lb = kb.lb;
   const int nblocks = int((M + kSortTile - 1) / kSortTile);
   uint32_t *k0 = nullptr, *k1 = nullptr;
   int *v1 = nullptr, *hist = nullptr, *tstart = nullptr, *tend = nullptr, *cnt = nullptr, *total = nullptr;
@@ -1094,20 +1142,10 @@ int build_bins(const double* uv, int64_t M, const Geometry& g, int chunk, Pos<T>
   fail(setup_alloc(&bsum, 1024 * sizeof(int), s));
   if (rc == 0) {
     const int tb = 256;
-    k_bin_keys<<<int((M + tb - 1) / tb), tb, 0, s>>>(uv, R > 1 ? blocks : nullptr, M, g.K, g.TB, lb, g.ntile1d,
-                                                     tbits, k0, perm);
+    k_bin_keys<<<int((M + tb - 1) / tb), tb, 0, s>>>(uv, R > 1 ? blocks : nullptr, M, g.K, g.TB, lb, g.ntv,
+                                                     kb.tbits, true, k0, perm);
     uint32_t* kin = k0;
-    uint32_t* kout = k1;
-    int* vin = perm;
-    int* vout = v1;
-    for (int p = 0; p < passes; ++p) {
-      k_radix_hist<<<nblocks, kSortThreads, 0, s>>>(kin, M, 8 * p, nblocks, hist);
-      launch_scan(hist, int64_t(256) * nblocks, nullptr, bsum, s);
-      k_radix_scatter<<<nblocks, kSortThreads, 0, s>>>(kin, vin, M, 8 * p, nblocks, hist, kout, vout);
-      std::swap(kin, kout);
-      std::swap(vin, vout);
-    }
-    if (vin != perm) fail(cudaMemcpyAsync(perm, vin, M * sizeof(int), cudaMemcpyDeviceToDevice, s));
+    fail(sort_pairs(kin, k1, perm, v1, M, kb.bits, nblocks, hist, bsum, s));
     fail(cudaMemsetAsync(tstart, 0, size_t(ntiles) * sizeof(int), s));
     fail(cudaMemsetAsync(tend, 0, size_t(ntiles) * sizeof(int), s));
     // bin index = key >> 2 lb = block << tbits | tile; with tiles_per_block a power of

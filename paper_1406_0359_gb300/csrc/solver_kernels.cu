@@ -286,7 +286,13 @@ __global__ void k_wait_selftest(int deliver) {
 
 template <typename C>
 __global__ void k_gather(const C* __restrict__ src, const int* __restrict__ perm, size_t M, C* __restrict__ dst) {
-  for (size_t i = size_t(blockIdx.x) * kT + threadIdx.x; i < M; i += size_t(gridDim.x) * kT) dst[i] = src[perm[i]];
+  for (size_t i = size_t(blockIdx.x) * kT + threadIdx.x; i < M; i += size_t(gridDim.x) * kT) dst[i] = perm_value(perm[i], src[perm_index(perm[i])]);
+}
+// The inverse: dst[perm[i]] = src[i].
+template <typename C>
+__global__ void k_scatter(const C* __restrict__ src, const int* __restrict__ perm, size_t M, C* __restrict__ dst) {
+  for (size_t i = size_t(blockIdx.x) * kT + threadIdx.x; i < M; i += size_t(gridDim.x) * kT)
+    dst[perm_index(perm[i])] = perm_value(perm[i], src[i]);
 }
 
 inline int nblk(size_t N) {
@@ -359,6 +365,9 @@ template <typename T> void launch_scale(T* v, size_t N, const double* sc, int id
 template <typename C> void launch_gather(const C* src, const int* perm, size_t M, C* dst, cudaStream_t s) {
   k_gather<C><<<nblk(M), kT, 0, s>>>(src, perm, M, dst);
 }
+template <typename C> void launch_scatter(const C* src, const int* perm, size_t M, C* dst, cudaStream_t s) {
+  k_scatter<C><<<nblk(M), kT, 0, s>>>(src, perm, M, dst);
+}
 template <typename T> void launch_check_finite(const T* v, size_t n, int* flag, cudaStream_t s) {
   k_check_finite<T><<<nblk(n), kT, 0, s>>>(v, n, flag);
 }
@@ -397,5 +406,7 @@ template void launch_fill<float2>(float2*, size_t, float2, cudaStream_t);
 template void launch_fill<double2>(double2*, size_t, double2, cudaStream_t);
 template void launch_gather<float2>(const float2*, const int*, size_t, float2*, cudaStream_t);
 template void launch_gather<double2>(const double2*, const int*, size_t, double2*, cudaStream_t);
+template void launch_scatter<float2>(const float2*, const int*, size_t, float2*, cudaStream_t);
+template void launch_scatter<double2>(const double2*, const int*, size_t, double2*, cudaStream_t);
 
 }  // namespace purify

@@ -37,6 +37,8 @@ void launch_finalize_blocks(const double* part0, const double* part1, const int*
 template <typename T> void launch_reweight(T* w, size_t N, double delta, cudaStream_t s);
 template <typename T> void launch_fill(T* v, size_t N, T val, cudaStream_t s);
 template <typename T> void launch_scale(T* v, size_t N, const double* sc, int idx, double mul, cudaStream_t s);
+// Into and out of the operator's sorted order (perm_index, perm_value).
+template <typename C> void launch_scatter(const C* src, const int* perm, size_t M, C* dst, cudaStream_t s);
 template <typename C> void launch_gather(const C* src, const int* perm, size_t M, C* dst, cudaStream_t s);
 // Batched vector steps of instances of one size (argument tables in device
 // memory; instance = blockIdx.y, one grid for all).
