@@ -439,9 +439,11 @@ template <typename T> class OpImpl : public purify_op {
     g.ntv = n / g.TB;
     g.M = M;
     levels = L;
-    // default work-item length by M (what purify_autotune usually picks:
-    // many short items for small M, fewer long ones for large M)
-    chunk = chunk_opt > 0 ? chunk_opt : (M < (int64_t(1) << 20) ? 256 : M >= (int64_t(1) << 21) ? 2048 : 1024);
+    // default work-item length by M: a warp walks an item alone, so short
+    // items spread a small M over the chip (256^2 / 131072: Phi^H 29 us at 128,
+    // 33 at 256, 50 at 1024) and end a large one together (512^2 / 4M: 110 at
+    // 256..1024, 149 at 2048; 1024^2 / 4M: 150..154 at 256..2048)
+    chunk = chunk_opt > 0 ? chunk_opt : (M < (int64_t(1) << 20) ? 128 : 512);
     if (!light) {  // a set-up operator runs only on the caller's stream
       // the ball block is the longer branch of an iteration: its kernels'
       // CTAs go first when several branches have work waiting, then the

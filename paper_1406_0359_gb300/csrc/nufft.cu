@@ -131,31 +131,6 @@ template <> PD void stage_store<double>(double* st, const double (&wu)[kJ], cons
 }
 static_assert(kStage == 2 * kJ + 4 && kJ == 8, "stage_store writes 2J + 4 values");
 
-// Gridding's staged record: {u.re, u.im, cell bits, pad}, then wu interleaved
-// as (wu[a], wu[a + 4]) pairs, then wv[0..7] -- lane (ta, tc) reads the first
-// 16 bytes, one 8-byte pair and one value per visibility.
-template <typename T> PD void stage_store_grid(T* st, const T (&wu)[kJ], const T (&wv)[kJ], T ux, T uy, int cell);
-template <> PD void stage_store_grid<float>(float* st, const float (&wu)[kJ], const float (&wv)[kJ], float ux,
-                                            float uy, int cell) {
-  float4* d = reinterpret_cast<float4*>(st);
-  d[0] = make_float4(ux, uy, __int_as_float(cell), 0.f);
-  d[1] = make_float4(wu[0], wu[4], wu[1], wu[5]);
-  d[2] = make_float4(wu[2], wu[6], wu[3], wu[7]);
-  d[3] = make_float4(wv[0], wv[1], wv[2], wv[3]);
-  d[4] = make_float4(wv[4], wv[5], wv[6], wv[7]);
-}
-template <> PD void stage_store_grid<double>(double* st, const double (&wu)[kJ], const double (&wv)[kJ], double ux,
-                                             double uy, int cell) {
-  double2* d = reinterpret_cast<double2*>(st);
-  d[0] = make_double2(ux, uy);
-  d[1] = make_double2(__hiloint2double(0, cell), 0.0);
-#pragma unroll
-  for (int a = 0; a < kJ / 2; ++a) {
-    d[2 + a] = make_double2(wu[a], wu[a + 4]);
-    d[2 + kJ / 2 + a] = make_double2(wv[2 * a], wv[2 * a + 1]);
-  }
-}
-
 template <typename T> __host__ __device__ inline size_t tile_patch_bytes(int TB) {
   const size_t PW = size_t(TB + kJ);
   return PW * (sizeof(T) == 4 ? 24 : PW + 2) * sizeof(typename cplx_t<T>::type);
@@ -363,7 +338,12 @@ __global__ void __launch_bounds__(kThreads) k_tile(Geometry g, const __grid_cons
 // patch and mbarrier (degridding) or its own accumulator patch (gridding), so
 // there are no CTA-wide barriers and no cross-warp merges; items are ordered
 // largest first so the hardware's CTA scheduling balances the load.
-constexpr int kWItems = kThreads / 32;  // items (warps) per CTA
+// Two warps per CTA: a CTA of 8 holds its shared memory and registers until its
+// longest item ends (1024^2 / 4M points: Phi 99.7 against 108.4 us, Phi^H 155
+// against 160); single-warp CTAs measured the same alone, but a batch's grid of
+// the largest instance's items per instance launches twice as many (16
+// instances: 1227 against 1215 us an iteration).
+constexpr int kWItems = 2;  // items (warps) per CTA
 
 // Row pitch (cells) of the staged patch.  A warp's lanes read cells of one
 // grid row after another; FP32 cells are 8 bytes and served per half-warp (16
@@ -401,7 +381,7 @@ PD bool warp_stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu
 // summed by shuffles, 7.8 cycles: 141 us a launch against 84 (1024^2,
 // M = 4,194,304).
 template <typename T, typename Src>
-__global__ void __launch_bounds__(kThreads) k_degrid_w(Src src, KbPoly<T> kb, const __grid_constant__ CUtensorMap map0) {
+__global__ void __launch_bounds__(32 * kWItems) k_degrid_w(Src src, KbPoly<T> kb, const __grid_constant__ CUtensorMap map0) {
   typedef typename cplx_t<T>::type C;
   decltype(auto) a = src.get();
   const Geometry& g = a.g;
@@ -488,134 +468,243 @@ __global__ void __launch_bounds__(kThreads) k_degrid_w(Src src, KbPoly<T> kb, co
   }
 }
 
-// A gridding accumulator cell (one complex value); a run sum is added into
-// it with one 8-byte (FP32) shared read-modify-write.  Rows of the per-warp
-// patch are padded so that the quarter-warps of an update (four patch rows,
-// 8 consecutive cells each) that share a half-warp fall in different banks.
+// Gridding: the warp splits its item into two contiguous slices, one per group
+// of 16 lanes; a lane of a group sums four cells (one row and column parity) of
+// its visibility's J x J footprint in registers for as long as the group's cell
+// stays the same, and adds the run to the group's own patch of plain cells in
+// shared memory (no atomics, nothing shared between groups) when it changes.
+// The patches are merged at the end, one vector atomic per two cells.  Two
+// visibilities take 4 shared-memory cycles and 8 FMAs a lane; bound by
+// instruction issue (72%) and the shared-memory pipe (60%).  One visibility at
+// a time on 32 lanes took 165 us a launch, this form 115 (1024^2, M =
+// 4,194,304, half grid); four groups of 8 lanes win where cells are full (512^2:
+// 128 against 149 us for Phi^H) but hold 16 warps an SM and lose elsewhere (187
+// against 150).
+constexpr int kGroups = 2;
+constexpr int kGrLanes = 32 / kGroups;      // lanes of a group: 8 rows x 2 column parities
+constexpr int kGrCols = 8 * kJ / kGrLanes;  // columns per lane
+constexpr int kGrRec = 2 * kJ + 4;          // staged record: wu[J], wv[J], u.re, u.im, pad
+constexpr int kGrStage = kGrLanes * kGrRec + 8;  // a group's records; the pad puts the groups on distinct banks
 template <typename T> struct __align__(2 * sizeof(T)) GCell { T x, y; };
-template <typename T> PD void cell_add(GCell<T>* cell, T vx, T vy) {
-  GCell<T> k = *cell;
-  k.x += vx;
-  k.y += vy;
-  *cell = k;
+// Row stride 2 mod 16 or 10 mod 16 (even): the 8 rows x 2 neighbouring columns
+// that a group's 16 lanes update at once (8-byte FP32 cells) fall on 16
+// distinct bank pairs; pairs of cells stay 16-byte aligned.
+__host__ __device__ constexpr int grid_row_stride(int TB) { return TB + kJ + 2; }
+template <typename T> __host__ __device__ inline size_t grid_patch_cells(int TB) {
+  return size_t(TB + kJ) * grid_row_stride(TB);
 }
-// FP32 cells are 8 bytes, and a warp's 8-byte accesses are served per
-// half-warp: its two quarter-warps (two patch rows) must fall on disjoint
-// banks, i.e. rows an odd multiple of 64 bytes apart (stride = 8 mod 16
-// cells).  FP64 cells (16 bytes) are served per quarter-warp and need none.
-template <typename T> __host__ __device__ constexpr int grid_row_stride(int pw) {
-  return (sizeof(T) == 4 && pw % 16 == 0) ? pw + 8 : pw;
+template <typename T> __host__ __device__ inline size_t grid_warp_bytes(int TB) {
+  return kGroups * (grid_patch_cells<T>(TB) * sizeof(GCell<T>) + kGrStage * sizeof(T));
+}
+
+// One lane's sums of W complex cells of one column parity, FP32 as packed pairs of
+// columns (an FMA of two by one instruction, same rounding).
+template <typename T, int W> struct RowAcc;
+template <int W> struct RowAcc<double, W> {
+  double x[W], y[W];
+  PD void zero() {
+#pragma unroll
+    for (int b = 0; b < W; ++b) x[b] = y[b] = 0.0;
+  }
+  PD void add(const double* wv, double ax, double ay) {
+#pragma unroll
+    for (int b = 0; b < W; ++b) {
+      x[b] = fma(wv[b], ax, x[b]);
+      y[b] = fma(wv[b], ay, y[b]);
+    }
+  }
+  PD void flush(GCell<double>* c) {
+#pragma unroll
+    for (int b = 0; b < W; ++b) {
+      c[2 * b].x += x[b];
+      c[2 * b].y += y[b];
+    }
+  }
+};
+template <int W> struct RowAcc<float, W> {
+  unsigned long long x[W / 2], y[W / 2];
+  PD void zero() {
+#pragma unroll
+    for (int b = 0; b < W / 2; ++b) x[b] = y[b] = 0ull;
+  }
+  static PD void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+  }
+  PD void add(const float* wv, float ax, float ay) {
+    unsigned long long px, py, w[W / 2];
+    asm("mov.b64 %0, {%1, %1};" : "=l"(px) : "f"(ax));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(py) : "f"(ay));
+    if constexpr (W == 2) {
+      w[0] = *reinterpret_cast<const unsigned long long*>(wv);
+    } else {
+#pragma unroll
+      for (int b = 0; b < W / 4; ++b) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(wv + 4 * b);
+        w[2 * b] = v.x;
+        w[2 * b + 1] = v.y;
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < W / 2; ++b) {
+      fma2(x[b], w[b], px);
+      fma2(y[b], w[b], py);
+    }
+  }
+  PD void flush(GCell<float>* c) {
+    GCell<float> k[W];
+#pragma unroll
+    for (int b = 0; b < W; ++b) k[b] = c[2 * b];
+#pragma unroll
+    for (int b = 0; b < W / 2; ++b) {
+      float x0, x1, y0, y1;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x[b]));
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(y0), "=f"(y1) : "l"(y[b]));
+      k[2 * b].x += x0;
+      k[2 * b].y += y0;
+      k[2 * b + 1].x += x1;
+      k[2 * b + 1].y += y1;
+    }
+#pragma unroll
+    for (int b = 0; b < W; ++b) c[2 * b] = k[b];
+  }
+};
+
+PD void cell_pair(float2 (&c)[2], const GCell<float>* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  c[0] = make_float2(v.x, v.y);
+  c[1] = make_float2(v.z, v.w);
+}
+PD void cell_pair(double2 (&c)[2], const GCell<double>* p) {
+  c[0] = make_double2(p[0].x, p[0].y);
+  c[1] = make_double2(p[1].x, p[1].y);
+}
+// Two neighbouring merged cells into the grid (16-byte aligned for FP32).
+PD void atomic_add_pair(float2* p, float2 a, float2 b) {
+  atomicAdd(reinterpret_cast<float4*>(p), make_float4(a.x, a.y, b.x, b.y));
+}
+PD void atomic_add_pair(double2* p, double2 a, double2 b) {
+  atomic_add_global(p, a);
+  atomic_add_global(p + 1, b);
 }
 
 template <typename T, typename Src>
-__global__ void __launch_bounds__(kThreads) k_grid_w(Src src, KbPoly<T> kb) {
+__global__ void __launch_bounds__(32 * kWItems) k_grid_w(Src src, KbPoly<T> kb) {
   typedef typename cplx_t<T>::type C;
   decltype(auto) a = src.get();
   const Geometry& g = a.g;
-  const WorkItem* __restrict__ items = a.items;
   const int n_items = a.n_items;
   const Pos<T>* __restrict__ pos = a.pos;
   const int* __restrict__ perm = a.perm;
   const GridPro<C>& gpro = a.gpro;
-  C* __restrict__ Q = a.Q;
   extern __shared__ __align__(128) unsigned char sm_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int item = blockIdx.x * kWItems + warp;
   if (item >= n_items) return;
-  const WorkItem it = items[item];
+  const WorkItem it = a.items[item];
   const int tu = it.tile / g.ntv, tv = it.tile - tu * g.ntv;
-  const int PW = g.TB + kJ;
-  // per warp: a PW x PW patch of cells (row stride PS), then the staging rows
-  const int PS = grid_row_stride<T>(PW);
-  GCell<T>* wacc = reinterpret_cast<GCell<T>*>(sm_raw) + warp * PW * PS;
-  T* wst = reinterpret_cast<T*>(reinterpret_cast<GCell<T>*>(sm_raw) + kWItems * PW * PS) + warp * 32 * kStage;
-  for (int e = lane; e < PW * PS; e += 32) wacc[e] = GCell<T>{T(0), T(0)};
-  __syncwarp();
+  const int PW = g.TB + kJ, PS = grid_row_stride(g.TB);
+  const int cells = int(grid_patch_cells<T>(g.TB));
+  unsigned char* wbase = sm_raw + warp * grid_warp_bytes<T>(g.TB);
+  GCell<T>* patches = reinterpret_cast<GCell<T>*>(wbase);
+  T* stage = reinterpret_cast<T*>(patches + kGroups * cells);
+  const int grp = lane / kGrLanes, q = lane % kGrLanes;
+  const int r = q % kJ, h = q / kJ;  // the lane's footprint row and column parity
+  // this group's slice; the first positions (and permutation) travel while the patches are zeroed
+  const int cnt = it.end - it.begin, per = (cnt + kGroups - 1) / kGroups;
+  const int lo = it.begin + min(cnt, grp * per), hi = it.begin + min(cnt, (grp + 1) * per);
+  int i = lo + q;
+  Pos<T> p = pos[min(i, it.end - 1)];
+  int pm = gpro.mode == GP_PERM ? perm[min(i, it.end - 1)] : 0;
+  {
+    uint4* zp = reinterpret_cast<uint4*>(patches);  // cells are even in number
+    const int nz = kGroups * cells * int(sizeof(GCell<T>)) / 16;
+    for (int e = lane; e < nz; e += 32) zp[e] = make_uint4(0, 0, 0, 0);
+  }
   T scale = 0;
   if (gpro.mode == GP_BALL) scale = T(gpro.block_scale ? gpro.block_scale[it.pad] : gpro.scalars[gpro.scale_idx]);
-  // lane (ta, tc) accumulates footprint cells (ta, tc) and (ta + 4, tc), so
-  // each quarter-warp updates 8 consecutive cells of one patch row.
-  const int ta = lane >> 3, tc = lane & 7;
-  const int lo = ta * PS + tc;  // the lane's first cell relative to a footprint's corner
-  int scell = -1;               // the current run's cell, as its footprint corner's offset in the patch
-  C s0 = cz<C>(), s1 = cz<C>();
-  for (int base = it.begin; base < it.end; base += 32) {
-    const int i = base + lane;
-    const bool valid = i < it.end;
-    const int nv = min(32, it.end - base);
+  GCell<T>* mine = patches + grp * cells + r * PS + h;
+  T* gst = stage + grp * kGrStage;
+  int run = -1, last = -1;  // the current run's cell; the slice's last staged cell
+  RowAcc<T, kGrCols> acc;
+  acc.zero();
+  for (int b = 0; b < per; b += kGrLanes, i += kGrLanes) {
+    const bool valid = i < hi;
+    const int is = min(i, it.end - 1);
+    C u = cz<C>(), yv = cz<C>();
+    if (gpro.mode == GP_PERM) {
+      u = perm_value(pm, gpro.y[perm_index(pm)]);
+    } else if (gpro.mode == GP_SORTED) {
+      u = gpro.y[is];
+    } else {
+      u = gpro.z[is];
+      yv = gpro.ys[is];
+    }
+    const Pos<T> cur = p;
+    p = pos[min(i + kGrLanes, it.end - 1)];
+    if (gpro.mode == GP_PERM) pm = perm[min(i + kGrLanes, it.end - 1)];
+    int cu, cv;
+    T fu, fv, wu[kJ], wv[kJ];
+    decode(cur, cu, fu, cv, fv);
+    kb_eval(kb, fu, wu);
+    kb_eval(kb, fv, wv);
+    if (gpro.mode == GP_BALL) {  // v = z, c = nu y: project, keep the dual, grid 2r - v
+      const C v = u;
+      const T nu = T(gpro.nu);
+      const T cx = nu * yv.x, cy = nu * yv.y;
+      const T rx = fma(v.x - cx, scale, cx), ry = fma(v.y - cy, scale, cy);
+      if (valid) gpro.z[i] = cmk<C>(v.x - rx, v.y - ry);
+      u = cmk<C>(T(2) * rx - v.x, T(2) * ry - v.y);
+    }
+    if (!valid) u = cz<C>();  // adds nothing, changes no cell
+    int cell = cu * PS + cv;
+    int before = __shfl_up_sync(0xffffffffu, cell, 1, kGrLanes);
+    if (q == 0) before = last;
+    const unsigned changes = __ballot_sync(0xffffffffu, valid && cell != before);
+    last = __shfl_sync(0xffffffffu, cell, kGrLanes - 1, kGrLanes);
+    __syncwarp();  // the previous batch's records are read
     {
-      T wu[kJ], wv[kJ];
-      int cu = 0, cv = 0;
-      C u = cz<C>();
-      if (valid) {
-        T fu, fv;
-        decode(pos[i], cu, fu, cv, fv);
-        kb_eval(kb, fu, wu);
-        kb_eval(kb, fv, wv);
-        if (gpro.mode == GP_PERM) {
-          u = perm_value(perm[i], gpro.y[perm_index(perm[i])]);
-        } else if (gpro.mode == GP_SORTED) {
-          u = gpro.y[i];
-        } else {  // GP_BALL
-          const C v = gpro.z[i], yv = gpro.ys[i];
-          const T nu = T(gpro.nu);
-          const T cx = nu * yv.x, cy = nu * yv.y;
-          const T rx = fma(v.x - cx, scale, cx), ry = fma(v.y - cy, scale, cy);
-          gpro.z[i] = cmk<C>(v.x - rx, v.y - ry);
-          u = cmk<C>(T(2) * rx - v.x, T(2) * ry - v.y);
-        }
-      } else {
-#pragma unroll
-        for (int a = 0; a < kJ; ++a) wu[a] = wv[a] = T(0);
-      }
-      stage_store_grid(wst + lane * kStage, wu, wv, u.x, u.y, cu * PS + cv);
+      T* st = gst + q * kGrRec;
+      const T wo[kJ] = {wv[0], wv[2], wv[4], wv[6], wv[1], wv[3], wv[5], wv[7]};
+      stage_store(st, wu, wo, u.x, u.y, 0);
     }
     __syncwarp();
-    for (int j = 0; j < nv; ++j) {
-      const T* sj = wst + j * kStage;
-      T ux, uy;
-      int cell;
-      if constexpr (sizeof(T) == 4) {
-        const float4 h = *reinterpret_cast<const float4*>(sj);
-        ux = h.x;
-        uy = h.y;
-        cell = __float_as_int(h.z);
-      } else {
-        ux = sj[0];
-        uy = sj[1];
-        cell = *reinterpret_cast<const int*>(sj + 2);
-      }
-      if (cell != scell) {  // warp-uniform
-        if (scell >= 0) {
-          const int o = scell + lo;
-          cell_add(wacc + o, s0.x, s0.y);
-          cell_add(wacc + o + 4 * PS, s1.x, s1.y);
-          s0 = s1 = cz<C>();
+    const int nj = min(kGrLanes, per - b);
+    constexpr unsigned kFirst = kGroups == 4 ? 0x01010101u : (kGroups == 2 ? 0x00010001u : 1u);
+#pragma unroll 4
+    for (int j = 0; j < nj; ++j) {
+      if (changes & (kFirst << j)) {
+        const int next = __shfl_sync(0xffffffffu, cell, j, kGrLanes);
+        if ((changes >> (grp * kGrLanes + j)) & 1u) {
+          if (run >= 0) {
+            acc.flush(mine + run);
+            acc.zero();
+          }
+          run = next;
         }
-        scell = cell;
       }
-      typedef typename Pair2<T>::type T2;
-      const T wb = sj[4 + kJ + tc];
-      const T2 wa = *reinterpret_cast<const T2*>(sj + 4 + 2 * ta);  // (wu[ta], wu[ta + 4])
-      const T a0 = wa.x * wb, a1 = wa.y * wb;
-      s0.x = fma(a0, ux, s0.x);
-      s0.y = fma(a0, uy, s0.y);
-      s1.x = fma(a1, ux, s1.x);
-      s1.y = fma(a1, uy, s1.y);
+      const T* rec = gst + j * kGrRec;
+      const T w = rec[r];
+      acc.add(rec + kJ + h * kGrCols, w * rec[2 * kJ], w * rec[2 * kJ + 1]);
     }
-    __syncwarp();
   }
-  if (scell >= 0) {
-    const int o = scell + lo;
-    cell_add(wacc + o, s0.x, s0.y);
-    cell_add(wacc + o + 4 * PS, s1.x, s1.y);
-  }
+  if (run >= 0) acc.flush(mine + run);
   __syncwarp();
-  for (int e = lane; e < PW * PW; e += 32) {
-    const int r = e / PW, c = e - r * PW;
-    const GCell<T> kc = wacc[r * PS + c];
-    const C v = cmk<C>(kc.x, kc.y);
-    if (v.x != 0 || v.y != 0) atomic_add_global(Q + size_t(tu * g.TB + r) * g.KC + (tv * g.TB + c), v);
+  // pairs of cells, 8 (tiles of 8) or 12 of 16 (tiles of 16) lanes to a row
+  const int ls = g.TB == 8 ? 3 : 4, pc = 2 * (lane & ((1 << ls) - 1));
+  if (pc < PW) {
+    C* dst = a.Q + size_t(tu * g.TB) * g.KC + (tv * g.TB + pc);
+    for (int pr = lane >> ls; pr < PW; pr += 32 >> ls) {
+      const GCell<T>* k = patches + pr * PS + pc;
+      C v[2] = {cz<C>(), cz<C>()};
+#pragma unroll
+      for (int z = 0; z < kGroups; ++z) {
+        C c[2];
+        cell_pair(c, k + z * cells);
+        v[0] = cadd(v[0], c[0]);
+        v[1] = cadd(v[1], c[1]);
+      }
+      if (v[0].x != 0 || v[0].y != 0 || v[1].x != 0 || v[1].y != 0) atomic_add_pair(dst + size_t(pr) * g.KC, v[0], v[1]);
+    }
   }
 }
 
@@ -998,7 +1087,7 @@ void launch_degrid(const Geometry& g, const CUtensorMap& map, const WorkItem* it
   if (n_items <= 0) return;
   const size_t sm = kWItems * warp_patch_elems<T>(g.TB) * sizeof(typename cplx_t<T>::type);
   ArgVal<DegridArgs<T>> src{DegridArgs<T>{g, nullptr, items, n_items, pos, perm, ep, err}};
-  k_degrid_w<T><<<(n_items + kWItems - 1) / kWItems, kThreads, sm, s>>>(src, kb, map);
+  k_degrid_w<T><<<(n_items + kWItems - 1) / kWItems, 32 * kWItems, sm, s>>>(src, kb, map);
 }
 
 template <typename T>
@@ -1009,7 +1098,7 @@ void launch_degrid_batch(const DegridArgs<T>* tab, int count, int max_items, int
   CUtensorMap unused;
   std::memset(&unused, 0, sizeof(unused));
   ArgTab<DegridArgs<T>> src{tab};
-  k_degrid_w<T><<<dim3((max_items + kWItems - 1) / kWItems, count), kThreads, sm, s>>>(src, kb, unused);
+  k_degrid_w<T><<<dim3((max_items + kWItems - 1) / kWItems, count), 32 * kWItems, sm, s>>>(src, kb, unused);
 }
 
 template <typename T>
@@ -1017,20 +1106,17 @@ void launch_grid(const Geometry& g, const WorkItem* items, int n_items, const Po
                  const KbPoly<T>& kb, const GridPro<typename cplx_t<T>::type>& pro, typename cplx_t<T>::type* Q,
                  cudaStream_t s) {
   if (n_items <= 0) return;
-  const size_t PW = size_t(g.TB + kJ);
-  const size_t sm = kWItems * (PW * size_t(grid_row_stride<T>(int(PW))) * sizeof(GCell<T>) + 32 * kStage * sizeof(T));
   ArgVal<GridArgs<T>> src{GridArgs<T>{g, items, n_items, pos, perm, pro, Q}};
-  k_grid_w<T><<<(n_items + kWItems - 1) / kWItems, kThreads, sm, s>>>(src, kb);
+  k_grid_w<T><<<(n_items + kWItems - 1) / kWItems, 32 * kWItems, kWItems * grid_warp_bytes<T>(g.TB), s>>>(src, kb);
 }
 
 template <typename T>
 void launch_grid_batch(const GridArgs<T>* tab, int count, int max_items, int max_tb, const KbPoly<T>& kb,
                        cudaStream_t s) {
   if (max_items <= 0 || count <= 0) return;
-  const size_t PW = size_t(max_tb + kJ);
-  const size_t sm = kWItems * (PW * size_t(grid_row_stride<T>(int(PW))) * sizeof(GCell<T>) + 32 * kStage * sizeof(T));
   ArgTab<GridArgs<T>> src{tab};
-  k_grid_w<T><<<dim3((max_items + kWItems - 1) / kWItems, count), kThreads, sm, s>>>(src, kb);
+  k_grid_w<T><<<dim3((max_items + kWItems - 1) / kWItems, count), 32 * kWItems,
+                kWItems * grid_warp_bytes<T>(max_tb), s>>>(src, kb);
 }
 
 template <typename T>
