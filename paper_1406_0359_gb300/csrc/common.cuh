@@ -226,6 +226,27 @@ __device__ __forceinline__ bool last_block_done_t0(unsigned int* ticket, unsigne
   return last;
 }
 
+// Programmatic dependent launch: a kernel lets the next one on its stream be
+// scheduled at once (pdl_trigger) and, before it touches anything an earlier
+// kernel wrote or still reads, waits for all earlier kernels to have completed
+// (pdl_wait).  Both do nothing in a launch without the attribute.
+PD void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+PD void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename K, typename... A>
+inline cudaError_t launch_pdl(K kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Kernel arguments: by value for one operator (ArgVal, kernel parameter
 // space), or from a device table for a batch of independent instances of the
 // same size (ArgTab: instance blockIdx.y, every instance the same grid).

@@ -530,7 +530,6 @@ template <int U, int V, typename T>
 PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al, T (&va)[U][V], T (&vb)[U][V]) {
   if (pro.mode == PRO_CG_STEP) {
     // x += alpha p, r -= alpha Ap, p = r + beta p (alpha, beta of the previous step)
-    const T alpha = T(pro.scalars[S_ALPHA]), beta = T(pro.scalars[S_BETA]);
     T xv[2 * U][V], rv[2 * U][V], pv[2 * U][V], av[2 * U][V];
 #pragma unroll
     for (int u = 0; u < 2 * U; ++u) {
@@ -538,8 +537,14 @@ PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al
       vload(xv[u], pro.xu + i, true);
       vload(rv[u], pro.r + i, true);
       vload(pv[u], pro.p + i, true);
-      vload(av[u], pro.ap + i, true);
     }
+    // x, r and p come from the previous step's forward pass, which had
+    // completed before its column pass let this chain go on; A p and the
+    // scalars from the pass just before
+    pdl_wait();
+    const T alpha = T(pro.scalars[S_ALPHA]), beta = T(pro.scalars[S_BETA]);
+#pragma unroll
+    for (int u = 0; u < 2 * U; ++u) vload(av[u], pro.ap + ia[u >> 1] + size_t(u & 1) * n, true);
 #pragma unroll
     for (int u = 0; u < 2 * U; ++u) {
       const size_t i = ia[u >> 1] + size_t(u & 1) * n;
@@ -558,6 +563,7 @@ PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al
     }
   } else if (pro.mode == PRO_CG_START) {
     // r = b - A x_hat, p = r (b in pro.x, A x_hat in pro.ap)
+    pdl_wait();
     T bv[2 * U][V], av[2 * U][V];
 #pragma unroll
     for (int u = 0; u < 2 * U; ++u) {
@@ -579,6 +585,7 @@ PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al
       vstore(pro.p + i, rn, true);
     }
   } else {
+    pdl_wait();
     const T scl = pro.mode == PRO_SCALE ? T(pro.scalars[pro.idx]) : T(1);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -775,6 +782,7 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
 #pragma unroll
   for (int m = 0; m < E; ++m) s[t + m * TT] = v[m];
   __syncthreads();
+  pdl_trigger();
   // separate the pairs: column c = 2m + odd from elements m and -m of its half
   constexpr int PC = sizeof(T) == 4 ? 2 : 1;  // pairs per 32-byte store
   static_assert(H::PAIRS % PC == 0, "whole sectors");
@@ -819,6 +827,7 @@ __global__ void __launch_bounds__(ColHalf<T, LOGN>::COL_THREADS, ColHalf<T, LOGN
   const T* __restrict__ khat = a.khat;
   const C* __restrict__ tw = a.tw;
   extern __shared__ __align__(16) unsigned char sm_raw[];
+  pdl_wait();
   C* bufs = reinterpret_cast<C*>(sm_raw);
   const int half = threadIdx.x / TT, t = threadIdx.x - half * TT;
   const int col = int(blockIdx.x) * H::COLS + (half >> 1), odd = half & 1;
@@ -856,6 +865,7 @@ __global__ void __launch_bounds__(ColHalf<T, LOGN>::COL_THREADS, ColHalf<T, LOGN
   }
   half_fft<H, 1>(v, t, s, half, a.tws);
   if (odd) half_omega<H, 1>(v, t, tw);
+  pdl_trigger();
   half_join<H>(v, t, odd, bufs, half, Bc);
 }
 
@@ -975,6 +985,9 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
   T* ops = reinterpret_cast<T*>(sm_raw + align16(size_t(H::PAIRS) * 2 * H::BUF * sizeof(C)));
   const T* opd[2] = {nullptr, nullptr};
   const int nop = ep_staged(ep, opd);
+  // a CG step's operands p and r come from its forward pass, complete before
+  // the column pass let this one start; other modes' may be the last kernel's
+  if (ep.mode != EP_CG_AP) pdl_wait();
   if (nop > 0 && threadIdx.x == 0) {
     mbar_init(&bar, 1);
     fence_barrier_init();
@@ -984,6 +997,7 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
       for (int k = 0; k < nop; ++k)
         bulk_load(ops + (size_t(q) * 2 + k) * 2 * n, opd[k] + size_t(r0 + 2 * q) * n, pair_bytes, &bar);
   }
+  if (ep.mode == EP_CG_AP) pdl_wait();
   // the halves' spectra: column c = 2m + odd gives elements m and -m of its half
   constexpr int PC = sizeof(T) == 4 ? 2 : 1;
   constexpr int LT = n * (H::PAIRS / PC) / NT, LU = LT % 4 == 0 ? 4 : (LT % 2 == 0 ? 2 : 1);  // LU loads in flight
@@ -1027,6 +1041,7 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
   bool ok = true;
   if (nop > 0) ok = mbar_wait_bounded(&bar, 0, ep.err);
   __syncthreads();
+  pdl_trigger();
   EpAcc<T> part;
   if (ok) part = row_ep_all<LOGN>(ep, bufs, ops, a.deapod, r0);
   row_ep_finish(ep, part, red, int(blockIdx.x), a.nblocks);
@@ -1381,14 +1396,14 @@ template void half_twiddles<float>(int, std::vector<float2>&, size_t*);
 template void half_twiddles<double>(int, std::vector<double2>&, size_t*);
 template <typename T> void launch_row_fwd_h(const RowFwdArgs<T>& a, cudaStream_t s) {
   ArgVal<RowFwdArgs<T>> src{a};
-  PURIFY_LOGN_SWITCH(a.g.K, (k_row_fwd_h<T, L - 1><<<HalfShape<T, L - 1>::row_ctas, RowHalf<T, L - 1>::ROW_THREADS,
-                                                     HalfShape<T, L - 1>::fwd_smem(), s>>>(src)));
+  PURIFY_LOGN_SWITCH(a.g.K, (launch_pdl(k_row_fwd_h<T, L - 1, ArgVal<RowFwdArgs<T>>>, HalfShape<T, L - 1>::row_ctas,
+                                           RowHalf<T, L - 1>::ROW_THREADS, HalfShape<T, L - 1>::fwd_smem(), s, src)));
 }
 
 template <typename T> void launch_col_conv_h(const ColConvArgs<T>& a, cudaStream_t s) {
   ArgVal<ColConvArgs<T>> src{a};
-  PURIFY_LOGN_SWITCH(a.g.K, (k_col_conv_h<T, L - 1><<<HalfShape<T, L - 1>::col_ctas, ColHalf<T, L - 1>::COL_THREADS,
-                                                      HalfShape<T, L - 1>::conv_smem(), s>>>(src)));
+  PURIFY_LOGN_SWITCH(a.g.K, (launch_pdl(k_col_conv_h<T, L - 1, ArgVal<ColConvArgs<T>>>, HalfShape<T, L - 1>::col_ctas,
+                                           ColHalf<T, L - 1>::COL_THREADS, HalfShape<T, L - 1>::conv_smem(), s, src)));
 }
 
 template <typename T> void launch_col_fwd_h(const ColFwdArgs<T>& a, cudaStream_t s) {
@@ -1406,8 +1421,9 @@ template <typename T> void launch_col_inv_h(const ColInvArgs<T>& a, cudaStream_t
 template <typename T> void launch_row_inv_h(const RowInvArgs<T>& a, cudaStream_t s) {
   ArgVal<RowInvArgs<T>> src{a};
   const bool operands = a.ep.mode != EP_STORE && a.ep.mode != EP_POWER;
-  PURIFY_LOGN_SWITCH(a.g.K, (k_row_inv_h<T, L - 1><<<HalfShape<T, L - 1>::row_ctas, RowHalf<T, L - 1>::ROW_THREADS,
-                                                     HalfShape<T, L - 1>::inv_smem(operands), s>>>(src)));
+  PURIFY_LOGN_SWITCH(a.g.K, (launch_pdl(k_row_inv_h<T, L - 1, ArgVal<RowInvArgs<T>>>, HalfShape<T, L - 1>::row_ctas,
+                                           RowHalf<T, L - 1>::ROW_THREADS, HalfShape<T, L - 1>::inv_smem(operands), s,
+                                           src)));
 }
 
 // Batched passes: `count` instances of one grid side (g gives the shared
