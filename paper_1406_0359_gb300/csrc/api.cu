@@ -655,13 +655,29 @@ template <typename T> class OpImpl : public purify_op {
     pro.x = x;
     return pro;
   }
-  // Re(Phi^H Phi) up to the row epilogue: forward passes, gram, inverse column pass.
+  // Re(Phi^H Phi) up to the row epilogue: forward passes, degridding into the
+  // sorted buffer gram_y and gridding from it, inverse column pass.  (One kernel
+  // doing both, a CTA of 256 threads per work item, took 455 us at 2048^2 / 1.5M
+  // points, where an item holds some 20 visibilities; the two warp-per-item
+  // kernels take 170 together.)
   void gram_front(const RowPro<T>& pro, cudaStream_t s) {
     fwd_grid(pro, s);
     zero_q(s);
-    PROF(KK_GRAM, s, launch_gram<T>(g, tmap, items, n_items, pos, kb, gridQ, err, s));
+    DegridEp<C> dep{};
+    dep.mode = DG_STORE_SORTED;
+    dep.y = gram_y;
+    GridPro<C> gp{};
+    gp.mode = GP_SORTED;
+    gp.y = gram_y;
+    PROF(KK_GRAM, s, {
+      launch_degrid<T>(g, tmap, items, n_items, pos, perm, kb, dep, err, s);
+      launch_grid<T>(g, items, n_items, pos, perm, kb, gp, gridQ, s);
+    });
     col_inv(s);
   }
+  // The NUFFT form's visibilities, allocated on its first use.
+  int ensure_gram() { return gram_y ? PURIFY_OK : alloc(&gram_y, size_t(g.M)); }
+  C* gram_y = nullptr;
   int row_ep(const RowEp<T>& ep, cudaStream_t s) {
     const RowInvArgs<T> a = row_inv_args(gridA, deapod, ep);
     if (rec) record(R_RI, s).ri = a;
@@ -756,10 +772,8 @@ template <typename T> class OpImpl : public purify_op {
 
   int gram(const void* x, void* out, int mode, cudaStream_t s) override {
     if (mode != 0 && mode != 1) return PURIFY_ERR_INVALID;
-    if (mode == 1) {
-      const int rc = ensure_toeplitz(s);
-      if (rc) return rc;
-    }
+    const int rc = mode == 1 ? ensure_toeplitz(s) : ensure_gram();
+    if (rc) return rc;
     toep = mode == 1;
     normal_front(plain(static_cast<const T*>(x)), s);
     RowEp<T> ep{};
@@ -1158,7 +1172,7 @@ template <typename T> class OpImpl : public purify_op {
       if (!(e > 0)) return PURIFY_ERR_INVALID;
     CK(cudaMemcpyAsync(eps_dev, run.eps_b.data(), nblocks * sizeof(double), cudaMemcpyHostToDevice, s));
     const int gmode = P->gram < 0 ? (g.n <= 1024 ? 1 : 0) : P->gram;
-    if (gmode == 1 && (rc = ensure_toeplitz(s))) return rc;
+    if ((rc = gmode == 1 ? ensure_toeplitz(s) : ensure_gram())) return rc;
     toep = gmode == 1;
     launch_gather<C>(static_cast<const C*>(y), perm, M, ys, s);
     launch_check_finite<T>(reinterpret_cast<const T*>(ys), 2 * M, err + 1, s);

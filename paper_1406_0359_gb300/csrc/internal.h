@@ -285,10 +285,6 @@ void launch_degrid_batch(const DegridArgs<T>* tab, int count, int max_items, int
 template <typename T>
 void launch_grid_batch(const GridArgs<T>* tab, int count, int max_items, int max_tb, const KbPoly<T>& kb,
                        cudaStream_t s);
-template <typename T>
-void launch_gram(const Geometry& g, const CUtensorMap& map, const WorkItem* items, int n_items, const Pos<T>* pos,
-                 const KbPoly<T>& kb, typename cplx_t<T>::type* Q, int* err, cudaStream_t s);
-
 // Stream-ordered memory for set-up temporaries (binning scratch, the PSF
 // operator and its buffers): one pool per device that keeps up to
 // kSetupPoolKeep bytes of released memory mapped, so that repeated operator

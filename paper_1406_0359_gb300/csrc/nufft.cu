@@ -1,19 +1,15 @@
 // Kaiser-Bessel interpolation G of Phi = G F Z S (Section 4) and its adjoint
 // G^H, over uv-sorted visibility tiles.
 //
-// Visibilities are binned once per operator into TB x TB tiles of the K x K
-// oversampled grid (stable LSD radix sort on the tile id) and cut into work
-// items of at most `chunk` visibilities.  One CTA runs one work item:
+// Visibilities are binned once per operator into TB x TB tiles of the half
+// oversampled grid (stable LSD radix sort on the tile id and cell) and cut into
+// work items of at most `chunk` visibilities; a warp owns an item:
 //   degrid: the tile's (TB+J)^2 grid patch is staged in shared memory by one
-//           TMA tile load (the grid carries a periodic J-wide halo, so the
-//           patch is contiguous); every thread then gathers its visibilities'
-//           J x J taps from shared memory.
-//   grid:   every thread scatters its visibilities' J x J taps into a
-//           shared-memory patch accumulator with shared atomics; the patch is
-//           flushed to the padded global grid with one vector atomic per
-//           non-zero cell.
-//   gram:   both at once for the CG operator Phi^H Phi: y_m is formed from the
-//           staged patch and scattered straight back with the same weights.
+//           TMA tile load (the grid carries a J-wide halo, so the patch is
+//           contiguous); every lane gathers its visibility's J x J taps.
+//   grid:   groups of lanes sum runs of visibilities of one cell in registers,
+//           then in patches in shared memory, flushed to the padded global grid
+//           with vector atomics.
 // Kernel weights come from a per-tap polynomial in the fractional offset
 // (Chebyshev fit of the Kaiser-Bessel kernel, computed on the host).
 #include <cstdio>
@@ -28,8 +24,6 @@
 namespace purify {
 
 namespace {
-
-constexpr int kThreads = 256;
 
 PD void decode(const Pos<float>& p, int& cu, float& fu, int& cv, float& fv) {
   const float sc = 1.0f / 16777216.0f;
@@ -74,52 +68,19 @@ template <> PD void atomic_add_global<double2>(double2* p, double2 v) {
   atomicAdd(&p->y, v.y);
 }
 
-// Stage the work item's grid patch by TMA; false (for every thread) when the
-// bounded wait gave up in any thread.
-// Staged patch: PW = TB + J rows of PP = PW + 2 grid values (the wider pitch
-// spreads consecutive patch rows over distinct shared banks; the two extra
-// columns are read past the grid's edge on the last tile column, where the
-// tensor copy fills zeros, and never used).
-template <typename C>
-PD bool stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu, int tv, int TB, int PW, int PP, int* err) {
-  if (threadIdx.x == 0) {
-    mbar_init(bar, 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    mbar_arrive_expect_tx(bar, uint32_t(PW * PP * sizeof(C)));
-    const int cw = int(sizeof(C) / 8);
-    tma_load_2d(patch, map, tv * TB * cw, tu * TB, bar);
-  }
-  const bool ok = mbar_wait_bounded(bar, 0, err);
-  return __syncthreads_and(ok) != 0;
-}
-
-enum TileMode : int { TM_DEGRID = 0, TM_GRID = 1, TM_GRAM = 2 };
-constexpr int kWarps = kThreads / 32;
-constexpr int kStage = 2 * kJ + 4;  // wu[J], wv[J], u.re, u.im, packed cell (int bits), pad
-
-template <typename T> struct Pair2;
-template <> struct Pair2<float> { typedef float2 type; };
-template <> struct Pair2<double> { typedef double2 type; };
-
-// One lane's staged visibility record (kStage values: wu[J], wv[J], e0, e1,
-// the packed cell as int bits, pad) written as 16-byte vectors: at the 80-byte
-// (FP32) lane stride each quarter-warp's vector stores hit distinct bank
-// groups, where scalar stores at that stride collide four ways.
-template <typename T> PD void stage_store(T* st, const T (&wu)[kJ], const T (&wv)[kJ], T e0, T e1, int cell);
-template <> PD void stage_store<float>(float* st, const float (&wu)[kJ], const float (&wv)[kJ], float e0, float e1,
-                                       int cell) {
+// One lane's staged visibility record (kGrRec values)
+// written as 16-byte vectors: at the 80-byte (FP32) lane stride each
+// quarter-warp's vector stores hit distinct bank groups, where scalar stores at
+// that stride collide four ways.
+PD void stage_store(float* st, const float (&wu)[kJ], const float (&wv)[kJ], float e0, float e1) {
   float4* d = reinterpret_cast<float4*>(st);
   d[0] = make_float4(wu[0], wu[1], wu[2], wu[3]);
   d[1] = make_float4(wu[4], wu[5], wu[6], wu[7]);
   d[2] = make_float4(wv[0], wv[1], wv[2], wv[3]);
   d[3] = make_float4(wv[4], wv[5], wv[6], wv[7]);
-  d[4] = make_float4(e0, e1, __int_as_float(cell), 0.f);
+  *reinterpret_cast<float2*>(d + 4) = make_float2(e0, e1);
 }
-template <> PD void stage_store<double>(double* st, const double (&wu)[kJ], const double (&wv)[kJ], double e0,
-                                        double e1, int cell) {
+PD void stage_store(double* st, const double (&wu)[kJ], const double (&wv)[kJ], double e0, double e1) {
   double2* d = reinterpret_cast<double2*>(st);
 #pragma unroll
   for (int a = 0; a < kJ / 2; ++a) {
@@ -127,210 +88,8 @@ template <> PD void stage_store<double>(double* st, const double (&wu)[kJ], cons
     d[kJ / 2 + a] = make_double2(wv[2 * a], wv[2 * a + 1]);
   }
   d[kJ] = make_double2(e0, e1);
-  d[kJ + 1] = make_double2(__hiloint2double(0, cell), 0.0);
 }
-static_assert(kStage == 2 * kJ + 4 && kJ == 8, "stage_store writes 2J + 4 values");
-
-template <typename T> __host__ __device__ inline size_t tile_patch_bytes(int TB) {
-  const size_t PW = size_t(TB + kJ);
-  return PW * (sizeof(T) == 4 ? 24 : PW + 2) * sizeof(typename cplx_t<T>::type);
-}
-template <typename T> __host__ __device__ inline size_t tile_acc_bytes(int TB) {
-  const size_t PW = size_t(TB + kJ);
-  return size_t(kWarps) * PW * (PW + 1) * sizeof(typename cplx_t<T>::type);
-}
-template <typename T> __host__ __device__ inline size_t tile_stage_bytes() {
-  return size_t(kWarps) * 32 * kStage * sizeof(T);
-}
-
-template <typename C> PD C warp_allsum(C v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-  }
-  return v;
-}
-
-// One CTA per work item; visibilities arrive sorted by grid cell inside the
-// tile.  Warp w takes a contiguous slice of the item.  In 32-wide batches
-// every lane first computes its own visibility's kernel weights (and, for
-// gridding, its value) into a per-warp staging row; then the warp walks the
-// batch one visibility at a time with lane l owning taps (l/4, 2(l%4)) and
-// (l/4, 2(l%4)+1) of the J x J footprint.  For a run of visibilities in the
-// same cell the lanes keep the footprint's grid values (gather) and its
-// scatter sums (gridding) in registers; shared memory is touched only when
-// the cell changes.  Gathered values are summed across the warp by a
-// butterfly of shuffles.  Scatter sums go to the warp's private accumulator
-// patch (no atomics); the patches are merged and flushed with one vector
-// atomic per non-zero cell at the end.
-template <typename T, int MODE>
-__global__ void __launch_bounds__(kThreads) k_tile(Geometry g, const __grid_constant__ CUtensorMap map,
-                                                   const WorkItem* __restrict__ items,
-                                                   const Pos<T>* __restrict__ pos, const int* __restrict__ perm,
-                                                   KbPoly<T> kb, DegridEp<typename cplx_t<T>::type> dep,
-                                                   GridPro<typename cplx_t<T>::type> gpro,
-                                                   typename cplx_t<T>::type* __restrict__ Q, int* err) {
-  typedef typename cplx_t<T>::type C;
-  typedef typename Pair2<T>::type T2;
-  constexpr bool kGather = MODE != TM_GRID;
-  constexpr bool kScatter = MODE != TM_DEGRID;
-  extern __shared__ __align__(128) unsigned char sm_raw[];
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ double red[32];
-  const WorkItem it = items[blockIdx.x];
-  const int tu = it.tile / g.ntv, tv = it.tile - tu * g.ntv;
-  const int PW = g.TB + kJ, PA = PW + 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned char* cur = sm_raw;
-  C* patch = reinterpret_cast<C*>(cur);
-  if (kGather) cur += tile_patch_bytes<T>(g.TB);
-  C* acc = reinterpret_cast<C*>(cur);
-  if (kScatter) {
-    cur += tile_acc_bytes<T>(g.TB);
-    for (int e = threadIdx.x; e < kWarps * PW * PA; e += kThreads) acc[e] = cz<C>();
-  }
-  T* stage = reinterpret_cast<T*>(cur);
-  if (kGather) {
-    if (!stage_patch(patch, &bar, &map, tu, tv, g.TB, PW, sizeof(T) == 4 ? 24 : PW + 2, err)) return;
-  } else {
-    __syncthreads();
-  }
-  C* wacc = acc + warp * PW * PA;
-  T* wst = stage + warp * 32 * kStage;
-  T scale = 0;
-  if (MODE == TM_GRID && gpro.mode == GP_BALL) scale = T(gpro.scalars[gpro.scale_idx]);
-  // this warp's contiguous slice of the work item
-  const int cnt = it.end - it.begin;
-  const int per = (cnt + kWarps - 1) / kWarps;
-  const int w0 = it.begin + min(cnt, warp * per), w1 = it.begin + min(cnt, (warp + 1) * per);
-  const int ta = lane >> 2, tb = (lane & 3) * 2;
-  int cell_cur = -1;
-  C g0 = cz<C>(), g1 = cz<C>();   // footprint grid values of the current cell (gather)
-  C s0 = cz<C>(), s1 = cz<C>();   // footprint scatter sums of the current cell
-  Acc<T> p0, p1;
-  for (int base = w0; base < w1; base += 32) {
-    const int i = base + lane;
-    const bool valid = i < w1;
-    T wu[kJ], wv[kJ];
-    int cu = 0, cv = 0;
-    C u = cz<C>();
-    if (valid) {
-      T fu, fv;
-      decode(pos[i], cu, fu, cv, fv);
-      kb_eval(kb, fu, wu);
-      kb_eval(kb, fv, wv);
-      if (MODE == TM_GRID) {
-        if (gpro.mode == GP_PERM) {
-          u = perm_value(perm[i], gpro.y[perm_index(perm[i])]);
-        } else if (gpro.mode == GP_SORTED) {
-          u = gpro.y[i];
-        } else {  // GP_BALL
-          const C v = gpro.z[i], yv = gpro.ys[i];
-          const T nu = T(gpro.nu);
-          const T cx = nu * yv.x, cy = nu * yv.y;
-          const T rx = fma(v.x - cx, scale, cx), ry = fma(v.y - cy, scale, cy);
-          gpro.z[i] = cmk<C>(v.x - rx, v.y - ry);
-          u = cmk<C>(T(2) * rx - v.x, T(2) * ry - v.y);
-        }
-      }
-    } else {
-#pragma unroll
-      for (int a = 0; a < kJ; ++a) wu[a] = wv[a] = T(0);
-    }
-    T* st = wst + lane * kStage;
-#pragma unroll
-    for (int a = 0; a < kJ; ++a) {
-      st[a] = wu[a];
-      st[kJ + a] = wv[a];
-    }
-    st[2 * kJ] = u.x;
-    st[2 * kJ + 1] = u.y;
-    *reinterpret_cast<int*>(st + 2 * kJ + 2) = cu * 256 + cv;
-    __syncwarp();
-    const int nv = min(32, w1 - base);
-    C mine = cz<C>();  // gathered value of this lane's own visibility
-    for (int j = 0; j < nv; ++j) {
-      const T* sj = wst + j * kStage;
-      const int cell = *reinterpret_cast<const int*>(sj + 2 * kJ + 2);
-      if (cell != cell_cur) {  // warp-uniform
-        const int ro = ((cell >> 8) + ta) * (sizeof(T) == 4 ? 24 : PW + 2) + (cell & 255) + tb;
-        if (kScatter && cell_cur >= 0) {
-          C* row = wacc + ((cell_cur >> 8) + ta) * PA + (cell_cur & 255) + tb;
-          row[0] = cadd(row[0], s0);
-          row[1] = cadd(row[1], s1);
-          s0 = s1 = cz<C>();
-        }
-        if (kGather) {
-          g0 = patch[ro];
-          g1 = patch[ro + 1];
-        }
-        cell_cur = cell;
-      }
-      const T wa = sj[ta];
-      const T2 wbp = *reinterpret_cast<const T2*>(sj + kJ + tb);
-      const T wb0 = wa * wbp.x, wb1 = wa * wbp.y;
-      C uj;
-      if (kGather) {
-        C part = cmk<C>(fma(wb0, g0.x, wb1 * g1.x), fma(wb0, g0.y, wb1 * g1.y));
-        uj = warp_allsum(part);
-        if (lane == j) mine = uj;
-      } else {
-        uj = cmk<C>(sj[2 * kJ], sj[2 * kJ + 1]);
-      }
-      if (kScatter) {
-        s0.x = fma(wb0, uj.x, s0.x);
-        s0.y = fma(wb0, uj.y, s0.y);
-        s1.x = fma(wb1, uj.x, s1.x);
-        s1.y = fma(wb1, uj.y, s1.y);
-      }
-    }
-    __syncwarp();
-    if (MODE == TM_DEGRID && valid) {
-      if (dep.mode == DG_STORE_PERM) {
-        dep.y[perm_index(perm[i])] = perm_value(perm[i], mine);
-      } else if (dep.mode == DG_STORE_SORTED) {
-        dep.y[i] = mine;
-      } else {  // DG_BALL
-        const C z = dep.z[i], yv = dep.ys[i];
-        const T nu = T(dep.nu);
-        const C v = cmk<C>(fma(nu, mine.x, z.x), fma(nu, mine.y, z.y));
-        dep.z[i] = v;
-        const T dx = fma(-nu, yv.x, v.x), dy = fma(-nu, yv.y, v.y);
-        p0.add_prod(dx, dx);
-        p0.add_prod(dy, dy);
-        const T ex = mine.x - yv.x, ey = mine.y - yv.y;
-        p1.add_prod(ex, ex);
-        p1.add_prod(ey, ey);
-      }
-    }
-  }
-  if (MODE == TM_DEGRID) {
-    if (dep.mode == DG_BALL) {
-      const Acc<T> r0 = block_merge<kThreads>(p0, red);
-      const Acc<T> r1 = block_merge<kThreads>(p1, red);
-      if (threadIdx.x == 0) {
-        reinterpret_cast<Acc<T>*>(dep.part0)[blockIdx.x] = r0;
-        reinterpret_cast<Acc<T>*>(dep.part1)[blockIdx.x] = r1;
-      }
-    }
-    return;
-  }
-  if (cell_cur >= 0) {
-    C* row = wacc + ((cell_cur >> 8) + ta) * PA + (cell_cur & 255) + tb;
-    row[0] = cadd(row[0], s0);
-    row[1] = cadd(row[1], s1);
-  }
-  __syncthreads();
-  // merge the warps' accumulators and flush the patch (one vector atomic per non-zero cell)
-  for (int e = threadIdx.x; e < PW * PW; e += kThreads) {
-    const int r = e / PW, c = e - r * PW;
-    C v = cz<C>();
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) v = cadd(v, acc[w * PW * PA + r * PA + c]);
-    if (v.x != 0 || v.y != 0) atomic_add_global(Q + size_t(tu * g.TB + r) * g.KC + (tv * g.TB + c), v);
-  }
-}
+static_assert(kJ == 8, "stage_store writes 2J + 2 values");
 
 // ---------------------------------------------------------------------------
 // Warp-per-item forms of degridding and gridding (the ball block and the
@@ -665,7 +424,7 @@ __global__ void __launch_bounds__(32 * kWItems) k_grid_w(Src src, KbPoly<T> kb) 
     {
       T* st = gst + q * kGrRec;
       const T wo[kJ] = {wv[0], wv[2], wv[4], wv[6], wv[1], wv[3], wv[5], wv[7]};
-      stage_store(st, wu, wo, u.x, u.y, 0);
+      stage_store(st, wu, wo, u.x, u.y);
     }
     __syncwarp();
     const int nj = min(kGrLanes, per - b);
@@ -1055,7 +814,6 @@ template <typename T> cudaError_t configure_nufft() {
   if (e == cudaSuccess) e = raise_smem_limit(k_grid_w<T, ArgVal<GridArgs<T>>>);
   if (e == cudaSuccess) e = raise_smem_limit(k_degrid_w<T, ArgTab<DegridArgs<T>>>);
   if (e == cudaSuccess) e = raise_smem_limit(k_grid_w<T, ArgTab<GridArgs<T>>>);
-  if (e == cudaSuccess) e = raise_smem_limit(k_tile<T, TM_GRAM>);
   return e;
 }
 template cudaError_t configure_nufft<float>();
@@ -1066,19 +824,6 @@ cudaError_t set_wait_spins_nufft(uint32_t spins) { return set_module_wait_spins(
 template <typename T> int degrid_patch_pitch(int TB) { return patch_pitch<T>(TB); }
 template int degrid_patch_pitch<float>(int);
 template int degrid_patch_pitch<double>(int);
-
-size_t tile_smem_bytes(int precision_bytes, int TB, int mode) {
-  if (precision_bytes == 4) {
-    size_t b = tile_stage_bytes<float>();
-    if (mode != TM_GRID) b += tile_patch_bytes<float>(TB);
-    if (mode != TM_DEGRID) b += tile_acc_bytes<float>(TB);
-    return b;
-  }
-  size_t b = tile_stage_bytes<double>();
-  if (mode != TM_GRID) b += tile_patch_bytes<double>(TB);
-  if (mode != TM_DEGRID) b += tile_acc_bytes<double>(TB);
-  return b;
-}
 
 template <typename T>
 void launch_degrid(const Geometry& g, const CUtensorMap& map, const WorkItem* items, int n_items, const Pos<T>* pos,
@@ -1117,16 +862,6 @@ void launch_grid_batch(const GridArgs<T>* tab, int count, int max_items, int max
   ArgTab<GridArgs<T>> src{tab};
   k_grid_w<T><<<dim3((max_items + kWItems - 1) / kWItems, count), 32 * kWItems,
                 kWItems * grid_warp_bytes<T>(max_tb), s>>>(src, kb);
-}
-
-template <typename T>
-void launch_gram(const Geometry& g, const CUtensorMap& map, const WorkItem* items, int n_items, const Pos<T>* pos,
-                 const KbPoly<T>& kb, typename cplx_t<T>::type* Q, int* err, cudaStream_t s) {
-  if (n_items <= 0) return;
-  const size_t sm = tile_smem_bytes(sizeof(T), g.TB, TM_GRAM);
-  DegridEp<typename cplx_t<T>::type> ep{};
-  GridPro<typename cplx_t<T>::type> gp{};
-  k_tile<T, TM_GRAM><<<n_items, kThreads, sm, s>>>(g, map, items, pos, nullptr, kb, ep, gp, Q, err);
 }
 
 template <typename T>
@@ -1291,8 +1026,6 @@ int build_bins(const double* uv, int64_t M, const Geometry& g, int chunk, Pos<T>
                                cudaStream_t);                                                                  \
   template void launch_degrid_batch<T>(const DegridArgs<T>*, int, int, int, const KbPoly<T>&, cudaStream_t);    \
   template void launch_grid_batch<T>(const GridArgs<T>*, int, int, int, const KbPoly<T>&, cudaStream_t);        \
-  template void launch_gram<T>(const Geometry&, const CUtensorMap&, const WorkItem*, int, const Pos<T>*,        \
-                               const KbPoly<T>&, cplx_t<T>::type*, int*, cudaStream_t);                         \
   template void launch_encode_x2<T>(const double*, const int*, int64_t, int, int, Pos<T>*, cudaStream_t);     \
   template int build_bins<T>(const double*, int64_t, const Geometry&, int, Pos<T>*, int*, WorkItem**, int*,     \
                              cudaStream_t, const int*, int, cudaMemPool_t);
