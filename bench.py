@@ -254,7 +254,7 @@ def run_ours(args, ws, rank, local):
     hbm, peak_kind = peaks()
     bytes_launch = algorithmic_bytes(dom, n, M, levels=L, cg=w.cg_iters)
     achieved = bytes_launch / (dom_ms / dom_n / 1e3) / 1e9
-    kernels_per_call = {"sara_analysis": 1 + L, "sara_synthesis": L}
+    kernels_per_call = {"sara_analysis": L, "sara_synthesis": L}  # one launch per level
     launches = sum(v[1] * kernels_per_call.get(k, 1) for k, v in kt.items() if k != "memset")
     per_kernel = {}
     for k, v in busy.items():
