@@ -178,10 +178,8 @@ template <typename T> class OpImpl : public purify_op {
   KbPoly<T> kb;
   SaraPlan<T> sara{};
   double* partials = nullptr;
-  double* cg_part = nullptr;        // CG partial sums (row pass, CG update)
-  unsigned int* tickets = nullptr;  // last-block tickets: CG reductions (0, 1), ball scalars (2)
+  unsigned int* tickets = nullptr;  // last-block ticket of the ball scalars
   double* fin_part = nullptr;       // per-CTA partials of the ball-scalar merge (2 x kFinCtas)
-  static constexpr int kCgPart = 4096;
   double* sc = nullptr;
   double* h_sc = nullptr;
   int* err = nullptr;
@@ -258,7 +256,7 @@ template <typename T> class OpImpl : public purify_op {
 
   int partials_cap = 0;
   int size_partials() {
-    const int np = std::max({2 * n_items, row_inv_blocks<T>(g), sara_partials_capacity(g.n, levels),
+    const int np = std::max({2 * n_items, sara_partials_capacity(g.n, levels),
                              vec_blocks(9 * N()), tv_partials(g.n), 1});
     if (2 * n_items > bpart_cap) {
       double* bnew = nullptr;
@@ -536,7 +534,6 @@ template <typename T> class OpImpl : public purify_op {
     block_sizes.assign(1, M);
     if ((rc = size_partials())) return rc;
     if ((rc = alloc(&eps_dev, 64)) || (rc = alloc(&scale_dev, 64))) return rc;
-    if ((rc = alloc(&cg_part, 5 * kCgPart))) return rc;
     if ((rc = alloc(&tickets, 4))) return rc;
     if ((rc = alloc(&fin_part, 2 * kFinCtas))) return rc;
     CK(cudaMemsetAsync(tickets, 0, 4 * sizeof(unsigned int), s));
@@ -601,7 +598,7 @@ template <typename T> class OpImpl : public purify_op {
   RowInvArgs<T> row_inv_args(const C* B, const T* dea, const RowEp<T>& ep_in) const {
     RowEp<T> ep = ep_in;
     if (!ep.err) ep.err = err;
-    return RowInvArgs<T>{g, B, dea, ep, tw, tws, row_inv_blocks<T>(g)};
+    return RowInvArgs<T>{g, B, dea, ep, tw, tws};
   }
   void fwd_grid(const RowPro<T>& pro, cudaStream_t s) {
     if (rec) {
@@ -678,11 +675,10 @@ template <typename T> class OpImpl : public purify_op {
   // The NUFFT form's visibilities, allocated on its first use.
   int ensure_gram() { return gram_y ? PURIFY_OK : alloc(&gram_y, size_t(g.M)); }
   C* gram_y = nullptr;
-  int row_ep(const RowEp<T>& ep, cudaStream_t s) {
+  void row_ep(const RowEp<T>& ep, cudaStream_t s) {
     const RowInvArgs<T> a = row_inv_args(gridA, deapod, ep);
     if (rec) record(R_RI, s).ri = a;
     else PROF(KK_ROW_INV, s, launch_row_inv_h<T>(a, s));
-    return a.nblocks;
   }
 
   // Set-up of the convolution form of Re(Phi^H Phi): the PSF
@@ -751,12 +747,11 @@ template <typename T> class OpImpl : public purify_op {
       gram_front(pro, s);
     }
   }
-  int normal_back(const RowEp<T>& ep, cudaStream_t s, C* B = nullptr) {
+  void normal_back(const RowEp<T>& ep, cudaStream_t s, C* B = nullptr) {
     if (!toep && !rec) return row_ep(ep, s);
     const RowInvArgs<T> a = row_inv_args(B ? B : gridA, nullptr, ep);
     if (rec) record(R_RI, s).ri = a;
     else PROF(KK_ROW_INV_H, s, launch_row_inv_h<T>(a, s));
-    return a.nblocks;
   }
 
   // out = (nu2 Re Phi^H Phi + 2I) x
@@ -881,37 +876,32 @@ template <typename T> class OpImpl : public purify_op {
     return PURIFY_OK;
   }
 
-  // ||Phi||^2 by power iteration on Re(Phi^H Phi) from the all-ones image / n.
-  int power_norm_sq(int iters, double* lam, cudaStream_t s) {
+  // ||Phi||^2 by power iteration on Re(Phi^H Phi) from the all-ones image / n
+  // (enqueue only; the result is power_norm_sq() once the scalars are read).
+  void power_iterations(int iters, cudaStream_t s) {
     launch_fill<T>(p, N(), T(1.0 / g.n), s);
     for (int it = 0; it < iters; ++it) {
-      RowPro<T> pro{};
-      if (it == 0) {
-        pro = plain(p);
-      } else {
+      RowPro<T> pro = plain(it == 0 ? p : Ap);
+      if (it > 0) {
         pro.mode = PRO_SCALE;
-        pro.x = Ap;
-        pro.scalars = sc;
-        pro.idx = S_INVNORM;
+        pro.acc = sc + S_POW0 + ((it - 1) & 1);
       }
+      pro.zero = sc + S_POW0 + (it & 1);
+      pro.nzero = 1;
       normal_front(pro, s);
       RowEp<T> ep{};
       ep.mode = EP_POWER;
       ep.out = Ap;
-      ep.partials = partials;
-      const int np = normal_back(ep, s);
-      fin(partials, np, FIN_NORM, 0.0, s);
+      ep.acc = pro.zero;
+      normal_back(ep, s);
     }
-    int rc = check(s, true);
-    if (rc) return rc;
-    if ((rc = read_scalars(s))) return rc;
-    *lam = h_sc[S_LAMBDA];
-    return PURIFY_OK;
   }
+  double power_norm_sq(int iters) const { return std::sqrt(h_sc[S_POW0 + ((iters - 1) & 1)]); }
 
   // 1e-3 ||Psi^H (nu^2 Re Phi^H y)||_inf with y the sorted visibilities
   // (Psi^H = I for the TV prior).
-  int default_gamma(double nu, double* gamma, cudaStream_t s) {
+  // (enqueue only; default_gamma() once the scalars are read).
+  void gamma_passes(cudaStream_t s) {
     zero_q(s);
     GridPro<C> pro{};
     pro.mode = GP_SORTED;
@@ -929,11 +919,10 @@ template <typename T> class OpImpl : public purify_op {
     }
     const int np = launch_reduce<T>(coef, D(), RED_MAXABS, sc, partials, s);
     launch_max_partials(partials, np, sc, s);
-    int rc = check(s, true);
-    if (rc) return rc;
-    if ((rc = read_scalars(s))) return rc;
-    *gamma = 1e-3 * nu * nu * h_sc[S_MAXABS];
-    return PURIFY_OK;
+  }
+  double default_gamma(double nu) const {
+    const double gamma = 1e-3 * nu * nu * h_sc[S_MAXABS];
+    return gamma > 0 ? gamma : 1e-12;
   }
 
   // Population standard deviation of Psi^H x_hat (reweighting delta_1), or
@@ -959,10 +948,9 @@ template <typename T> class OpImpl : public purify_op {
     const size_t n2 = N();
     // step 5: x_hat = (Phi^H Phi + 2I)^-1 sum_i x_i by CG, warm-started at x_hat.
     // The scalars stay on the device and need no launches of their own: the
-    // last block of the inverse row pass sets <r,r> (initial residual), or
-    // alpha and beta (CG step, from five inner products of the step's vectors);
-    // the forward row pass of the next step applies x += alpha p,
-    // r -= alpha Ap, p = r + beta p on the fly.  With the convolution form the
+    // inverse row pass accumulates five inner products of the step's vectors,
+    // and the forward row pass of the next step forms alpha and beta from them
+    // and applies x += alpha p, r -= alpha Ap, p = r + beta p on the fly.  With the convolution form the
     // initial residual b - A x_hat needs no operator pass here: A x_hat was
     // formed at the end of the previous iteration beside the ball block (or by
     // the round set-up), and the first forward row pass takes r = p = b - A x_hat.
@@ -975,10 +963,6 @@ template <typename T> class OpImpl : public purify_op {
       ep.p = xh;
       ep.b = xs;
       ep.nu2 = nu2;
-      ep.partials = cg_part;
-      ep.pstride = kCgPart;
-      ep.scalars = sc;
-      ep.ticket = tickets;
       normal_back(ep, s);
     }
     for (int it = 0; it < cg_iters; ++it) {
@@ -995,8 +979,10 @@ template <typename T> class OpImpl : public purify_op {
         pro.r = r;
         pro.xu = xh;
         pro.ap = Ap;
-        pro.scalars = sc;
+        pro.acc = sc + S_CG0 + 5 * ((it - 1) & 1);
       }
+      pro.zero = sc + S_CG0 + 5 * (it & 1);
+      pro.nzero = 5;
       normal_front(pro, s);
       RowEp<T> ep{};
       ep.mode = EP_CG_AP;
@@ -1004,15 +990,13 @@ template <typename T> class OpImpl : public purify_op {
       ep.p = p;
       ep.r = r;
       ep.nu2 = nu2;
-      ep.partials = cg_part;
-      ep.pstride = kCgPart;
-      ep.scalars = sc;
-      ep.ticket = tickets + 1;
+      ep.acc = pro.zero;
       normal_back(ep, s);
     }
     if (cg_iters > 0) {  // last step: x += alpha p
-      if (rec) record(R_AXPY, s).ax = AxpyArgs<T>{xh, p, sc, S_ALPHA, n2};
-      else PROF(KK_VEC, s, launch_axpy<T>(xh, p, sc, S_ALPHA, n2, s));
+      const double* acc = sc + S_CG0 + 5 * ((cg_iters - 1) & 1);
+      if (rec) record(R_AXPY, s).ax = AxpyArgs<T>{xh, p, acc, n2};
+      else PROF(KK_VEC, s, launch_axpy<T>(xh, p, acc, n2, s));
     }
     // The three proximal blocks (steps 6-8) are independent until their sum:
     // the ball block's degridding, projection and gridding run on the second
@@ -1053,10 +1037,10 @@ template <typename T> class OpImpl : public purify_op {
     dep.part1 = bpart + n_items;
     degrid(dep, b3);
     if (rec)
-      record(R_B1, b3).b1 = Ball1Args{bpart, bpart + n_items, n_items, nu, eps_dev, scale_dev, sc, fin_part, tickets + 2};
+      record(R_B1, b3).b1 = Ball1Args{bpart, bpart + n_items, n_items, nu, eps_dev, scale_dev, sc, fin_part, tickets};
     else
       PROF(KK_VEC, b3, launch_finalize_blocks<T>(bpart, bpart + n_items, reinterpret_cast<const int*>(items), n_items,
-                                                  nblocks, nu, eps_dev, scale_dev, sc, fin_part, tickets + 2, b3));
+                                                  nblocks, nu, eps_dev, scale_dev, sc, fin_part, tickets, b3));
     if (zpar) cudaStreamWaitEvent(b3, ev_zjoin, 0);
     else zero_q(b3);
     GridPro<C> gp{};
@@ -1132,6 +1116,7 @@ template <typename T> class OpImpl : public purify_op {
     double nu = 0, gamma = 0, decay = 0.1, delta1 = 0, prev = -1;
     int round = 0, t = 0, total = 0, converged = 0;
     bool active = false, round_ready = false;
+    bool early = false;  // nu and gamma given: the graph was captured before the set-up finished
     cudaGraphExec_t gexec = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr, ev_sc = nullptr;
   } run;
@@ -1145,7 +1130,10 @@ template <typename T> class OpImpl : public purify_op {
     run.active = false;
   }
 
-  int begin(const void* y, const purify_params* P, cudaStream_t user) override {
+  // begin in three parts, between which a batch lets its other instances'
+  // streams run: the set-up and the power iteration for nu (enqueued); nu, and
+  // the passes for gamma (enqueued); gamma, the graph and the round's start.
+  int begin_front(const void* y, const purify_params* P, cudaStream_t user) {
     if (!(P->eps > 0) || P->t_max < 1 || P->cg_iters < 1 || P->n_reweight < 0 || P->xi < 0 ||
         (P->nu <= 0 && P->power_iters < 1))
       return PURIFY_ERR_INVALID;
@@ -1183,24 +1171,45 @@ template <typename T> class OpImpl : public purify_op {
     // device still runs the set-up above (the PSF spectrum, the gather).
     const bool early = run.nu > 0 && run.gamma > 0;
     if (early && (rc = capture_iteration(s))) return rc;
-    CK(cudaStreamSynchronize(s));
+    run.early = early;
+    if (!(run.nu > 0)) power_iterations(run.P.power_iters, s);
+    CK(cudaMemcpyAsync(h_sc, sc, kNumScalars * sizeof(double), cudaMemcpyDeviceToHost, s));
+    return check(s, false);
+  }
+  int begin_gamma() {
+    cudaStream_t s = own;
+    int rc = check(s, true);
+    if (rc) return rc;
     if ((rc = take_input_flag("purify_sdmm_solve", "y holds a non-finite visibility"))) return rc;
     if (!(run.nu > 0)) {
-      double lam = 0;
-      if ((rc = power_norm_sq(P->power_iters, &lam, s))) return rc;
+      const double lam = power_norm_sq(run.P.power_iters);
       run.nu = lam > 0 ? 1.0 / std::sqrt(lam) : 1.0;
     }
     if (!(run.gamma > 0)) {
-      if ((rc = default_gamma(run.nu, &run.gamma, s))) return rc;
-      if (!(run.gamma > 0)) run.gamma = 1e-12;
+      gamma_passes(s);
+      CK(cudaMemcpyAsync(h_sc, sc, kNumScalars * sizeof(double), cudaMemcpyDeviceToHost, s));
     }
-    if (!early && (rc = capture_iteration(s))) return rc;
+    return check(s, false);
+  }
+  int begin_round() {
+    cudaStream_t s = own;
+    int rc;
+    if (!(run.gamma > 0)) {
+      if ((rc = check(s, true))) return rc;
+      run.gamma = default_gamma(run.nu);
+    }
+    if (!run.early && (rc = capture_iteration(s))) return rc;
     launch_fill<T>(w, D(), T(1), s);
-    CK(cudaMemsetAsync(xh, 0, n2 * sizeof(T), s));
-    CK(cudaMemsetAsync(sc + S_CG0, 0, 5 * sizeof(double), s));  // the CG's accumulators start at zero
+    CK(cudaMemsetAsync(xh, 0, N() * sizeof(T), s));
     run.active = true;
     own_pending = true;
     return check(s, false);
+  }
+  int begin(const void* y, const purify_params* P, cudaStream_t user) override {
+    int rc = begin_front(y, P, user);
+    if (!rc) rc = begin_gamma();
+    if (!rc) rc = begin_round();
+    return rc;
   }
 
   // One SDMM iteration captured as a CUDA graph (when the parameters ask for
@@ -1847,16 +1856,22 @@ int batch_solve(int count, purify_op* const* ops_in, const void* const* y, const
     b.ops.push_back(o);
   }
   // every instance's set-up (its CG operator, nu, gamma, state) on its own stream
-  for (int i = 0; i < count; ++i) {
-    purify_params P = params[i];
-    P.use_graph = 0;
-    P.gram = 1;
-    const int rc = b.ops[i]->begin(y[i], &P, user);
-    if (rc) {
-      for (int j = 0; j <= i; ++j) b.ops[j]->run_release();
-      return rc;
+  // (part by part, so that the instances' power iterations run side by side)
+  for (int part = 0; part < 3; ++part)
+    for (int i = 0; i < count; ++i) {
+      purify_params P = params[i];
+      P.use_graph = 0;
+      P.gram = 1;
+      OpImpl<T>* o = b.ops[i];
+      const int rc = part == 0 ? o->begin_front(y[i], &P, user) : (part == 1 ? o->begin_gamma() : o->begin_round());
+      if (rc) {
+        for (OpImpl<T>* q : b.ops) {
+          cudaStreamSynchronize(q->own);  // nothing left running that reads the caller's arrays
+          q->run_release();
+        }
+        return rc;
+      }
     }
-  }
   int rc = b.build();
   cudaStream_t bs = b.bs;
   if (!rc) {

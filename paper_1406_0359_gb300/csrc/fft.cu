@@ -523,11 +523,39 @@ PD void row_ep_store(const RowEp<T>& ep, size_t idx, bool al, const T (&val)[V],
   if constexpr (MODE == EP_CG_R0) vstore(ep.out2 + idx, o, al);
 }
 
+// The scalars of a prologue from the sums an earlier epilogue left (one thread;
+// FP64 arithmetic is slow, and its latency hides behind the loads in flight):
+//   PRO_CG_STEP: from <p,Ap>, <r,Ap>, <Ap,Ap>, <r,p> and <r,r> of the step's
+//             vectors the exact line search alpha = <r,p> / <p,Ap> (equal to
+//             <r,r> / <p,Ap> in exact arithmetic); the next residual norm by
+//             ||r - alpha Ap||^2 = <r,r> - 2 alpha <r,Ap> + alpha^2 <Ap,Ap>
+//             (clamped at 0); beta = ||r_new||^2 / <r,r>.
+//   PRO_SCALE: 1 / ||x||.
+template <typename T> PD void pro_scalars(const RowPro<T>& pro, T* ab) {
+  if (threadIdx.x == 0) {
+    if (pro.mode == PRO_CG_STEP) {
+      double q[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) q[k] = __ldcg(pro.acc + k);
+      const double alpha = cg_alpha(q[3], q[0]);
+      double rr = q[4] - 2.0 * alpha * q[1] + alpha * alpha * q[2];
+      if (rr < 0.0) rr = 0.0;
+      ab[0] = T(alpha);
+      ab[1] = T(q[4] > 0.0 ? rr / q[4] : 0.0);
+    } else {
+      const double l = sqrt(__ldcg(pro.acc));
+      ab[0] = T(l > 0.0 ? 1.0 / l : 0.0);
+    }
+  }
+  __syncthreads();
+}
+
 // Forward row prologue (see RowProMode) of V consecutive pixels of U chunks
 // of a row pair (pixel offsets ia of row a; row b is n further on).  All loads
 // precede the CG step's stores.
 template <int U, int V, typename T>
-PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al, T (&va)[U][V], T (&vb)[U][V]) {
+PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al, T (&va)[U][V], T (&vb)[U][V],
+                     T* ab /*[2], shared*/) {
   if (pro.mode == PRO_CG_STEP) {
     // x += alpha p, r -= alpha Ap, p = r + beta p (alpha, beta of the previous step)
     T xv[2 * U][V], rv[2 * U][V], pv[2 * U][V], av[2 * U][V];
@@ -542,9 +570,10 @@ PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al
     // completed before its column pass let this chain go on; A p and the
     // scalars from the pass just before
     pdl_wait();
-    const T alpha = T(pro.scalars[S_ALPHA]), beta = T(pro.scalars[S_BETA]);
 #pragma unroll
     for (int u = 0; u < 2 * U; ++u) vload(av[u], pro.ap + ia[u >> 1] + size_t(u & 1) * n, true);
+    pro_scalars(pro, ab);
+    const T alpha = ab[0], beta = ab[1];
 #pragma unroll
     for (int u = 0; u < 2 * U; ++u) {
       const size_t i = ia[u >> 1] + size_t(u & 1) * n;
@@ -586,7 +615,8 @@ PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al
     }
   } else {
     pdl_wait();
-    const T scl = pro.mode == PRO_SCALE ? T(pro.scalars[pro.idx]) : T(1);
+    if (pro.mode == PRO_SCALE) pro_scalars(pro, ab);
+    const T scl = pro.mode == PRO_SCALE ? ab[0] : T(1);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       vload(va[u], pro.x + ia[u], al);
@@ -602,104 +632,24 @@ PD void row_prologue(const RowPro<T>& pro, const size_t (&ia)[U], int n, bool al
   }
 }
 
-// Per-CTA partials of the epilogue sums (ep.partials + k * ep.pstride for the
-// k-th sum); the last CTA finalises the CG scalars in FP64:
-//   EP_CG_R0: <r, r>.
-//   EP_CG_AP: from <p,Ap>, <r,Ap>, <Ap,Ap>, <r,p> and <r,r> of this step's
-//             vectors: the exact line search alpha = <r,p> / <p,Ap> (equal to
-//             <r,r> / <p,Ap> in exact arithmetic); the next residual norm by
-//             ||r - alpha Ap||^2 = <r,r> - 2 alpha <r,Ap> + alpha^2 <Ap,Ap>
-//             (clamped at 0); beta = ||r_new||^2 / <r,r>.
-template <typename T>
-PD void row_ep_finish(const RowEp<T>& ep, EpAcc<T> part, double* red /*[5*32]*/, int bid, int nblocks) {
-  if (!ep.partials) return;
+// The epilogue's sums: each CTA's go into FP64 accumulators (ep.acc) by atomics;
+// the pass that needs them reads them there (row_prologue, k_axpy), so no CTA
+// waits for the others.
+template <typename T> PD void row_ep_finish(const RowEp<T>& ep, EpAcc<T> part, double* red /*[5*32]*/) {
+  if (!ep.acc) return;
   const int nsum = ep.mode == EP_CG_AP ? 5 : 1;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = int((blockDim.x + 31) >> 5);
   Acc<T>* st = reinterpret_cast<Acc<T>*>(red);
-  Acc<T>* P = reinterpret_cast<Acc<T>*>(ep.partials);
   for (int k = 0; k < nsum; ++k) {
     warp_merge(part.a[k]);
     if (lane == 0) st[k * 32 + w] = part.a[k];
   }
   __syncthreads();
-  // CG step: the CTA's five sums go straight into FP64 accumulators (atomic
-  // adds as the CTAs finish), so that the last CTA only reads five values
-  const bool acc64 = ep.mode == EP_CG_AP && ep.ticket;
-  if (w == 0) {
-    for (int k = 0; k < nsum; ++k) {
-      Acc<T> b = lane < nw ? st[k * 32 + lane] : Acc<T>();
-      warp_merge(b);
-      if (lane == 0) {
-        if (acc64) atomicAdd(ep.scalars + S_CG0 + k, b.value());
-        else P[size_t(k) * ep.pstride + bid] = b;
-      }
-    }
-  }
-  if (!ep.ticket || !last_block_done_t0(ep.ticket, unsigned(nblocks))) return;
-  if (acc64) {
-    if (threadIdx.x != 0) return;
-    double sum[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      sum[k] = __ldcg(ep.scalars + S_CG0 + k);
-      ep.scalars[S_CG0 + k] = 0.0;  // ready for the next step
-    }
-    double* sc = ep.scalars;
-    const double rr = sum[4];
-    const double alpha = sum[0] > 0.0 ? sum[3] / sum[0] : 0.0;
-    double rr_new = rr - 2.0 * alpha * sum[1] + alpha * alpha * sum[2];
-    if (rr_new < 0.0) rr_new = 0.0;
-    sc[S_PAP] = sum[0];
-    sc[S_ALPHA] = alpha;
-    sc[S_BETA] = rr > 0.0 ? rr_new / rr : 0.0;
-    sc[S_RR] = rr_new;
-    return;
-  }
-  // last block: merge all blocks' partials (fixed order), FP64 only at the end
-  EpAcc<T> tot;
-  int i = threadIdx.x;
-  for (; i + int(blockDim.x) < nblocks; i += 2 * blockDim.x) {  // two CTAs' partials in flight
-    Acc<T> v[2][5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k)
-      if (k < nsum) {
-        v[0][k] = P[size_t(k) * ep.pstride + i];
-        v[1][k] = P[size_t(k) * ep.pstride + i + blockDim.x];
-      }
-#pragma unroll
-    for (int k = 0; k < 5; ++k)
-      if (k < nsum) {
-        acc_merge(tot.a[k], v[0][k]);
-        acc_merge(tot.a[k], v[1][k]);
-      }
-  }
-  for (; i < nblocks; i += blockDim.x)
-    for (int k = 0; k < nsum; ++k) acc_merge(tot.a[k], P[size_t(k) * ep.pstride + i]);
-  for (int k = 0; k < nsum; ++k) {
-    warp_merge(tot.a[k]);
-    if (lane == 0) st[k * 32 + w] = tot.a[k];
-  }
-  __syncthreads();
-  if (w != 0) return;
-  double sum[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int k = 0; k < nsum; ++k) {
+  // one warp per sum where there are enough
+  for (int k = w; k < nsum; k += nw) {
     Acc<T> b = lane < nw ? st[k * 32 + lane] : Acc<T>();
     warp_merge(b);
-    sum[k] = b.value();
-  }
-  if (lane != 0) return;
-  double* sc = ep.scalars;
-  if (ep.mode == EP_CG_R0) {
-    sc[S_RR] = sum[0];
-  } else if (ep.mode == EP_CG_AP) {
-    const double rr = sum[4];
-    const double alpha = sum[0] > 0.0 ? sum[3] / sum[0] : 0.0;
-    double rr_new = rr - 2.0 * alpha * sum[1] + alpha * alpha * sum[2];
-    if (rr_new < 0.0) rr_new = 0.0;
-    sc[S_PAP] = sum[0];
-    sc[S_ALPHA] = alpha;
-    sc[S_BETA] = rr > 0.0 ? rr_new / rr : 0.0;
-    sc[S_RR] = rr_new;
+    if (lane == 0) atomicAdd(ep.acc + k, b.value());
   }
 }
 
@@ -732,6 +682,7 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
   extern __shared__ __align__(16) unsigned char sm_raw[];
   C* zb = reinterpret_cast<C*>(sm_raw);      // [PAIRS][n]: the packed rows
   C* bufs = zb + H::PAIRS * n;               // [PAIRS][2][BUF]
+  __shared__ T ab[2];
   const int r0 = int(blockIdx.x) * 2 * H::PAIRS;
   {
     constexpr int CH = H::PAIRS * n / V;     // chunks of V pixels of a row pair
@@ -749,7 +700,7 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
         at[u] = pr * n + i;
         ia[u] = size_t(r0 + 2 * pr) * n + i;
       }
-      row_prologue<U, V>(pro, ia, n, al, va, vb);
+      row_prologue<U, V>(pro, ia, n, al, va, vb, ab);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (deapod) {  // S: deapodisation of both rows (the Phi form; the convolution form has none)
@@ -770,6 +721,9 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
       }
     }
   }
+  // (every prologue has waited by now) the accumulators of this pass's product
+  if (pro.zero && blockIdx.x == 0)
+    for (int k = threadIdx.x; k < pro.nzero; k += NT) pro.zero[k] = 0.0;
   __syncthreads();
   const int half = threadIdx.x / TT, t = threadIdx.x - half * TT;
   const int pr = half >> 1, odd = half & 1;
@@ -1044,7 +998,7 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
   pdl_trigger();
   EpAcc<T> part;
   if (ok) part = row_ep_all<LOGN>(ep, bufs, ops, a.deapod, r0);
-  row_ep_finish(ep, part, red, int(blockIdx.x), a.nblocks);
+  row_ep_finish(ep, part, red);
 }
 
 // Real-form column passes of Phi and Phi^H on the padded half grid (K + J rows,
@@ -1360,14 +1314,6 @@ template <typename T, int LOGN> struct HalfShape {
   static size_t grid_smem() { return size_t(HG::COLS) * 2 * HG::BUF * sizeof(C); }
   static size_t conv_smem() { return size_t(HC::COLS) * 2 * HC::BUF * sizeof(C); }
 };
-// CTAs of one inverse row pass (its epilogue's partial sums).
-template <typename T> int row_inv_blocks(const Geometry& g) {
-  int b = 0;
-  PURIFY_LOGN_SWITCH(g.K, (b = HalfShape<T, L - 1>::row_ctas));
-  return b;
-}
-template int row_inv_blocks<float>(const Geometry&);
-template int row_inv_blocks<double>(const Geometry&);
 // Twiddles of the half transforms of length n: per stage after the first,
 // W(r k) = exp(-2 pi i r k / (Ns R)) as [r - 1][k], k < Ns; the row passes'
 // table, then the column passes' from element *col_at on.

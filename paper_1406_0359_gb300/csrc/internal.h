@@ -65,9 +65,9 @@ template <typename T> struct DbFilters { T h[kMaxDb][kMaxTaps]; T g[kMaxDb][kMax
 // Row-pass epilogues (inverse row FFT -> image): val = Re(.) * s[i1] s[i2].
 enum RowEpMode : int {
   EP_STORE = 0,     // out = val
-  EP_CG_AP = 1,     // out = nu2 val + 2 p (= A p);  partials <p,Ap>, <r,Ap>, <Ap,Ap>, <r,p>, <r,r>
-  EP_CG_R0 = 2,     // out = b - (nu2 val + 2 p); out2 = out; partial += out^2
-  EP_POWER = 3,     // out = val;                      partial += val^2
+  EP_CG_AP = 1,     // out = nu2 val + 2 p (= A p);  acc += <p,Ap>, <r,Ap>, <Ap,Ap>, <r,p>, <r,r>
+  EP_CG_R0 = 2,     // out = b - (nu2 val + 2 p); out2 = out
+  EP_POWER = 3,     // out = val;                      acc += |val|^2
   EP_XS_ADD = 4,    // out = b + nu val   (b may alias out)
   EP_QX = 5         // out = nu2 val + 2 p
 };
@@ -79,21 +79,15 @@ template <typename T> struct RowEp {
   const T* b;
   const T* r;        // EP_CG_AP: the CG residual
   double nu, nu2;
-  double* partials;  // per-CTA partial sums; the k-th sum at partials + k * pstride
-  size_t pstride;
-  // Device scalars (solver slots) finalised by the last block when ticket is
-  // set: EP_CG_R0 sets S_RR; EP_CG_AP sets S_PAP, S_ALPHA = <r,p> / <p,Ap>,
-  // S_BETA and the next <r,r> (from the five sums, see fft.cu).
-  double* scalars;
-  unsigned int* ticket;
+  double* acc;       // accumulators of the mode's sums (zeroed by the forward pass before), or null
   int* err;          // device error flag (timed-out operand staging)
 };
 
 // Forward row-pass prologues (image -> row FFT input).
 enum RowProMode : int {
   PRO_PLAIN = 0,    // src = x
-  PRO_CG_STEP = 1,  // x += alpha p, r -= alpha Ap, p = r + beta p (scalars S_ALPHA, S_BETA); src = p
-  PRO_SCALE = 2,    // src = x * scalars[scale_idx]   (power iteration normalisation)
+  PRO_CG_STEP = 1,  // x += alpha p, r -= alpha Ap, p = r + beta p (alpha, beta from acc); src = p
+  PRO_SCALE = 2,    // src = x / sqrt(acc[0])   (power iteration normalisation)
   PRO_CG_START = 3  // r = x - ap (b - A x_hat, A x_hat kept from the previous iteration), p = r; src = p
 };
 template <typename T> struct RowPro {
@@ -103,8 +97,9 @@ template <typename T> struct RowPro {
   T* r;
   T* xu;        // PRO_CG_STEP: the CG iterate
   const T* ap;  // PRO_CG_STEP: A p of the previous step
-  const double* scalars;
-  int idx;
+  const double* acc;  // PRO_CG_STEP, PRO_SCALE: the sums of the inverse pass before
+  double* zero;       // accumulators to zero for the next inverse pass (nzero of them), or null
+  int nzero;
 };
 
 // Degridding epilogues (per visibility slot i, value acc = (G F Z S x)_i).
@@ -165,7 +160,6 @@ template <typename T> struct RowInvArgs {
   RowEp<T> ep;
   const typename cplx_t<T>::type* tw;
   const typename cplx_t<T>::type* tws;
-  int nblocks;  // CTAs of the instance (its epilogue partials, its ticket)
 };
 template <typename T> struct ColFwdArgs {
   Geometry g;
@@ -225,8 +219,6 @@ template <typename T> cudaError_t configure_fft();
 template <typename T> cudaError_t configure_nufft();
 template <typename T> cudaError_t configure_sara();
 
-// CTAs of one inverse row pass (the partial sums its epilogue writes).
-template <typename T> int row_inv_blocks(const Geometry& g);
 // Stage twiddles of the row passes and (from element *col_at on) the column
 // passes for image side n.
 template <typename T> void half_twiddles(int n, std::vector<typename cplx_t<T>::type>& out, size_t* col_at);
@@ -244,8 +236,7 @@ template <typename T> void launch_col_conv_h(const ColConvArgs<T>& a, cudaStream
 // its Hermitian part).
 template <typename T> void launch_col_fwd_h(const ColFwdArgs<T>& a, cudaStream_t s);
 template <typename T> void launch_col_inv_h(const ColInvArgs<T>& a, cudaStream_t s);
-// Inverse row pass with the row epilogue (deapod: S^T, or null); its epilogue
-// writes row_inv_blocks partial sums.
+// Inverse row pass with the row epilogue (deapod: S^T, or null).
 template <typename T> void launch_row_inv_h(const RowInvArgs<T>& a, cudaStream_t s);
 // Batched real-form passes: `count` instances of the grid side g.K (image
 // sides 64..1024), one launch, arguments from a device table (instance =

@@ -15,18 +15,19 @@ template <typename T> struct Vec16;
 template <> struct Vec16<float> { typedef float4 type; static constexpr int W = 4; };
 template <> struct Vec16<double> { typedef double2 type; static constexpr int W = 2; };
 
-// x += sc[idx] p on 16-byte vectors (N / W of them, both arrays 16-byte aligned).
+// x += alpha p on 16-byte vectors (N / W of them, both arrays 16-byte aligned).
 template <typename T, typename Src>
 __global__ void __launch_bounds__(kT) k_axpy(Src src) {
   typedef typename Vec16<T>::type V;
   decltype(auto) args = src.get();
   T* __restrict__ x = args.x;
   const T* __restrict__ p = args.p;
-  const double* __restrict__ sc = args.sc;
-  const int idx = args.idx;
   const size_t N = args.N;
   constexpr int W = Vec16<T>::W;
-  const T a = T(sc[idx]);
+  __shared__ T alpha;
+  if (threadIdx.x == 0) alpha = T(cg_alpha(args.acc[3], args.acc[0]));
+  __syncthreads();
+  const T a = alpha;
   V* xv = reinterpret_cast<V*>(x);
   const V* pv = reinterpret_cast<const V*>(p);
   for (size_t i = size_t(blockIdx.x) * kT + threadIdx.x; i < N / W; i += size_t(gridDim.x) * kT) {
@@ -56,11 +57,6 @@ __global__ void __launch_bounds__(kT) k_finalize(Src src) {
     case FIN_OBJ:
       sc[S_OBJ] = a;
       break;
-    case FIN_NORM: {
-      const double l = sqrt(a);
-      sc[S_LAMBDA] = l;
-      sc[S_INVNORM] = l > 0.0 ? 1.0 / l : 0.0;
-    } break;
     case FIN_MEAN:  // arg = element count
       sc[S_MEAN] = a / arg;
       break;
@@ -304,10 +300,10 @@ inline int nblk(size_t N) {
 
 int vec_blocks(size_t N) { return nblk(N); }
 
-template <typename T> void launch_axpy(T* x, const T* p, const double* sc, int idx, size_t N, cudaStream_t s) {
+template <typename T> void launch_axpy(T* x, const T* p, const double* acc, size_t N, cudaStream_t s) {
   // one 16-byte vector per thread; N and the pointers are multiples of 16
   // bytes (n x n images, n >= 16; cudaMalloc'd arrays)
-  k_axpy<T><<<nblk((N + 3) / 4), kT, 0, s>>>(ArgVal<AxpyArgs<T>>{AxpyArgs<T>{x, p, sc, idx, N}});
+  k_axpy<T><<<nblk((N + 3) / 4), kT, 0, s>>>(ArgVal<AxpyArgs<T>>{AxpyArgs<T>{x, p, acc, N}});
 }
 template <typename T> void launch_axpy_batch(const AxpyArgs<T>* tab, int count, size_t N, cudaStream_t s) {
   k_axpy<T><<<dim3(nblk((N + 3) / 4), count), kT, 0, s>>>(ArgTab<AxpyArgs<T>>{tab});
@@ -387,7 +383,7 @@ cudaError_t wait_selftest(int deliver, cudaStream_t s, int* timed_out) {
 }
 
 #define INST(T)                                                                                       \
-  template void launch_axpy<T>(T*, const T*, const double*, int, size_t, cudaStream_t);                \
+  template void launch_axpy<T>(T*, const T*, const double*, size_t, cudaStream_t);                \
   template void launch_axpy_batch<T>(const AxpyArgs<T>*, int, size_t, cudaStream_t);                   \
   template void launch_finalize_batch<T>(const FinArgs*, int, cudaStream_t);                            \
   template void launch_finalize_ball1_batch<T>(const Ball1Args*, int, cudaStream_t);                    \

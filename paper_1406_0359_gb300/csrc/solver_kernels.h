@@ -9,17 +9,22 @@ namespace purify {
 
 // Device scalar slots (double[kNumScalars]).
 enum ScalarSlot : int {
-  S_RR = 0, S_ALPHA, S_BETA, S_PAP, S_BALLSCALE, S_BALLNORM, S_RESID, S_OBJ,
-  S_LAMBDA, S_INVNORM, S_MEAN, S_STD, S_MAXABS, S_FEAS,
-  S_CG0,  // S_CG0 .. S_CG0 + 4: a CG step's five inner products, accumulated across CTAs (zero between steps)
-  kNumScalars = S_CG0 + 5
+  S_BALLSCALE = 0, S_RESID, S_OBJ, S_MEAN, S_STD, S_MAXABS, S_FEAS,
+  // sums of the row passes' epilogues, accumulated across CTAs; two sets taken
+  // in turn, each zeroed by the forward pass of the step that fills it
+  S_CG0,                // a CG step's five inner products
+  S_POW0 = S_CG0 + 10,  // a power iteration's squared norm
+  kNumScalars = S_POW0 + 2
 };
-enum FinOp : int { FIN_OBJ = 0, FIN_NORM, FIN_MEAN, FIN_VAR };
+enum FinOp : int { FIN_OBJ = 0, FIN_MEAN, FIN_VAR };
 enum RedOp : int { RED_SQ = 0, RED_SUM, RED_VAR, RED_MAXABS };
 
 int vec_blocks(size_t N);
-// x += sc[idx] p; N a multiple of 4, both arrays 16-byte aligned.
-template <typename T> void launch_axpy(T* x, const T* p, const double* sc, int idx, size_t N, cudaStream_t s);
+// The step length of a CG step from its sums <r,p> and <p,Ap> (0 when the latter is).
+__host__ __device__ inline double cg_alpha(double rp, double pap) { return pap > 0.0 ? rp / pap : 0.0; }
+// The last CG step's x += alpha p, alpha from its sums; N a multiple of 4, both
+// arrays 16-byte aligned.
+template <typename T> void launch_axpy(T* x, const T* p, const double* acc, size_t N, cudaStream_t s);
 // Merge na partials (Acc<T> values in double-sized slots) and apply `op`.
 template <typename T> void launch_finalize(const double* pa, int na, int op, double arg, double* sc, cudaStream_t s);
 template <typename T>
@@ -42,7 +47,7 @@ template <typename C> void launch_scatter(const C* src, const int* perm, size_t 
 template <typename C> void launch_gather(const C* src, const int* perm, size_t M, C* dst, cudaStream_t s);
 // Batched vector steps of instances of one size (argument tables in device
 // memory; instance = blockIdx.y, one grid for all).
-template <typename T> struct AxpyArgs { T* x; const T* p; const double* sc; int idx; size_t N; };
+template <typename T> struct AxpyArgs { T* x; const T* p; const double* acc; size_t N; };
 template <typename T> void launch_axpy_batch(const AxpyArgs<T>* tab, int count, size_t N, cudaStream_t s);
 struct FinArgs { const double* pa; int na; int op; double arg; double* sc; };
 template <typename T> void launch_finalize_batch(const FinArgs* tab, int count, cudaStream_t s);
