@@ -1041,6 +1041,7 @@ __global__ void __launch_bounds__(GridHalf<T, LOGN>::NT, GridHalf<T, LOGN>::MINB
   const int half = threadIdx.x / TT, t = threadIdx.x - half * TT, odd = half & 1;
   const int c0 = NC * int(blockIdx.x) + 1;
   const bool packed = c0 + NC - 1 == n;  // this CTA's last column
+  pdl_wait();
   C* s = bufs + size_t(half) * H::BUF;
   {
     const int c = c0 + (half >> 1);
@@ -1054,6 +1055,7 @@ __global__ void __launch_bounds__(GridHalf<T, LOGN>::NT, GridHalf<T, LOGN>::MINB
     for (int m = 0; m < E; ++m) s[t + m * TT] = v[m];
   }
   __syncthreads();
+  pdl_trigger();
   for (int q = threadIdx.x; q < K; q += H::NT) {
     const int o = q & 1, m = q >> 1;
     C out[NC], col0 = cz<C>();
@@ -1114,6 +1116,7 @@ __global__ void __launch_bounds__(GridHalf<T, LOGN>::NT, GridHalf<T, LOGN>::MINB
   };
   constexpr int IT = K / H::NT, U = IT % 4 == 0 ? 4 : (IT % 2 == 0 ? 2 : 1);  // U sector loads in flight
   static_assert(K % H::NT == 0, "E is a multiple of COLS");
+  pdl_wait();
   for (int it = 0; it < IT; it += U) {
     C in[U][NC];
 #pragma unroll
@@ -1158,6 +1161,7 @@ __global__ void __launch_bounds__(GridHalf<T, LOGN>::NT, GridHalf<T, LOGN>::MINB
   half_sync<TT>(half);
   half_fft<H, 1>(v, t, s, half, a.tws);
   if (odd) half_omega<H, 1>(v, t, a.tw);
+  pdl_trigger();
   const int c = c0 + (half >> 1);
   half_join<H>(v, t, odd, bufs, half, a.B + (c == n ? size_t(0) : half_at(c, 0, n)));
 }
@@ -1354,14 +1358,14 @@ template <typename T> void launch_col_conv_h(const ColConvArgs<T>& a, cudaStream
 
 template <typename T> void launch_col_fwd_h(const ColFwdArgs<T>& a, cudaStream_t s) {
   ArgVal<ColFwdArgs<T>> src{a};
-  PURIFY_LOGN_SWITCH(a.g.K, (k_col_fwd_h<T, L - 1><<<HalfShape<T, L - 1>::grid_ctas, GridHalf<T, L - 1>::NT,
-                                                     HalfShape<T, L - 1>::grid_smem(), s>>>(src)));
+  PURIFY_LOGN_SWITCH(a.g.K, (launch_pdl(k_col_fwd_h<T, L - 1, ArgVal<ColFwdArgs<T>>>, HalfShape<T, L - 1>::grid_ctas,
+                                           GridHalf<T, L - 1>::NT, HalfShape<T, L - 1>::grid_smem(), s, src)));
 }
 
 template <typename T> void launch_col_inv_h(const ColInvArgs<T>& a, cudaStream_t s) {
   ArgVal<ColInvArgs<T>> src{a};
-  PURIFY_LOGN_SWITCH(a.g.K, (k_col_inv_h<T, L - 1><<<HalfShape<T, L - 1>::grid_ctas, GridHalf<T, L - 1>::NT,
-                                                     HalfShape<T, L - 1>::grid_smem(), s>>>(src)));
+  PURIFY_LOGN_SWITCH(a.g.K, (launch_pdl(k_col_inv_h<T, L - 1, ArgVal<ColInvArgs<T>>>, HalfShape<T, L - 1>::grid_ctas,
+                                           GridHalf<T, L - 1>::NT, HalfShape<T, L - 1>::grid_smem(), s, src)));
 }
 
 template <typename T> void launch_row_inv_h(const RowInvArgs<T>& a, cudaStream_t s) {

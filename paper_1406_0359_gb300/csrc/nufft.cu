@@ -134,18 +134,57 @@ PD bool warp_stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu
 // Degridding: one lane per visibility, its kernel weights in registers, its
 // J x J cells gathered from the warp's staged patch; visibilities are sorted by
 // cell, so a warp's lanes read neighbouring cells.  Bound by the shared-memory
-// pipe: 64 cells of 8 bytes at 128 bytes a clock are 4 cycles per visibility
-// (two for pairs of lanes in one cell, which share a read).  The form with
+// pipe -- 64 cells of 8 bytes at 128 bytes a clock are 4 cycles per visibility --
+// and instruction issue (14 warp instructions), both near 70%.  The form with
 // four lanes per visibility staged every weight through shared memory and
-// summed by shuffles, 7.8 cycles: 141 us a launch against 84 (1024^2,
+// summed by shuffles, 7.8 cycles: 141 us a launch against 80 (1024^2,
 // M = 4,194,304).
+// sum_b w[b] row[b] over a footprint row, FP32 as packed (re, im) pairs.
+template <typename C> struct TapRow;
+template <> struct TapRow<double2> {
+  double w[kJ];
+  PD void set(const double (&v)[kJ]) {
+#pragma unroll
+    for (int b = 0; b < kJ; ++b) w[b] = v[b];
+  }
+  PD void add(double2& acc, double wu, const double2* row) const {
+    double2 h = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int b = 0; b < kJ; ++b) {
+      const double2 c = row[b];
+      h.x = fma(w[b], c.x, h.x);
+      h.y = fma(w[b], c.y, h.y);
+    }
+    acc.x = fma(wu, h.x, acc.x);
+    acc.y = fma(wu, h.y, acc.y);
+  }
+};
+template <> struct TapRow<float2> {
+  unsigned long long w[kJ];  // (w, w)
+  PD void set(const float (&v)[kJ]) {
+#pragma unroll
+    for (int b = 0; b < kJ; ++b) asm("mov.b64 %0, {%1, %1};" : "=l"(w[b]) : "f"(v[b]));
+  }
+  PD void add(float2& acc, float wu, const float2* row) const {
+    unsigned long long h = 0ull;
+#pragma unroll
+    for (int b = 0; b < kJ; ++b) {
+      const unsigned long long c = *reinterpret_cast<const unsigned long long*>(row + b);
+      asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(h) : "l"(w[b]), "l"(c));
+    }
+    float x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(h));
+    acc.x = fmaf(wu, x, acc.x);
+    acc.y = fmaf(wu, y, acc.y);
+  }
+};
+
 template <typename T, typename Src>
 __global__ void __launch_bounds__(32 * kWItems) k_degrid_w(Src src, KbPoly<T> kb, const __grid_constant__ CUtensorMap map0) {
   typedef typename cplx_t<T>::type C;
   decltype(auto) a = src.get();
   const Geometry& g = a.g;
   const int n_items = a.n_items;
-  const Pos<T>* __restrict__ pos = a.pos;
   const int* __restrict__ perm = a.perm;
   const DegridEp<C>& dep = a.dep;
   const CUtensorMap* map = Src::kTable ? a.map : &map0;
@@ -160,13 +199,14 @@ __global__ void __launch_bounds__(32 * kWItems) k_degrid_w(Src src, KbPoly<T> kb
   const size_t pe = warp_patch_elems<T>(g.TB);
   C* patch = reinterpret_cast<C*>(sm_raw) + warp * pe;
   if (Src::kTable && lane == 0) tensormap_acquire(map);
+  const Pos<T>* __restrict__ pos = a.pos;
   int i = it.begin + lane;
   Pos<T> p = pos[min(i, it.end - 1)];  // the first positions arrive beside the patch
+  pdl_wait();  // (items and positions are the operator's, written at its set-up)
   if (!warp_stage_patch(patch, &bars[warp], map, tu, tv, g.TB, uint32_t(pe * sizeof(C)), lane, a.err)) return;
   const bool ball = dep.mode == DG_BALL;
   Acc<T> p0, p1;
   for (; i - lane < it.end; i += 32) {
-    const bool valid = i < it.end;
     const int is = min(i, it.end - 1);
     // the epilogue's operands and the next positions are on their way while the taps are summed
     C z = cz<C>(), yv = cz<C>();
@@ -184,22 +224,13 @@ __global__ void __launch_bounds__(32 * kWItems) k_degrid_w(Src src, KbPoly<T> kb
     decode(cur, cu, fu, cv, fv);
     kb_eval(kb, fu, wu);
     kb_eval(kb, fv, wv);
+    TapRow<C> taps;
+    taps.set(wv);
     const C* row = patch + cu * PP + cv;
     C acc = cz<C>();
 #pragma unroll
-    for (int r = 0; r < kJ; ++r) {
-      C h = cz<C>();
-#pragma unroll
-      for (int b = 0; b < kJ; ++b) {
-        const C c = row[b];
-        h.x = fma(wv[b], c.x, h.x);
-        h.y = fma(wv[b], c.y, h.y);
-      }
-      acc.x = fma(wu[r], h.x, acc.x);
-      acc.y = fma(wu[r], h.y, acc.y);
-      row += PP;
-    }
-    if (!valid) continue;
+    for (int r = 0; r < kJ; ++r, row += PP) taps.add(acc, wu[r], row);
+    if (i >= it.end) continue;
     if (ball) {
       const T nu = T(dep.nu);
       const C v = cmk<C>(fma(nu, acc.x, z.x), fma(nu, acc.y, z.y));
@@ -217,6 +248,7 @@ __global__ void __launch_bounds__(32 * kWItems) k_degrid_w(Src src, KbPoly<T> kb
     }
   }
   __syncwarp();
+  pdl_trigger();
   if (ball) {
     warp_merge(p0);
     warp_merge(p1);
@@ -379,6 +411,7 @@ __global__ void __launch_bounds__(32 * kWItems) k_grid_w(Src src, KbPoly<T> kb) 
     const int nz = kGroups * cells * int(sizeof(GCell<T>)) / 16;
     for (int e = lane; e < nz; e += 32) zp[e] = make_uint4(0, 0, 0, 0);
   }
+  pdl_wait();
   T scale = 0;
   if (gpro.mode == GP_BALL) scale = T(gpro.block_scale ? gpro.block_scale[it.pad] : gpro.scalars[gpro.scale_idx]);
   GCell<T>* mine = patches + grp * cells + r * PS + h;
@@ -447,6 +480,7 @@ __global__ void __launch_bounds__(32 * kWItems) k_grid_w(Src src, KbPoly<T> kb) 
     }
   }
   if (run >= 0) acc.flush(mine + run);
+  pdl_trigger();
   __syncwarp();
   // pairs of cells, 8 (tiles of 8) or 12 of 16 (tiles of 16) lanes to a row
   const int ls = g.TB == 8 ? 3 : 4, pc = 2 * (lane & ((1 << ls) - 1));
@@ -832,7 +866,7 @@ void launch_degrid(const Geometry& g, const CUtensorMap& map, const WorkItem* it
   if (n_items <= 0) return;
   const size_t sm = kWItems * warp_patch_elems<T>(g.TB) * sizeof(typename cplx_t<T>::type);
   ArgVal<DegridArgs<T>> src{DegridArgs<T>{g, nullptr, items, n_items, pos, perm, ep, err}};
-  k_degrid_w<T><<<(n_items + kWItems - 1) / kWItems, 32 * kWItems, sm, s>>>(src, kb, map);
+  launch_pdl(k_degrid_w<T, ArgVal<DegridArgs<T>>>, (n_items + kWItems - 1) / kWItems, 32 * kWItems, sm, s, src, kb, map);
 }
 
 template <typename T>
@@ -852,7 +886,8 @@ void launch_grid(const Geometry& g, const WorkItem* items, int n_items, const Po
                  cudaStream_t s) {
   if (n_items <= 0) return;
   ArgVal<GridArgs<T>> src{GridArgs<T>{g, items, n_items, pos, perm, pro, Q}};
-  k_grid_w<T><<<(n_items + kWItems - 1) / kWItems, 32 * kWItems, kWItems * grid_warp_bytes<T>(g.TB), s>>>(src, kb);
+  launch_pdl(k_grid_w<T, ArgVal<GridArgs<T>>>, (n_items + kWItems - 1) / kWItems, 32 * kWItems,
+             kWItems * grid_warp_bytes<T>(g.TB), s, src, kb);
 }
 
 template <typename T>
