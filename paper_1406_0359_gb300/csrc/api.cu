@@ -178,8 +178,7 @@ template <typename T> class OpImpl : public purify_op {
   KbPoly<T> kb;
   SaraPlan<T> sara{};
   double* partials = nullptr;
-  unsigned int* tickets = nullptr;  // last-block ticket of the ball scalars
-  double* fin_part = nullptr;       // per-CTA partials of the ball-scalar merge (2 x kFinCtas)
+  double* ball_acc = nullptr;       // accumulators of the ball block's norms (one block; zero between iterations)
   double* sc = nullptr;
   double* h_sc = nullptr;
   int* err = nullptr;
@@ -534,9 +533,7 @@ template <typename T> class OpImpl : public purify_op {
     block_sizes.assign(1, M);
     if ((rc = size_partials())) return rc;
     if ((rc = alloc(&eps_dev, 64)) || (rc = alloc(&scale_dev, 64))) return rc;
-    if ((rc = alloc(&tickets, 4))) return rc;
-    if ((rc = alloc(&fin_part, 2 * kFinCtas))) return rc;
-    CK(cudaMemsetAsync(tickets, 0, 4 * sizeof(unsigned int), s));
+    if ((rc = alloc(&ball_acc, 2 * kBallAcc))) return rc;
     if (light) return check(s, false);  // its user synchronises s
     // TMA descriptor of the padded forward grid, 8-byte elements
     EncodeTiledFn enc = encode_fn();
@@ -1035,12 +1032,14 @@ template <typename T> class OpImpl : public purify_op {
     dep.nu = nu;
     dep.part0 = bpart;
     dep.part1 = bpart + n_items;
+    dep.acc = nblocks == 1 ? ball_acc : nullptr;
     degrid(dep, b3);
-    if (rec)
-      record(R_B1, b3).b1 = Ball1Args{bpart, bpart + n_items, n_items, nu, eps_dev, scale_dev, sc, fin_part, tickets};
+    const Ball1Args b1{ball_acc, nu, eps_dev, scale_dev, sc};
+    if (rec) record(R_B1, b3).b1 = b1;
+    else if (nblocks == 1) PROF(KK_VEC, b3, launch_finalize_ball1(b1, b3));
     else
       PROF(KK_VEC, b3, launch_finalize_blocks<T>(bpart, bpart + n_items, reinterpret_cast<const int*>(items), n_items,
-                                                  nblocks, nu, eps_dev, scale_dev, sc, fin_part, tickets, b3));
+                                                  nblocks, nu, eps_dev, scale_dev, sc, b3));
     if (zpar) cudaStreamWaitEvent(b3, ev_zjoin, 0);
     else zero_q(b3);
     GridPro<C> gp{};
@@ -1079,13 +1078,13 @@ template <typename T> class OpImpl : public purify_op {
     } else {
       // block 1 (l1 on Psi^H x_hat) fused into the analysis, block 2 (positivity)
       // fused into the synthesis: xs = x_1 + x_2
-      L1Block<T> b1{};
-      b1.z1 = z1;
-      b1.w = w;
-      b1.gamma = gamma;
-      b1.partials = partials;
+      L1Block<T> lb{};
+      lb.z1 = z1;
+      lb.w = w;
+      lb.gamma = gamma;
+      lb.partials = partials;
       int npo = 0;
-      PROF(KK_SARA_ANA, s, npo = sara_analysis_prox<T>(sara, xh, b1, s));
+      PROF(KK_SARA_ANA, s, npo = sara_analysis_prox<T>(sara, xh, lb, s));
       fin(partials, npo, FIN_OBJ, 0.0, s);
       PROF(KK_SARA_SYN, s, sara_synthesis_pos<T>(sara, xh, z2, xs, s));
     }
@@ -1201,6 +1200,7 @@ template <typename T> class OpImpl : public purify_op {
     if (!run.early && (rc = capture_iteration(s))) return rc;
     launch_fill<T>(w, D(), T(1), s);
     CK(cudaMemsetAsync(xh, 0, N() * sizeof(T), s));
+    CK(cudaMemsetAsync(ball_acc, 0, 2 * kBallAcc * sizeof(double), s));
     run.active = true;
     own_pending = true;
     return check(s, false);
@@ -1782,7 +1782,7 @@ template <typename T> class BatchImpl {
             launch_grid_batch<T>(static_cast<const GridArgs<T>*>(tab), cnt, gr.max_items, gr.max_tb,
                                  ops[gr.idx[0]]->kb, s);
             break;
-          case OpImpl<T>::R_B1: launch_finalize_ball1_batch<T>(static_cast<const Ball1Args*>(tab), cnt, s); break;
+          case OpImpl<T>::R_B1: launch_finalize_ball1_batch(static_cast<const Ball1Args*>(tab), cnt, s); break;
           case OpImpl<T>::R_ZERO: launch_zero_batch(static_cast<const ZeroArgs*>(tab), cnt, gr.max_q, s); break;
           case OpImpl<T>::R_AXPY: launch_axpy_batch<T>(static_cast<const AxpyArgs<T>*>(tab), cnt, N, s); break;
           case OpImpl<T>::R_FIN: launch_finalize_batch<T>(static_cast<const FinArgs*>(tab), cnt, s); break;

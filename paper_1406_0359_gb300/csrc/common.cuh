@@ -192,40 +192,6 @@ template <int NT> __device__ double block_max(double v, double* sh) {
   return r;
 }
 
-// Last-block reduction: every block has written partials[blockIdx.x]; the
-// block that finishes last (atomic ticket, no waiting) returns true in all
-// its threads, after which it may read all partials.  It resets the ticket.
-__device__ __forceinline__ bool last_block_done(unsigned int* ticket,
-                                                unsigned int count = gridDim.x * gridDim.y * gridDim.z) {
-  __shared__ bool last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned int t = atomicAdd(ticket, 1u);
-    last = (t == count - 1);
-    if (last) *ticket = 0u;
-  }
-  __syncthreads();
-  if (last) __threadfence();
-  return last;
-}
-
-// As last_block_done, for blocks whose global results for the last block
-// were all written by thread 0 (only thread 0 fences before the ticket);
-// `count` blocks take part (one instance's blocks of a batched launch).
-__device__ __forceinline__ bool last_block_done_t0(unsigned int* ticket, unsigned int count) {
-  __shared__ bool last;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned int t = atomicAdd(ticket, 1u);
-    last = (t == count - 1);
-    if (last) *ticket = 0u;
-  }
-  __syncthreads();
-  if (last) __threadfence();
-  return last;
-}
-
 // Programmatic dependent launch: a kernel lets the next one on its stream be
 // scheduled at once (pdl_trigger) and, before it touches anything an earlier
 // kernel wrote or still reads, waits for all earlier kernels to have completed

@@ -114,9 +114,11 @@ template <typename C> struct DegridEp {
   C* z;
   const C* ys;
   double nu;
-  double* part0;
+  double* part0;  // DG_BALL: per work item, its two sums ...
   double* part1;
+  double* acc;    // ... or, if set, kBallAcc pairs of FP64 accumulators instead
 };
+constexpr int kBallAcc = 64;
 
 // Gridding prologues (value u scattered for slot i).
 enum GridMode : int {

@@ -252,7 +252,11 @@ __global__ void __launch_bounds__(32 * kWItems) k_degrid_w(Src src, KbPoly<T> kb
   if (ball) {
     warp_merge(p0);
     warp_merge(p1);
-    if (lane == 0) {
+    if (lane == 0 && dep.acc) {
+      double* acc = dep.acc + 2 * (item % kBallAcc);
+      atomicAdd(acc, p0.value());
+      atomicAdd(acc + 1, p1.value());
+    } else if (lane == 0) {
       reinterpret_cast<Acc<T>*>(dep.part0)[item] = p0;
       reinterpret_cast<Acc<T>*>(dep.part1)[item] = p1;
     }

@@ -2,6 +2,7 @@
 // reweighting: the last CG update, deterministic finalisation of device
 // scalars from compensated per-block partials (the l2-ball scales, the
 // objective, norms), visibility permutation and the reweighting rule.
+#include "internal.h"
 #include "solver_kernels.h"
 
 namespace purify {
@@ -127,64 +128,33 @@ __global__ void __launch_bounds__(kFinT) k_finalize_blocks(const double* __restr
   }
 }
 
-// The same scalars for one visibility block (R = 1) in two levels: kFinCtas
-// CTAs each merge a contiguous slice of the items' partials (fixed order),
-// the last CTA to finish (ticket) merges the CTAs' partials in index order.
-template <typename T, typename Src>
-__global__ void __launch_bounds__(kT) k_finalize_ball1(Src src) {
-  __shared__ double red[32];
-  decltype(auto) args = src.get();
-  const double* __restrict__ part0 = args.part0;
-  const double* __restrict__ part1 = args.part1;
-  const int n_items = args.n_items;
-  const double nu = args.nu;
-  const double* __restrict__ eps_b = args.eps_b;
-  double* __restrict__ scale_b = args.scale_b;
-  double* __restrict__ sc = args.sc;
-  double* __restrict__ cpart = args.cpart;
-  unsigned int* __restrict__ ticket = args.ticket;
-  const Acc<T>* p0 = reinterpret_cast<const Acc<T>*>(part0);
-  const Acc<T>* p1 = reinterpret_cast<const Acc<T>*>(part1);
-  Acc<T>* c0 = reinterpret_cast<Acc<T>*>(cpart);
-  Acc<T>* c1 = c0 + gridDim.x;
-  const int per = (n_items + int(gridDim.x) - 1) / int(gridDim.x);
-  const int lo = int(blockIdx.x) * per, hi = min(n_items, lo + per);
-  constexpr int U = 4;
-  Acc<T> a, c;
-  int i = lo + int(threadIdx.x);
-  for (; i + (U - 1) * kT < hi; i += U * kT) {
-    Acc<T> x[U], y[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      x[u] = p0[i + u * kT];
-      y[u] = p1[i + u * kT];
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      acc_merge(a, x[u]);
-      acc_merge(c, y[u]);
-    }
+// The same scalars for one visibility block (R = 1) from the accumulators that
+// degridding's work items added to (kBallAcc pairs, zeroed again here): one CTA,
+// on the iteration's critical path.  Merging the items' compensated partials
+// in two levels instead took 8.5-9 us at 7000 to 45000 items.
+template <typename Src> __global__ void __launch_bounds__(kBallAcc) k_finalize_ball1(Src src) {
+  __shared__ double red[kBallAcc / 32][2];
+  decltype(auto) a = src.get();
+  pdl_wait();
+  double* acc = a.acc + 2 * threadIdx.x;
+  const double av = warp_sum(__ldcg(acc)), cv = warp_sum(__ldcg(acc + 1));
+  acc[0] = acc[1] = 0.0;
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5][0] = av;
+    red[threadIdx.x >> 5][1] = cv;
   }
-  for (; i < hi; i += kT) {
-    acc_merge(a, p0[i]);
-    acc_merge(c, p1[i]);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double v = 0.0, c = 0.0;
+  for (int w = 0; w < kBallAcc / 32; ++w) {
+    v += red[w][0];
+    c += red[w][1];
   }
-  a = block_merge<kT>(a, red);
-  c = block_merge<kT>(c, red);
-  if (threadIdx.x == 0) {
-    c0[blockIdx.x] = a;
-    c1[blockIdx.x] = c;
-  }
-  if (!last_block_done(ticket, gridDim.x)) return;
-  const double av = merge_array<kT>(c0, int(gridDim.x), red).value();
-  const double cv = merge_array<kT>(c1, int(gridDim.x), red).value();
-  if (threadIdx.x == 0) {
-    const double s = sqrt(av), rad = nu * eps_b[0];
-    scale_b[0] = s <= rad ? 1.0 : rad / s;
-    sc[S_RESID] = sqrt(cv);
-    sc[S_FEAS] = sqrt(cv) / eps_b[0];
-    sc[S_BALLSCALE] = scale_b[0];
-  }
+  const double s = sqrt(v), rad = a.nu * a.eps_b[0], scale = s <= rad ? 1.0 : rad / s;
+  a.scale_b[0] = scale;
+  a.sc[S_RESID] = sqrt(c);
+  a.sc[S_FEAS] = sqrt(c) / a.eps_b[0];
+  a.sc[S_BALLSCALE] = scale;
 }
 
 // Per-block partials of a reduction over v: compensated sums (RED_SUM, RED_VAR
@@ -311,8 +281,11 @@ template <typename T> void launch_axpy_batch(const AxpyArgs<T>* tab, int count, 
 template <typename T> void launch_finalize_batch(const FinArgs* tab, int count, cudaStream_t s) {
   k_finalize<T><<<dim3(1, count), kT, 0, s>>>(ArgTab<FinArgs>{tab});
 }
-template <typename T> void launch_finalize_ball1_batch(const Ball1Args* tab, int count, cudaStream_t s) {
-  k_finalize_ball1<T><<<dim3(kFinCtas, count), kT, 0, s>>>(ArgTab<Ball1Args>{tab});
+void launch_finalize_ball1(const Ball1Args& a, cudaStream_t s) {
+  launch_pdl(k_finalize_ball1<ArgVal<Ball1Args>>, 1, kBallAcc, 0, s, ArgVal<Ball1Args>{a});
+}
+void launch_finalize_ball1_batch(const Ball1Args* tab, int count, cudaStream_t s) {
+  k_finalize_ball1<<<dim3(1, count), kBallAcc, 0, s>>>(ArgTab<Ball1Args>{tab});
 }
 void launch_zero_batch(const ZeroArgs* tab, int count, size_t max_bytes, cudaStream_t s) {
   size_t b = (max_bytes / 16 + kT - 1) / kT;
@@ -333,16 +306,8 @@ int launch_reduce(const T* v, size_t N, int op, const double* sc, double* partia
 
 template <typename T>
 void launch_finalize_blocks(const double* part0, const double* part1, const int* items_as_int, int n_items, int R,
-                            double nu, const double* eps_b, double* scale_b, double* sc, double* cpart,
-                            unsigned int* ticket, cudaStream_t s) {
-  if (R == 1 && cpart && ticket) {
-    int nb = (n_items + 4 * kT - 1) / (4 * kT);
-    nb = nb < 1 ? 1 : (nb > kFinCtas ? kFinCtas : nb);
-    k_finalize_ball1<T><<<nb, kT, 0, s>>>(
-        ArgVal<Ball1Args>{Ball1Args{part0, part1, n_items, nu, eps_b, scale_b, sc, cpart, ticket}});
-  } else {
-    k_finalize_blocks<T><<<1, kFinT, 0, s>>>(part0, part1, items_as_int + 3, n_items, R, nu, eps_b, scale_b, sc);
-  }
+                            double nu, const double* eps_b, double* scale_b, double* sc, cudaStream_t s) {
+  k_finalize_blocks<T><<<1, kFinT, 0, s>>>(part0, part1, items_as_int + 3, n_items, R, nu, eps_b, scale_b, sc);
 }
 
 void launch_max_partials(const double* p, int np, double* sc, cudaStream_t s) {
@@ -386,11 +351,9 @@ cudaError_t wait_selftest(int deliver, cudaStream_t s, int* timed_out) {
   template void launch_axpy<T>(T*, const T*, const double*, size_t, cudaStream_t);                \
   template void launch_axpy_batch<T>(const AxpyArgs<T>*, int, size_t, cudaStream_t);                   \
   template void launch_finalize_batch<T>(const FinArgs*, int, cudaStream_t);                            \
-  template void launch_finalize_ball1_batch<T>(const Ball1Args*, int, cudaStream_t);                    \
   template void launch_finalize<T>(const double*, int, int, double, double*, cudaStream_t);             \
   template void launch_finalize_blocks<T>(const double*, const double*, const int*, int, int, double,           \
-                                          const double*, double*, double*, double*, unsigned int*,             \
-                                          cudaStream_t);                                                       \
+                                          const double*, double*, double*, cudaStream_t);                      \
   template int launch_reduce<T>(const T*, size_t, int, const double*, double*, cudaStream_t);           \
   template void launch_reweight<T>(T*, size_t, double, cudaStream_t);                                   \
   template void launch_fill<T>(T*, size_t, T, cudaStream_t);                                            \

@@ -30,15 +30,21 @@ template <typename T> void launch_finalize(const double* pa, int na, int op, dou
 template <typename T>
 int launch_reduce(const T* v, size_t N, int op, const double* sc, double* partials, cudaStream_t s);
 void launch_max_partials(const double* p, int np, double* sc, cudaStream_t s);
-// Ball scalars per visibility block; items_as_int points at the WorkItem array
-// (four ints per item, the block in the fourth).  With R = 1, cpart (2 x
-// kFinCtas doubles) and a zeroed ticket, the merge runs on up to kFinCtas
-// CTAs in two levels; otherwise on one CTA.
-constexpr int kFinCtas = 64;
+// Ball scalars per visibility block from the work items' partials; items_as_int
+// points at the WorkItem array (four ints per item, the block in the fourth).
 template <typename T>
 void launch_finalize_blocks(const double* part0, const double* part1, const int* items_as_int, int n_items, int R,
-                            double nu, const double* eps_b, double* scale_b, double* sc, double* cpart,
-                            unsigned int* ticket, cudaStream_t s);
+                            double nu, const double* eps_b, double* scale_b, double* sc, cudaStream_t s);
+// The same scalars for one block (R = 1) from kBallAcc accumulator pairs, which
+// are left at zero.
+struct Ball1Args {
+  double* acc;
+  double nu;
+  const double* eps_b;
+  double* scale_b;
+  double* sc;
+};
+void launch_finalize_ball1(const Ball1Args& a, cudaStream_t s);
 template <typename T> void launch_reweight(T* w, size_t N, double delta, cudaStream_t s);
 template <typename T> void launch_fill(T* v, size_t N, T val, cudaStream_t s);
 template <typename T> void launch_scale(T* v, size_t N, const double* sc, int idx, double mul, cudaStream_t s);
@@ -51,19 +57,7 @@ template <typename T> struct AxpyArgs { T* x; const T* p; const double* acc; siz
 template <typename T> void launch_axpy_batch(const AxpyArgs<T>* tab, int count, size_t N, cudaStream_t s);
 struct FinArgs { const double* pa; int na; int op; double arg; double* sc; };
 template <typename T> void launch_finalize_batch(const FinArgs* tab, int count, cudaStream_t s);
-struct Ball1Args {
-  const double* part0;
-  const double* part1;
-  int n_items;
-  double nu;
-  const double* eps_b;
-  double* scale_b;
-  double* sc;
-  double* cpart;
-  unsigned int* ticket;
-};
-// kFinCtas CTAs per instance (the two-level merge of the R = 1 ball scalars).
-template <typename T> void launch_finalize_ball1_batch(const Ball1Args* tab, int count, cudaStream_t s);
+void launch_finalize_ball1_batch(const Ball1Args* tab, int count, cudaStream_t s);
 struct ZeroArgs { void* p; size_t bytes; };  // bytes a multiple of 16
 void launch_zero_batch(const ZeroArgs* tab, int count, size_t max_bytes, cudaStream_t s);
 
