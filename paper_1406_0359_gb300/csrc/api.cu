@@ -498,7 +498,7 @@ template <typename T> class OpImpl : public purify_op {
     }
     if (!refine && (rc = alloc(&perm, M))) return rc;
     if ((rc = alloc(&gridA, size_t(n) * (g.K / 2)))) return rc;  // half-spectrum rows
-    if (!light && (rc = alloc(&gridP, grid_cells()))) return rc;
+    if (!light && ((rc = alloc(&gridP, grid_cells())) || (rc = alloc(&gram_y, size_t(M))))) return rc;
     if ((rc = alloc(&gridQ, grid_cells()))) return rc;
     if ((rc = alloc(&sc, kNumScalars))) return rc;
     if ((rc = alloc(&err, 2))) return rc;  // [0] timed-out wait, [1] non-finite input
@@ -669,9 +669,7 @@ template <typename T> class OpImpl : public purify_op {
     });
     col_inv(s);
   }
-  // The NUFFT form's visibilities, allocated on its first use.
-  int ensure_gram() { return gram_y ? PURIFY_OK : alloc(&gram_y, size_t(g.M)); }
-  C* gram_y = nullptr;
+  C* gram_y = nullptr;  // the NUFFT form's visibilities (taken at creation: its first call may be captured)
   void row_ep(const RowEp<T>& ep, cudaStream_t s) {
     const RowInvArgs<T> a = row_inv_args(gridA, deapod, ep);
     if (rec) record(R_RI, s).ri = a;
@@ -764,8 +762,10 @@ template <typename T> class OpImpl : public purify_op {
 
   int gram(const void* x, void* out, int mode, cudaStream_t s) override {
     if (mode != 0 && mode != 1) return PURIFY_ERR_INVALID;
-    const int rc = mode == 1 ? ensure_toeplitz(s) : ensure_gram();
-    if (rc) return rc;
+    if (mode == 1) {
+      const int rc = ensure_toeplitz(s);
+      if (rc) return rc;
+    }
     toep = mode == 1;
     normal_front(plain(static_cast<const T*>(x)), s);
     RowEp<T> ep{};
@@ -1159,7 +1159,7 @@ template <typename T> class OpImpl : public purify_op {
       if (!(e > 0)) return PURIFY_ERR_INVALID;
     CK(cudaMemcpyAsync(eps_dev, run.eps_b.data(), nblocks * sizeof(double), cudaMemcpyHostToDevice, s));
     const int gmode = P->gram < 0 ? (g.n <= 1024 ? 1 : 0) : P->gram;
-    if ((rc = gmode == 1 ? ensure_toeplitz(s) : ensure_gram())) return rc;
+    if (gmode == 1 && (rc = ensure_toeplitz(s))) return rc;
     toep = gmode == 1;
     launch_gather<C>(static_cast<const C*>(y), perm, M, ys, s);
     launch_check_finite<T>(reinterpret_cast<const T*>(ys), 2 * M, err + 1, s);
