@@ -32,7 +32,7 @@ UNIT = "iters/s"
 WORKLOAD = "large_1024"
 # DRAM bytes (read + write) per launch from the committed ncu capture of each
 # kernel at this workload (profiles/); kernels changed since have no entry.
-MEASURED_TRAFFIC = {"col_conv": 16.84224e6 + 0.0}
+MEASURED_TRAFFIC = {"col_conv": 16.849408e6}
 
 
 # ----------------------------------------------------------------- helpers
@@ -134,7 +134,7 @@ def workload_string(name: str, w) -> str:
 
 def algorithmic_bytes(kind: str, n: int, M: int, rsize: int = 4, levels: int = 4, cg: int = 10) -> float:
     """Bytes each kernel kind must move per launch (FP32: 4-byte reals, 8-byte
-    complex).  N = n^2 pixels; the oversampled grid holds 4N complex cells.
+    complex).  N = n^2 pixels; the oversampled half grid holds 2N complex cells.
     The SARA sets count one launch set (all levels) in their SDMM form:
     analysis with the l1 prox (x in; z_1, w in, z_1 and 2r - v out for the
     9N coefficients; LL scratch bands out and in level by level), synthesis
@@ -146,13 +146,13 @@ def algorithmic_bytes(kind: str, n: int, M: int, rsize: int = 4, levels: int = 4
     table = {
         "sara_analysis": N * rsize + 9 * N * 4 * rsize + 2 * band * rsize,
         "sara_synthesis": 9 * N * rsize + 2 * band * rsize + 4 * N * rsize,
-        "gram": 4 * N * c * 2 + 8 * M,          # read grid, write grid accumulator, read positions
-        "degrid": 4 * N * c + 8 * M + 3 * c * M,  # grid + positions + (z read, y read, z write)
-        "grid": 4 * N * c + 8 * M + 3 * c * M,    # grid write + positions + (z, y read, z write)
+        "gram": 2 * N * c * 2 + 8 * M,          # read grid, write grid accumulator, read positions
+        "degrid": 2 * N * c + 8 * M + 3 * c * M,  # grid + positions + (z read, y read, z write)
+        "grid": 2 * N * c + 8 * M + 3 * c * M,    # grid write + positions + (z, y read, z write)
         # Phi / Phi^H in real form: half-spectrum rows n x n complex
         "row_fwd": N * rsize + N * c,             # image in, half-spectrum rows out
-        "col_fwd": N * c + 4 * N * c,             # half-spectrum rows in, full grid out
-        "col_inv": 4 * N * c + N * c,             # accumulator in, half-spectrum rows out
+        "col_fwd": N * c + 2 * N * c,             # half-spectrum rows in, half grid out
+        "col_inv": 2 * N * c + N * c,             # accumulator in, half-spectrum rows out
         "row_inv": N * c + 2 * N * rsize,         # half-spectrum rows in, image in/out (epilogue)
         # convolution form (real image, half spectra n x n complex), averaged
         # over the cg + 1 launches per SDMM iteration: the CG's first forward
@@ -278,10 +278,11 @@ def run_ours(args, ws, rank, local):
     pair_ms = e0.elapsed_time(e1) / reps
     vis_per_s = M / (pair_ms / 1e3)
     # bytes of one Phi + Phi^H pair: the staged count (every pass's reads and
-    # writes, FP32: Phi 196N + 16M, Phi^H 204N + 16M) and the compulsory one
-    # (image in and out, uv positions and visibilities once: 2 (4N + 16M))
+    # writes, FP32: Phi 52N + 16M, Phi^H 68N + 16M with the accumulator's
+    # zeroing) and the compulsory one (image in and out, uv positions and
+    # visibilities once: 2 (4N + 16M))
     N = n * n
-    pair_bytes = {"staged": float(400 * N + 32 * M), "compulsory": float(8 * N + 32 * M)}
+    pair_bytes = {"staged": float(120 * N + 32 * M), "compulsory": float(8 * N + 32 * M)}
     pair_gbs = {k: round(v / (pair_ms / 1e3) / 1e9, 1) for k, v in pair_bytes.items()}
 
     # end to end through the public API from pinned host buffers

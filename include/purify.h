@@ -335,8 +335,8 @@ int purify_batch_solve(int count, purify_op* const* ops, const void* const* y, c
  *   precision, n, M, dictionary size, blocks, round, iteration counters,
  *   convergence state, nu, gamma, the first reweighting delta, the last
  *   objective) followed by x_hat, sum_i x_i, z_1, z_2, the SARA weights W and
- *   z_3 (reals of the operator's precision; z_3 in the operator's sorted
- *   visibility order).  CG vectors are not state: every SDMM iteration
+ *   z_3 (reals of the operator's precision; z_3 in the order of a stable
+ *   sort by (block, uv tile, cell) over the whole grid).  CG vectors are not state: every SDMM iteration
  *   restarts its CG from x_hat.
  * purify_solve_load -- after purify_solve_begin with the same y and
  *   parameters, replace the fresh state by a saved one; the next

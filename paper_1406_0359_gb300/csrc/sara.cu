@@ -4,8 +4,8 @@
 // increasing basis order (Dirac first).
 //
 // Analysis (Psi^H): one launch per wavelet level covers all selected
-// Daubechies filters (blockIdx.z = filter slot).  A CTA stages its periodic input tile once in
-// shared memory, filters the rows (axis 1) into low/high halves, then the
+// Daubechies filters (blockIdx.z = filter slot; the first level's also the Dirac
+// block).  A CTA stages its periodic input tile once in shared memory, filters the rows (axis 1) into low/high halves, then the
 // columns (axis 0), and writes the three detail sub-bands of the level to their
 // Mallat positions; the low-low band goes to a scratch band for the next level
 // (or to its final place at the last level).  Convention, per axis:

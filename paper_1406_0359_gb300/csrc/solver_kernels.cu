@@ -1,7 +1,8 @@
 // Small vector kernels of the SDMM solver (Algorithm 1) and the SARA
-// reweighting: the last CG update, deterministic finalisation of device
-// scalars from compensated per-block partials (the l2-ball scales, the
-// objective, norms), visibility permutation and the reweighting rule.
+// reweighting: the last CG update, finalisation of device scalars from
+// compensated per-block partials (the objective, the l2-ball scales of several
+// blocks) or FP64 accumulators (one block), visibility permutation and the
+// reweighting rule.
 #include "internal.h"
 #include "solver_kernels.h"
 
