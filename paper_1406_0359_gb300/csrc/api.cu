@@ -1161,6 +1161,9 @@ template <typename T> class OpImpl : public purify_op {
     const int gmode = P->gram < 0 ? (g.n <= 1024 ? 1 : 0) : P->gram;
     if (gmode == 1 && (rc = ensure_toeplitz(s))) return rc;
     toep = gmode == 1;
+    // the flag speaks of this y alone: a begin that failed beside this operator's
+    // (a batch) may have left an earlier y's unread
+    CK(cudaMemsetAsync(err + 1, 0, sizeof(int), s));
     launch_gather<C>(static_cast<const C*>(y), perm, M, ys, s);
     launch_check_finite<T>(reinterpret_cast<const T*>(ys), 2 * M, err + 1, s);
     run.nu = P->nu;
