@@ -1868,8 +1868,11 @@ int batch_solve(int count, purify_op* const* ops_in, const void* const* y, const
       OpImpl<T>* o = b.ops[i];
       const int rc = part == 0 ? o->begin_front(y[i], &P, user) : (part == 1 ? o->begin_gamma() : o->begin_round());
       if (rc) {
-        for (OpImpl<T>* q : b.ops) {
+        // the instances begun so far (an operator not reached keeps what it was doing)
+        for (int j = 0; j < (part == 0 ? i + 1 : count); ++j) {
+          OpImpl<T>* q = b.ops[j];
           cudaStreamSynchronize(q->own);  // nothing left running that reads the caller's arrays
+          cudaMemset(q->err, 0, sizeof(int));  // a wait that gave up in its set-up: this call has failed already
           q->run_release();
         }
         return rc;

@@ -46,3 +46,25 @@ def test_every_operator_solves_good_data_after_several_bad_instances(bad):
     for op, y, eps_k, a in zip(ops, ys, eps, alone):
         assert rel(host(op.solve(y, eps_k, t_max=3, cg_iters=3).x), host(a.x)) < 1e-5
         op.close()
+
+
+@pytest.mark.parametrize("reached", [1, 2])
+def test_solve_in_progress_on_an_unreached_operator_goes_on(reached):
+    """Instance reached - 1 is refused for its bound; the operators after it
+    have a solve begun and part way, which finishes as if undisturbed."""
+    from paper_1406_0359_gb300.binding import PurifyError, batch_solve
+
+    ps = problems(3)
+    ops, ys, eps = [list(c) for c in zip(*ps)]
+    alone = [op.solve(y, e, t_max=4, cg_iters=3) for op, y, e in ps]
+    for op, y, e in ps[reached:]:
+        op.solve_begin(y, e, t_max=4, cg_iters=3)
+        assert not op.solve_step(2)
+    with pytest.raises(PurifyError) as err:
+        batch_solve(ops, ys, [0.0 if k == reached - 1 else e for k, e in enumerate(eps)], t_max=4, cg_iters=3)
+    assert err.value.code == -1
+    for (op, y, e), a in list(zip(ps, alone))[reached:]:
+        assert op.solve_step(2)
+        assert rel(host(op.solve_end().x), host(a.x)) < 1e-5
+    for op in ops:
+        op.close()
