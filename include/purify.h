@@ -289,7 +289,8 @@ int purify_sdmm_solve(purify_op* op, const void* y, const purify_params* params,
 /*
  * purify_batch_solve -- many independent SARA solves (Eq. 3 by Algorithm 1,
  * as purify_sdmm_solve; e.g. frequency channels or fields) advanced
- * together.  Instances are grouped by image side; within a group every pass
+ * together.  Instances are grouped by image side, wavelet levels and
+ * dictionary; within a group every pass
  * of an SDMM iteration (CG passes, degridding, gridding, projections, SARA
  * levels, vector steps) is one kernel launch over all of the group's
  * instances, reading each instance's arguments from a device table, and one
@@ -297,7 +298,7 @@ int purify_sdmm_solve(purify_op* op, const void* y, const purify_params* params,
  * groups run side by side.
  *   count   number of instances (>= 1).
  *   ops     count distinct operators of one precision, image sides 64..1024,
- *           one visibility block, the l1 prior (any dictionary).
+ *           one visibility block, the l1 prior (any levels and dictionary).
  *   y       count device pointers, each instance's visibilities (caller order).
  *   params  count parameter sets: each instance's eps, gamma, nu (<= 0:
  *           computed per instance as in purify_sdmm_solve), delta rules; t_max,
@@ -399,7 +400,7 @@ const char* purify_kernel_name(int kind);
  * still running is left alone (no lock-step: a large image never holds back
  * a small one).  A finished solve frees its slot and memory at once.
  * Iteration-level batching (off by default, purify_server_set_batching): admitted solves that share
- * image side, precision, CG steps and dictionary, use the convolution form of
+ * image side, wavelet levels, precision, CG steps and dictionary, use the convolution form of
  * the CG operator (64 <= n <= 1024) and one visibility block advance together
  * -- one SDMM iteration of all of them is one batched graph, each pass one
  * launch over the group as in purify_batch_solve, cached while the group's

@@ -1262,13 +1262,18 @@ template <typename T> class OpImpl : public purify_op {
     return PURIFY_OK;
   }
 
+  // Image side, wavelet levels and dictionary: what solves whose SARA passes
+  // are one launch have in common (28 bits).
+  uint64_t sara_key() const {
+    return uint64_t(g.n) | (uint64_t(levels) << 12) | (uint64_t(dictionary(nullptr)) << 16);
+  }
   // ---- iteration-level batching in the request server: the solves of one
-  // key (image side, precision, CG steps, dictionary) advance together
+  // key (sara_key, precision, CG steps) advance together
   // through a batched graph; these hooks do each solve's part around it.
   uint64_t batch_key() const override {
     if (!run.active || !toep || prior != 0 || nblocks != 1 || g.n < 64 || g.n > 1024 || prof) return 0;
-    return uint64_t(g.n) | (uint64_t(sizeof(T) == 4 ? 1 : 2) << 12) | (uint64_t(run.P.cg_iters) << 16) |
-           (uint64_t(dictionary(nullptr)) << 32);
+    if (run.P.cg_iters > 0xFFFF) return 0;
+    return sara_key() | (uint64_t(sizeof(T) == 4 ? 1 : 2) << 28) | (uint64_t(run.P.cg_iters) << 32);
   }
   int prepare_iteration(cudaStream_t s) override {
     if (!run.active) return PURIFY_ERR_INVALID;
@@ -1596,7 +1601,7 @@ template <typename T> class OpImpl : public purify_op {
 // ---------------------------------------------------------------------------
 // Batched solver: many independent SARA-SDMM instances (different images, uv
 // coverages and visibility counts) advanced together.  Instances are grouped
-// by image side; for each group every pass of an SDMM iteration -- the CG
+// by image side, wavelet levels and dictionary; for each group every pass of an SDMM iteration -- the CG
 // passes, the ball block, the SARA blocks, the vector steps -- is ONE launch
 // over all of the group's instances, its arguments read from a device table
 // (one entry per instance, recorded from each instance's own iteration so
@@ -1645,7 +1650,7 @@ template <typename T> class BatchImpl {
     if (bs) cudaStreamDestroy(bs);
   }
 
-  // Record every instance's iteration, group by image side, upload the tables.
+  // Record every instance's iteration, group them, upload the tables.
   int build() {
     CK(cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&ev0, cudaEventDisableTiming));
@@ -1656,13 +1661,15 @@ template <typename T> class BatchImpl {
       o->iteration(o->run.nu, o->run.gamma, o->run.P.eps, o->run.P.cg_iters, o->own);
       o->rec = nullptr;
     }
-    std::map<int, int> gid;
+    // one group per image side, wavelet levels and dictionary: the SARA launches
+    // of a group share their filters, levels and grids
+    std::map<uint64_t, int> gid;
     for (size_t i = 0; i < ops.size(); ++i) {
-      auto it = gid.find(ops[i]->g.n);
+      const uint64_t key = ops[i]->sara_key();
+      auto it = gid.find(key);
       if (it == gid.end()) {
-        gid[ops[i]->g.n] = int(groups.size());
+        it = gid.emplace(key, int(groups.size())).first;
         groups.emplace_back();
-        it = gid.find(ops[i]->g.n);
       }
       groups[it->second].idx.push_back(int(i));
     }
@@ -1673,9 +1680,9 @@ template <typename T> class BatchImpl {
         gr.branches.push_back(r.branch);
       }
       for (int i : gr.idx) {
-        if (recs[i].size() != r0.size()) return invalid("instances of one image side differ in their passes");
+        if (recs[i].size() != r0.size()) return invalid("instances of one group differ in their passes");
         for (size_t k = 0; k < r0.size(); ++k)
-          if (recs[i][k].kind != r0[k].kind) return invalid("instances of one image side differ in their passes");
+          if (recs[i][k].kind != r0[k].kind) return invalid("instances of one group differ in their passes");
         gr.max_items = std::max(gr.max_items, ops[i]->n_items);
         gr.max_tb = std::max(gr.max_tb, ops[i]->g.TB);
         gr.max_q = std::max(gr.max_q, ops[i]->grid_bytes());

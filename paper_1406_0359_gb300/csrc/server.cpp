@@ -13,7 +13,7 @@
 // the next request can take its slot.
 //
 // Iteration-level batching (off by default): solves that share a batch key
-// (image side, precision, CG steps, dictionary; the convolution form of the
+// (image side, levels, precision, CG steps, dictionary; the convolution form of the
 // CG operator) and are between iterations advance together -- one SDMM
 // iteration of all of them is one batched graph (each pass one launch over
 // the group, see purify_batch_solve) on the group's own stream, cached for
