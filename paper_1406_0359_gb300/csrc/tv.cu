@@ -13,9 +13,10 @@
 //     q <- P(q + tau grad(v + div q)),  tau = 1/8,
 // a fixed number per SDMM iteration, warm-started from the previous
 // iteration's q (zero at the start of each round).  A step needs its
-// neighbours' previous q, so a launch takes kTvSteps of them on tiles with a
-// halo as wide, in shared memory, ping-ponging between two dual buffers from
-// launch to launch; the last launch's epilogue forms r_1 = v + div q, updates
+// neighbours' previous q: large FP32 images take kTvSteps of them a launch on
+// tiles with a halo as wide, in shared memory; other images one a launch
+// (tv_fused).  Both ping-pong between two dual buffers from launch to launch
+// and leave the dual in the first; the epilogue forms r_1 = v + div q, updates
 // z_1, applies the positivity block (f_2, L_2 = I) and writes x_1 + x_2, with the
 // objective's partial sums TV_w(x_hat).
 #include "internal.h"
@@ -51,10 +52,9 @@ template <typename T> struct TvArgs {
   T* xs;
   double* partials;
 };
-// The halo makes a tile 1.9 times its pixels' work, but a step in shared memory
-// costs two barriers where a launch per step cost 4.1 us (22 launches at 20 steps,
-// now 4; the TV solve at 512^2 5.41 -> 5.30 ms, where the ball block beside it is
-// the longer branch).
+// The halo makes a tile 1.9 times its pixels' work, but a step costs two barriers
+// in place of a launch and a pass over memory (the TV solve at 512^2, 20 steps an
+// iteration, 5.41 -> 5.30 ms, where the ball block beside it is the longer branch).
 template <typename T> __global__ void __launch_bounds__(kTvT) k_tv_steps(TvArgs<T> a) {
   __shared__ T q1[kTvR * kTvR], q2[kTvR * kTvR], ds[kTvR * kTvR];
   __shared__ double red[32];
@@ -148,6 +148,91 @@ template <typename T> __global__ void __launch_bounds__(kTvT) k_tv_steps(TvArgs<
   }
 }
 
+// ---- one launch per step and pixel, where that is the faster form (tv_fused)
+// d = v + div q at (i, j) (q1 plane first, then q2; n x n each).
+template <typename T> PD T dval(const T* __restrict__ v, const T* __restrict__ q, int n, int i, int j) {
+  const size_t N = size_t(n) * n, k = size_t(i) * n + j;
+  const T* q1 = q;
+  const T* q2 = q + N;
+  T d = v[k];
+  if (i < n - 1) d += q1[k];
+  if (i > 0) d -= q1[k - n];
+  if (j < n - 1) d += q2[k];
+  if (j > 0) d -= q2[k - 1];
+  return d;
+}
+
+// One projected-gradient step of the dual per launch: qo = P(qi + tau grad(v + div qi)),
+// P the pixelwise projection onto |q_ij| <= gamma w_ij.
+template <typename T>
+__global__ void __launch_bounds__(kTvT) k_tv_dual_step(const T* __restrict__ v, const T* __restrict__ w, T gamma,
+                                                       const T* __restrict__ qi, T* __restrict__ qo, int n) {
+  const size_t N = size_t(n) * n;
+  const size_t k = size_t(blockIdx.x) * kTvT + threadIdx.x;
+  if (k >= N) return;
+  const int i = int(k / n), j = int(k - size_t(i) * n);
+  const T d = dval(v, qi, n, i, j);
+  const T g1 = i < n - 1 ? dval(v, qi, n, i + 1, j) - d : T(0);
+  const T g2 = j < n - 1 ? dval(v, qi, n, i, j + 1) - d : T(0);
+  const T tau = T(0.125);
+  T a = fma(tau, g1, qi[k]), b = fma(tau, g2, qi[k + N]);
+  const T bound = gamma * (w ? w[k] : T(1));
+  const T m = sqrt(a * a + b * b);
+  if (m > bound) {
+    const T s = bound / m;
+    a *= s;
+    b *= s;
+  }
+  qo[k] = a;
+  qo[k + N] = b;
+}
+
+// v_1 = x_hat + z_1 (the TV block's input).
+template <typename T>
+__global__ void __launch_bounds__(kTvT) k_tv_input(const T* __restrict__ xh, const T* __restrict__ z1,
+                                                   T* __restrict__ v, size_t N) {
+  const size_t k = size_t(blockIdx.x) * kTvT + threadIdx.x;
+  if (k < N) v[k] = xh[k] + z1[k];
+}
+
+// Epilogue: r_1 = v + div q, z_1 = v - r_1, x_1 = 2 r_1 - v; positivity block
+// v_2 = x_hat + z_2, r_2 = max(v_2, 0), z_2 = v_2 - r_2; xs = x_1 + 2 r_2 - v_2;
+// per-CTA partials of TV_w(x_hat).  With qcopy set the final dual is also
+// written back to the buffer the next iteration starts from.
+template <typename T>
+__global__ void __launch_bounds__(kTvT) k_tv_epilogue(const T* __restrict__ v, const T* __restrict__ q,
+                                                      T* __restrict__ qcopy, const T* __restrict__ xh,
+                                                      const T* __restrict__ w, T* __restrict__ z1,
+                                                      T* __restrict__ z2, T* __restrict__ xs, double* partials,
+                                                      int n) {
+  __shared__ double red[32];
+  const size_t N = size_t(n) * n;
+  const size_t k = size_t(blockIdx.x) * kTvT + threadIdx.x;
+  Acc<T> part;
+  if (k < N) {
+    const int i = int(k / n), j = int(k - size_t(i) * n);
+    const T vk = v[k];
+    const T r1 = dval(v, q, n, i, j);
+    z1[k] = vk - r1;
+    const T v2 = xh[k] + z2[k];
+    const T r2 = v2 > T(0) ? v2 : T(0);
+    z2[k] = v2 - r2;
+    xs[k] = (T(2) * r1 - vk) + (T(2) * r2 - v2);
+    if (qcopy) {
+      qcopy[k] = q[k];
+      qcopy[k + N] = q[k + N];
+    }
+    const T x0 = xh[k];
+    const T g1 = i < n - 1 ? xh[k + n] - x0 : T(0);
+    const T g2 = j < n - 1 ? xh[k + 1] - x0 : T(0);
+    part.add(sqrt(g1 * g1 + g2 * g2) * (w ? w[k] : T(1)));
+  }
+  if (partials) {
+    const Acc<T> t = block_merge<kTvT>(part, red);
+    if (threadIdx.x == 0) reinterpret_cast<Acc<T>*>(partials)[blockIdx.x] = t;
+  }
+}
+
 // |grad x| per pixel (RWTV weights and their delta).
 template <typename T>
 __global__ void __launch_bounds__(kTvT) k_tv_magnitude(const T* __restrict__ x, T* __restrict__ out, int n) {
@@ -163,13 +248,37 @@ __global__ void __launch_bounds__(kTvT) k_tv_magnitude(const T* __restrict__ x, 
 
 inline int tv_blocks(int n) { return int((size_t(n) * n + kTvT - 1) / kTvT); }
 inline int tv_tiles(int n) { return (n + kTvTile - 1) / kTvTile; }
+// Whether the steps go kTvSteps a launch.  The halo makes 1.9 times the work
+// on tiles that are few on small images, and a launch per step costs only 1.9 us
+// inside a graph; FP64 is bound by its units whatever the size.  An SDMM
+// iteration with 100 dual steps, one a launch against five: FP32 64^2 293 / 376
+// us, 256^2 318 / 404, 512^2 479 / 482 (20 steps 239 / 232), 1024^2 1171 / 1072,
+// 2048^2 7742 / 6828; FP64 64^2 848 / 1899, 512^2 4002 / 5746.
+template <typename T> constexpr bool tv_fused(int n) { return sizeof(T) == 4 && n >= 512; }
 
 }  // namespace
 
-int tv_partials(int n) { return tv_tiles(n) * tv_tiles(n); }
+int tv_partials(int n) { return tv_blocks(n) > tv_tiles(n) * tv_tiles(n) ? tv_blocks(n) : tv_tiles(n) * tv_tiles(n); }
 
-template <typename T>
-int tv_block(const TvBlock<T>& b, cudaStream_t s) {
+// One launch per step: an odd number of them leaves the dual in qb, from where
+// the epilogue copies it back to qa.
+template <typename T> static int tv_single_steps(const TvBlock<T>& b, cudaStream_t s) {
+  const int n = b.n, nb = tv_blocks(n);
+  k_tv_input<T><<<nb, kTvT, 0, s>>>(b.xh, b.z1, b.v, size_t(n) * n);
+  const T* qi = b.qa;
+  T* qo = b.qb;
+  for (int it = 0; it < b.iters; ++it) {
+    k_tv_dual_step<T><<<nb, kTvT, 0, s>>>(b.v, b.w, T(b.gamma), qi, qo, n);
+    const T* t = qo;
+    qo = const_cast<T*>(qi);
+    qi = t;
+  }
+  k_tv_epilogue<T><<<nb, kTvT, 0, s>>>(b.v, qi, (b.iters & 1) ? b.qa : nullptr, b.xh, b.w, b.z1, b.z2, b.xs,
+                                       b.partials, n);
+  return nb;
+}
+
+template <typename T> static int tv_fused_steps(const TvBlock<T>& b, cudaStream_t s) {
   const int nt = tv_tiles(b.n);
   // an even number of launches, so that the dual leaves in the buffer it came in
   const int launches = 2 * ((b.iters + 2 * kTvSteps - 1) / (2 * kTvSteps));
@@ -185,6 +294,13 @@ int tv_block(const TvBlock<T>& b, cudaStream_t s) {
     a.qi = t;
   }
   return nt * nt;
+}
+
+template <typename T> int tv_block(const TvBlock<T>& b, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4) {
+    if (tv_fused<T>(b.n)) return tv_fused_steps(b, s);
+  }
+  return tv_single_steps(b, s);
 }
 
 template <typename T> void tv_magnitude(const T* x, T* out, int n, cudaStream_t s) {
