@@ -439,8 +439,13 @@ template <typename T> class OpImpl : public purify_op {
     // default work-item length by M: a warp walks an item alone, so short
     // items spread a small M over the chip (256^2 / 131072: Phi^H 29 us at 128,
     // 33 at 256, 50 at 1024) and end a large one together (512^2 / 4M: 110 at
-    // 256..1024, 149 at 2048; 1024^2 / 4M: 150..154 at 256..2048)
-    chunk = chunk_opt > 0 ? chunk_opt : (M < (int64_t(1) << 20) ? 128 : 512);
+    // 256..1024, 149 at 2048; 1024^2 / 4M: 150..154 at 256..2048).  FP64 takes
+    // about 10 us for each 32 visibilities of an item's walk: half as long below
+    // 2^18, where the items do not fill the chip (NUFFT-form Phi^H Phi at 32^2 /
+    // 512 points 99 us at 64, 146 at 128; 256^2 / 131072 262 / 280; 512^2 /
+    // 393217 728 / 720).
+    const int64_t half = sizeof(T) == 8 ? int64_t(1) << 18 : 0;
+    chunk = chunk_opt > 0 ? chunk_opt : (M < half ? 64 : (M < (int64_t(1) << 20) ? 128 : 512));
     if (!light) {  // a set-up operator runs only on the caller's stream
       // the ball block is the longer branch of an iteration: its kernels'
       // CTAs go first when several branches have work waiting, then the
