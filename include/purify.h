@@ -221,7 +221,10 @@ int purify_op_set_blocks(purify_op* op, const int* block_ids, int R, void* strea
  * purify_gram -- out = Re(Phi^H Phi x), the data term of the composite
  * operator sum_i L_i^H L_i = Phi^H Phi + 2I that the SDMM global update
  * inverts (Section 3).
- *   mode 0: Phi then Phi^H through the NUFFT (degridding and gridding fused).
+ *   mode 0: Phi then Phi^H through the NUFFT, the visibilities in between in
+ *           the operator's sorted order.  The first call (or solve in this
+ *           form) takes M complex values of operator memory and keeps them; it
+ *           may be made inside a stream capture.
  *   mode 1: the composite precomputed once, as Section 3 suggests: the PSF
  *           k(d) = sum_m exp(i (u_m d1 + v_m d2)) over offsets d in [-n, n)^2
  *           (from the NUFFT adjoint of unit visibilities on a 2n x 2n image)

@@ -503,7 +503,7 @@ template <typename T> class OpImpl : public purify_op {
     }
     if (!refine && (rc = alloc(&perm, M))) return rc;
     if ((rc = alloc(&gridA, size_t(n) * (g.K / 2)))) return rc;  // half-spectrum rows
-    if (!light && ((rc = alloc(&gridP, grid_cells())) || (rc = alloc(&gram_y, size_t(M))))) return rc;
+    if (!light && (rc = alloc(&gridP, grid_cells()))) return rc;
     if ((rc = alloc(&gridQ, grid_cells()))) return rc;
     if ((rc = alloc(&sc, kNumScalars))) return rc;
     if ((rc = alloc(&err, 2))) return rc;  // [0] timed-out wait, [1] non-finite input
@@ -674,7 +674,18 @@ template <typename T> class OpImpl : public purify_op {
     });
     col_inv(s);
   }
-  C* gram_y = nullptr;  // the NUFFT form's visibilities (taken at creation: its first call may be captured)
+  C* gram_y = nullptr;  // the NUFFT form's visibilities, from its first use on (most operators never take it)
+  // That first use may be inside a stream capture, where the calling thread may
+  // not allocate: the buffer comes on the operator's own stream, which no
+  // capture includes, with the thread's capture mode relaxed for the moment.
+  int ensure_gram() {
+    if (gram_y) return PURIFY_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    const int rc = alloc(&gram_y, size_t(g.M));
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return rc;
+  }
   void row_ep(const RowEp<T>& ep, cudaStream_t s) {
     const RowInvArgs<T> a = row_inv_args(gridA, deapod, ep);
     if (rec) record(R_RI, s).ri = a;
@@ -767,10 +778,8 @@ template <typename T> class OpImpl : public purify_op {
 
   int gram(const void* x, void* out, int mode, cudaStream_t s) override {
     if (mode != 0 && mode != 1) return PURIFY_ERR_INVALID;
-    if (mode == 1) {
-      const int rc = ensure_toeplitz(s);
-      if (rc) return rc;
-    }
+    const int rc = mode == 1 ? ensure_toeplitz(s) : ensure_gram();
+    if (rc) return rc;
     toep = mode == 1;
     normal_front(plain(static_cast<const T*>(x)), s);
     RowEp<T> ep{};
@@ -1164,7 +1173,7 @@ template <typename T> class OpImpl : public purify_op {
       if (!(e > 0)) return PURIFY_ERR_INVALID;
     CK(cudaMemcpyAsync(eps_dev, run.eps_b.data(), nblocks * sizeof(double), cudaMemcpyHostToDevice, s));
     const int gmode = P->gram < 0 ? (g.n <= 1024 ? 1 : 0) : P->gram;
-    if (gmode == 1 && (rc = ensure_toeplitz(s))) return rc;
+    if ((rc = gmode == 1 ? ensure_toeplitz(s) : ensure_gram())) return rc;
     toep = gmode == 1;
     // the flag speaks of this y alone: a begin that failed beside this operator's
     // (a batch) may have left an earlier y's unread

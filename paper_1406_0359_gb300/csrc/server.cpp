@@ -105,9 +105,9 @@ extern "C" int purify_estimate_bytes(int64_t M, int n, int dwt_levels, int preci
     b += M * (2 * r + 4 + 16) + n2 * K2 * c + 2 * KP2 * KP2 * c + 2 * 8 * (N2 / 4) * r + 9 * N2 * r;
     b += M * c + K * K * (r + c);
   }
-  // every operator also keeps M sorted visibilities for the NUFFT form: covered
-  // by the grids counted whole above (only half of each exists) and, up to
-  // n = 1024, by the composite's transients
+  // a solve in the NUFFT form (every one above n = 1024) also keeps M sorted
+  // visibilities: covered by the grids counted whole above (only half of each
+  // exists) and, up to n = 1024, by the composite's transients
   else if (M > 4 * N) {
     b += (M - 4 * N) * c;
   }
