@@ -309,6 +309,8 @@ int purify_sdmm_solve(purify_op* op, const void* y, const purify_params* params,
  *           CG operator is the precomputed convolution form (gram 0 refused).
  *   x_out   count device pointers, real[n_i][n_i].
  *   stats   host, count entries, may be NULL.
+ * The instances' set-ups run side by side as far as their scratch (see
+ * purify_op_create) stays within 256 MiB, or the largest instance's alone.
  * Each instance's result equals its purify_sdmm_solve up to rounding (the
  * gridding atomics and the order of partial sums).  Blocks until done;
  * PURIFY_ERR_INVALID (purify_last_error says which rule) for instances the

@@ -740,6 +740,16 @@ template <typename T> class OpImpl : public purify_op {
     return PURIFY_OK;
   }
 
+  // Set-up pool bytes that ensure_toeplitz holds until its kernels have run: the
+  // 2n operator's positions and grids, the unit visibilities, the PSF and its
+  // spectrum (and, where this binning does not serve, a binning's scratch).
+  size_t toeplitz_scratch() const {
+    const size_t M = size_t(g.M), n2 = 2 * size_t(g.n), K2 = 2 * n2;
+    size_t b = M * (sizeof(Pos<T>) + sizeof(C)) + n2 * n2 * (sizeof(T) + sizeof(C));
+    b += (n2 * n2 + (K2 + kJ) * (n2 + kJ)) * sizeof(C) + size_t(n_items) * (sizeof(WorkItem) + 4 * sizeof(double));
+    return g.TB == 8 ? b : b + M * (4 * sizeof(int));
+  }
+
   // Front half of Re(Phi^H Phi) x: up to the half-spectrum rows in gridA, by the
   // NUFFT (G^H G per application) or by the precomputed convolution.
   // (The convolution form may run in the half-spectrum buffer `B` instead,
@@ -1859,6 +1869,9 @@ template <typename T> int batch_graph_build(purify_op* const* ops, int count, cu
 // stream), record and capture the batched iteration, then run the rounds in
 // lock step -- the round set-ups per instance, the iterations as graph
 // replays -- and end every instance.
+// Set-up scratch that a batch's instances may hold at once (16 of 256^2 / 131072
+// points, say; the set-up pool keeps four times as much mapped).
+constexpr size_t kBatchScratch = size_t(256) << 20;
 template <typename T>
 int batch_solve(int count, purify_op* const* ops_in, const void* const* y, const purify_params* params,
                 void* const* x_out, purify_stats* stats, cudaStream_t user) {
@@ -1880,14 +1893,38 @@ int batch_solve(int count, purify_op* const* ops_in, const void* const* y, const
     b.ops.push_back(o);
   }
   // every instance's set-up (its CG operator, nu, gamma, state) on its own stream
-  // (part by part, so that the instances' power iterations run side by side)
+  // (part by part, so that the instances' power iterations run side by side).
+  // The CG operators' scratch in flight stays within kBatchScratch or the
+  // largest instance's alone: beyond that an instance's set-up comes after an
+  // earlier one's, whose memory it takes over.
+  size_t limit = kBatchScratch, in_flight = 0;
+  std::vector<std::pair<int, size_t>> held;  // (instance, bytes), oldest first from `oldest` on
+  size_t oldest = 0;
+  for (OpImpl<T>* o : b.ops)
+    if (!o->khat) limit = std::max(limit, o->toeplitz_scratch());
+  auto cg_operator = [&](int i) -> int {
+    OpImpl<T>* o = b.ops[i];
+    if (o->khat) return PURIFY_OK;
+    const size_t need = o->toeplitz_scratch();
+    for (; oldest < held.size() && in_flight + need > limit; ++oldest) {
+      CK(cudaStreamWaitEvent(o->own, b.ops[held[oldest].first]->ev_out, 0));
+      in_flight -= held[oldest].second;
+    }
+    const int rc = o->ensure_toeplitz(o->own);
+    if (rc) return rc;
+    CK(cudaEventRecord(o->ev_out, o->own));
+    held.emplace_back(i, need);
+    in_flight += need;
+    return PURIFY_OK;
+  };
   for (int part = 0; part < 3; ++part)
     for (int i = 0; i < count; ++i) {
       purify_params P = params[i];
       P.use_graph = 0;
       P.gram = 1;
       OpImpl<T>* o = b.ops[i];
-      const int rc = part == 0 ? o->begin_front(y[i], &P, user) : (part == 1 ? o->begin_gamma() : o->begin_round());
+      int rc = part == 0 ? cg_operator(i) : PURIFY_OK;
+      if (!rc) rc = part == 0 ? o->begin_front(y[i], &P, user) : (part == 1 ? o->begin_gamma() : o->begin_round());
       if (rc) {
         // the instances begun so far (an operator not reached keeps what it was doing)
         for (int j = 0; j < (part == 0 ? i + 1 : count); ++j) {
