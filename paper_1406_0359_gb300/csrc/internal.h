@@ -39,7 +39,7 @@ template <> struct KbDeg<double> { static constexpr int value = kDegD; };
 template <typename T> struct KbPoly { T c[kJ][KbDeg<T>::value + 1]; };
 
 // Encoded grid position of one visibility inside its uv tile.
-// FP32: 8 integer bits of cell + 24 fraction bits per axis (6e-8 cell resolution).
+// FP32: 7 bits of cell and an offset in [0, 1] in units of 2^-24 per axis.
 // FP64: the tile-local coordinate itself.
 template <typename T> struct Pos;
 template <> struct Pos<float> { uint32_t u, v; };

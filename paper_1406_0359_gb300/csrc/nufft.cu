@@ -25,12 +25,20 @@ namespace purify {
 
 namespace {
 
+// FP32 positions: the cell inside the tile in the top 7 bits, the offset in
+// units of 2^-24 below them, 0 and 1 both included (a mirrored grid node has
+// offset 1).
+constexpr int kOffBits = 24, kCellShift = kOffBits + 1;
+PD uint32_t encode_offset(int cell, double f) {
+  return (uint32_t(cell) << kCellShift) | uint32_t(f * double(1u << kOffBits) + 0.5);
+}
 PD void decode(const Pos<float>& p, int& cu, float& fu, int& cv, float& fv) {
-  const float sc = 1.0f / 16777216.0f;
-  cu = int(p.u >> 24);
-  cv = int(p.v >> 24);
-  fu = float(p.u & 0xFFFFFFu) * sc;
-  fv = float(p.v & 0xFFFFFFu) * sc;
+  constexpr float sc = 1.0f / float(1u << kOffBits);
+  constexpr uint32_t mask = (1u << kCellShift) - 1u;
+  cu = int(p.u >> kCellShift);
+  cv = int(p.v >> kCellShift);
+  fu = float(p.u & mask) * sc;
+  fv = float(p.v & mask) * sc;
 }
 PD void decode(const Pos<double>& p, int& cu, double& fu, int& cv, double& fv) {
   const double a = floor(p.u), b = floor(p.v);
@@ -782,15 +790,9 @@ __global__ void k_encode<float>(const double* __restrict__ uv, const int* __rest
   int cell[2];
   double f[2];
   grid_cells(uv, perm_index(perm[i]), K, true, cell, f);
-  uint32_t e[2];
-  for (int a = 0; a < 2; ++a) {
-    uint32_t q = uint32_t(f[a] * 16777216.0 + 0.5);
-    if (q > 0xFFFFFFu) q = 0xFFFFFFu;
-    e[a] = (uint32_t(cell[a] % TB) << 24) | q;
-  }
   Pos<float> p;
-  p.u = e[0];
-  p.v = e[1];
+  p.u = encode_offset(cell[0] % TB, f[0]);
+  p.v = encode_offset(cell[1] % TB, f[1]);
   pos[i] = p;
 }
 template <>
@@ -829,14 +831,8 @@ __global__ void k_encode_x2(const double* __restrict__ uv, const int* __restrict
   }
   Pos<T> p;
   if constexpr (sizeof(T) == 4) {
-    uint32_t e[2];
-    for (int a = 0; a < 2; ++a) {
-      uint32_t q = uint32_t(fr[a] * 16777216.0 + 0.5);
-      if (q > 0xFFFFFFu) q = 0xFFFFFFu;
-      e[a] = (uint32_t(cell[a]) << 24) | q;
-    }
-    p.u = e[0];
-    p.v = e[1];
+    p.u = encode_offset(cell[0], fr[0]);
+    p.v = encode_offset(cell[1], fr[1]);
   } else {
     p.u = fmin(double(cell[0]) + fr[0], nextafter(double(cell[0] + 1), 0.0));
     p.v = fmin(double(cell[1]) + fr[1], nextafter(double(cell[1] + 1), 0.0));
