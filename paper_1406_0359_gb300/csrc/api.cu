@@ -222,7 +222,7 @@ template <typename T> class OpImpl : public purify_op {
   cudaEvent_t ev_axf = nullptr, ev_axj = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr, ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_zfork = nullptr, ev_zjoin = nullptr;
-  double* bpart = nullptr;     // ball-block partials (2 per work item), apart from the l1 block's
+  double* bpart = nullptr;     // ball-block partials of several visibility blocks (2 per work item)
   int bpart_cap = 0;
   CUtensorMap* tmap_dev = nullptr;  // device copy of tmap (batched degridding reads it there)
 
@@ -257,12 +257,12 @@ template <typename T> class OpImpl : public purify_op {
   int size_partials() {
     const int np = std::max({2 * n_items, sara_partials_capacity(g.n, levels),
                              vec_blocks(9 * N()), tv_partials(g.n), 1});
-    if (2 * n_items > bpart_cap) {
+    if (nblocks > 1 && 2 * n_items > bpart_cap) {
       double* bnew = nullptr;
-      const int rc = alloc(&bnew, size_t(std::max(2 * n_items, 1)));
+      const int rc = alloc(&bnew, size_t(2 * n_items));
       if (rc) return rc;
       bpart = bnew;
-      bpart_cap = std::max(2 * n_items, 1);
+      bpart_cap = 2 * n_items;
     }
     if (np <= partials_cap) return PURIFY_OK;
     double* pnew = nullptr;
@@ -876,8 +876,9 @@ template <typename T> class OpImpl : public purify_op {
 
   // ---- solver
   int ensure_solver() {
-    if (xh) return PURIFY_OK;
     int rc;
+    if ((rc = size_partials())) return rc;  // again if set_blocks ran out of memory on them
+    if (xh) return PURIFY_OK;
     if ((rc = ensure_sara())) return rc;
     const size_t n2 = N();
     if ((rc = alloc(&xh, n2)) || (rc = alloc(&xs, n2)) || (rc = alloc(&r, n2)) || (rc = alloc(&p, n2)) ||
@@ -1054,9 +1055,12 @@ template <typename T> class OpImpl : public purify_op {
     dep.z = z3;
     dep.ys = ys;
     dep.nu = nu;
-    dep.part0 = bpart;
-    dep.part1 = bpart + n_items;
-    dep.acc = nblocks == 1 ? ball_acc : nullptr;
+    if (nblocks == 1) {
+      dep.acc = ball_acc;
+    } else {
+      dep.part0 = bpart;
+      dep.part1 = bpart + n_items;
+    }
     degrid(dep, b3);
     const Ball1Args b1{ball_acc, nu, eps_dev, scale_dev, sc};
     if (rec) record(R_B1, b3).b1 = b1;

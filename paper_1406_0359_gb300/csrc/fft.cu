@@ -517,7 +517,6 @@ PD void row_ep_store(const RowEp<T>& ep, size_t idx, bool al, const T (&val)[V],
       part.a[4].s = fma(b[k], b[k], part.a[4].s);
     } else if constexpr (MODE == EP_CG_R0) {
       o[k] = (a[k] - T(2) * b[k]) - T(ep.nu2) * val[k];
-      sq[k].add_prod(o[k], o[k]);
     } else if constexpr (MODE == EP_POWER) {
       o[k] = val[k];
       sq[k].add_prod(val[k], val[k]);
@@ -907,7 +906,7 @@ PD EpAcc<T> row_ep_rows(const RowEp<T>& ep, const typename cplx_t<T>::type* bufs
     for (int k = 0; k < 5; ++k) acc_merge(run.a[k], part.a[k]);
     return run;
   }
-  if constexpr (MODE == EP_CG_R0 || MODE == EP_POWER) {
+  if constexpr (MODE == EP_POWER) {
 #pragma unroll
     for (int k = 0; k < V; ++k) acc_merge(part.a[0], sq[k]);
   }

@@ -46,3 +46,30 @@ def test_solve_in_the_nufft_form_takes_the_buffer():
     assert rel(host(op.solve(to_dev(P["y"], "fp32"), P["eps"], gram=0, t_max=2, cg_iters=2).x),
                host(op.solve(to_dev(P["y"], "fp32"), P["eps"], gram=1, t_max=2, cg_iters=2).x)) < 1e-4
     op.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_ball_partials_come_with_several_blocks(prec):
+    """One visibility block adds its norms to accumulators; only several blocks
+    keep two partial sums per work item, sized again for every new binning."""
+    from paper_1406_0359_gb300.binding import Operator
+
+    P = measured_problem(64, 9001, 7)
+    op = Operator(torch.as_tensor(P["uv"]).cuda(), 64, 2, prec)
+    y = to_dev(P["y"], prec)
+    kw = dict(t_max=3, cg_iters=3)
+    one = op.solve(y, P["eps"], **kw)
+    before = op.info()["device_bytes"]
+    ids = torch.arange(9001, device="cuda", dtype=torch.int32)
+    op.set_blocks(ids % 3, 3)
+    three = op.info()
+    assert three["device_bytes"] - before >= 16 * three["n_items"]
+    a = op.solve(y, P["eps"], **kw)
+    op.set_blocks(ids % 7, 7)
+    b = op.solve(y, P["eps"], **kw)
+    op.set_blocks(0 * ids, 1)
+    again = op.solve(y, P["eps"], **kw)
+    assert rel(host(again.x), host(one.x)) < {"fp32": 1e-5, "fp64": 1e-11}[prec]
+    for r in (a, b):
+        assert rel(host(r.x), host(one.x)) < 0.1  # the same data within per-block bounds
+    op.close()
