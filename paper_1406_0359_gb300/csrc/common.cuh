@@ -221,14 +221,12 @@ template <typename A> struct ArgVal {
   A a;
   PD const A& get() const { return a; }
   PD const A& get_at(int) const { return a; }
-  PD int inst() const { return 0; }
 };
 template <typename A> struct ArgTab {
   static constexpr bool kTable = true;
   const A* t;
   PD A get() const { return t[blockIdx.y]; }
   PD A get_at(int i) const { return t[i]; }
-  PD int inst() const { return int(blockIdx.y); }
 };
 
 

@@ -246,15 +246,6 @@ PD void fft_seq(int t, C* s, int ss, const C* tw, int dir, Load load, Store stor
   run_stages<LOGN, 0, E>(v, t, 1, s, ss, tw, dir, store);
 }
 
-// Output position of the cnt-th value a thread's final stage hands to its
-// sink: the final radix-R stage has Ns = K/R and butterflies j = t + q T < Ns,
-// so its outputs come in the order (q, r) at t + q T + r K/R.
-template <int LOGN, int E = 16> PD int last_pos(int t, int cnt) {
-  typedef Plan<LOGN, E> P;
-  constexpr int R = P::radix(P::NST - 1);
-  return t + (cnt / R) * P::T + (cnt % R) * (P::N / R);
-}
-
 constexpr int kRowCta = 256;  // threads per CTA of the plain row transforms
 
 // Column passes read kColBytes contiguous bytes of each row: col_width

@@ -69,13 +69,6 @@ template <typename T> PD void kb_eval(const KbPoly<T>& kb, T f, T (&w)[kJ]) {
   }
 }
 
-template <typename C> PD void atomic_add_global(C* p, C v);
-template <> PD void atomic_add_global<float2>(float2* p, float2 v) { atomicAdd(p, v); }
-template <> PD void atomic_add_global<double2>(double2* p, double2 v) {
-  atomicAdd(&p->x, v.x);
-  atomicAdd(&p->y, v.y);
-}
-
 // One lane's staged visibility record (kGrRec values)
 // written as 16-byte vectors: at the 80-byte (FP32) lane stride each
 // quarter-warp's vector stores hit distinct bank groups, where scalar stores at
@@ -386,8 +379,10 @@ PD void atomic_add_pair(float2* p, float2 a, float2 b) {
   atomicAdd(reinterpret_cast<float4*>(p), make_float4(a.x, a.y, b.x, b.y));
 }
 PD void atomic_add_pair(double2* p, double2 a, double2 b) {
-  atomic_add_global(p, a);
-  atomic_add_global(p + 1, b);
+  atomicAdd(&p[0].x, a.x);
+  atomicAdd(&p[0].y, a.y);
+  atomicAdd(&p[1].x, b.x);
+  atomicAdd(&p[1].y, b.y);
 }
 
 template <typename T, typename Src>
@@ -473,7 +468,8 @@ __global__ void __launch_bounds__(32 * kWItems) k_grid_w(Src src, KbPoly<T> kb) 
     }
     __syncwarp();
     const int nj = min(kGrLanes, per - b);
-    constexpr unsigned kFirst = kGroups == 4 ? 0x01010101u : (kGroups == 2 ? 0x00010001u : 1u);
+    static_assert(kGroups == 2, "the first record of either group");
+    constexpr unsigned kFirst = 0x00010001u;
 #pragma unroll 4
     for (int j = 0; j < nj; ++j) {
       if (changes & (kFirst << j)) {

@@ -431,7 +431,6 @@ template <typename T> struct SynArgs {
   int fid[kMaxDb];  // Daubechies filter (K - 1) of each filter slot
   T scale;          // 1 / sqrt(number of bases)
   // finest level (fused over filters):
-  int fused;
   int pos_block;    // apply the positivity block
   T* x_out;
   const T* xh;
@@ -928,7 +927,6 @@ SynPlan<T> plan_synthesis(const SaraPlan<T>& P, const T* c, T* x, int pos_block,
   S.H = n / 2;
   S.n = n;
   select(S);
-  S.fused = 1;
   S.pos_block = pos_block;
   S.x_out = x;
   S.xh = xh;

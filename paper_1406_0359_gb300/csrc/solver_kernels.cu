@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kFinT) k_finalize_blocks(const double* __restr
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int j = i + u * kFinT;
-        in[u] = R == 1 || item_block[4 * j] == b;  // WorkItem::pad
+        in[u] = item_block[4 * j] == b;  // WorkItem::pad
         x[u] = p0[j];
         y[u] = p1[j];
       }
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kFinT) k_finalize_blocks(const double* __restr
         }
     }
     for (; i < n_items; i += kFinT) {
-      if (R == 1 || item_block[4 * i] == b) {
+      if (item_block[4 * i] == b) {
         acc_merge(a, p0[i]);
         acc_merge(c, p1[i]);
       }
