@@ -342,8 +342,11 @@ int purify_batch_solve(int count, purify_op* const* ops, const void* const* y, c
  *   convergence state, nu, gamma, the first reweighting delta, the last
  *   objective) followed by x_hat, sum_i x_i, z_1, z_2, the SARA weights W and
  *   z_3 (reals of the operator's precision; z_3 in the order of a stable
- *   sort by (block, uv tile, cell) over the whole grid).  CG vectors are not state: every SDMM iteration
- *   restarts its CG from x_hat.
+ *   sort by (block, uv tile, cell) over the whole grid).  CG vectors are not
+ *   state: every SDMM iteration restarts its CG from x_hat.  Saving and loading
+ *   bring z_3 into and out of that order with scratch from the set-up pool (up
+ *   to 37 bytes a visibility in FP32, 53 in FP64); PURIFY_ERR_NOMEM without it,
+ *   with the solve as it was.
  * purify_solve_load -- after purify_solve_begin with the same y and
  *   parameters, replace the fresh state by a saved one; the next
  *   purify_solve_step continues where the saved solve stopped.

@@ -1441,14 +1441,17 @@ template <typename T> class OpImpl : public purify_op {
     C* z3f = nullptr;
     CK(setup_alloc(&z3f, size_t(g.M) * sizeof(C), own));
     CK(cudaStreamSynchronize(own));
-    int rcl = PURIFY_OK;
-    for (int k = 0; k < na && !rcl; ++k) {
-      T* to = k == kStateZ3 ? reinterpret_cast<T*>(z3f) : a[k];
-      rcl = map_err(cudaMemcpy(to, src, len[k] * sizeof(T), cudaMemcpyHostToDevice), __LINE__);
-      src += len[k] * sizeof(T);
-    }
+    // z_3 first: its reordering takes scratch, and a load that fails for memory
+    // leaves the solve as it was
+    size_t at = 0;
+    for (int k = 0; k < kStateZ3; ++k) at += len[k] * sizeof(T);
+    int rcl = map_err(cudaMemcpy(z3f, src + at, len[kStateZ3] * sizeof(T), cudaMemcpyHostToDevice), __LINE__);
     if (!rcl) rcl = checkpoint_z3(z3f, false);
     cudaFreeAsync(z3f, own);
+    for (int k = 0; k < na && !rcl; ++k) {
+      if (k != kStateZ3) rcl = map_err(cudaMemcpy(a[k], src, len[k] * sizeof(T), cudaMemcpyHostToDevice), __LINE__);
+      src += len[k] * sizeof(T);
+    }
     if (rcl) return rcl;
     run.round = h.round;
     run.t = h.t;
