@@ -27,14 +27,16 @@ namespace purify {
 
 namespace {
 
-// Let the next pass's CTAs start.  Not in FP64: those passes are bound by the
-// FP64 units, and CTAs that start early pile up on the SMs that finish first,
-// which then take twice as long while others idle (one to three CTAs an SM:
-// Phi^H Phi at n = 512 207 us with the trigger, 124 without, 131 by plain
-// launches; Phi at 512 226 / 194 / 198, at 256 87 / 76 / 93, the rest equal).
-// The next launch then waits for the last CTA's end, its set-up already done.
-template <typename T> PD void pass_trigger() {
-  if constexpr (sizeof(T) == 4) pdl_trigger();
+// Let the next pass's CTAs start.  Not in FP64 from image side 512 on (the grid's
+// column passes: 256): those passes are bound by the FP64 units, and CTAs that
+// start early pile up on the SMs that finish first, which then take twice as
+// long while others idle (one to three CTAs an SM).  With the trigger, without,
+// by plain launches: Phi^H Phi at n = 512 207, 124, 131 us, at 256 43.3, 43.9, 52;
+// Phi at 512 / 131072 points 226, 194, 198, at 256 / 65536 112, 94, -.  Without it
+// the next launch waits for the last CTA's end, its set-up already done; smaller
+// images lose that wait (an SDMM iteration at 128^2 629 -> 638 us).
+template <typename T, int LOGN, int LARGEST = 8> PD void pass_trigger() {
+  if constexpr (sizeof(T) == 4 || LOGN <= LARGEST) pdl_trigger();
 }
 
 template <typename C> PD C cneg(C a) { a.x = -a.x; a.y = -a.y; return a; }
@@ -736,7 +738,7 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
 #pragma unroll
   for (int m = 0; m < E; ++m) s[t + m * TT] = v[m];
   __syncthreads();
-  pass_trigger<T>();
+  pass_trigger<T, LOGN>();
   // separate the pairs: column c = 2m + odd from elements m and -m of its half
   constexpr int PC = sizeof(T) == 4 ? 2 : 1;  // pairs per 32-byte store
   static_assert(H::PAIRS % PC == 0, "whole sectors");
@@ -819,7 +821,7 @@ __global__ void __launch_bounds__(ColHalf<T, LOGN>::COL_THREADS, ColHalf<T, LOGN
   }
   half_fft<H, 1>(v, t, s, half, a.tws);
   if (odd) half_omega<H, 1>(v, t, tw);
-  pass_trigger<T>();
+  pass_trigger<T, LOGN>();
   half_join<H>(v, t, odd, bufs, half, Bc);
 }
 
@@ -995,7 +997,7 @@ __global__ void __launch_bounds__(RowHalf<T, LOGN>::ROW_THREADS, RowHalf<T, LOGN
   bool ok = true;
   if (nop > 0) ok = mbar_wait_bounded(&bar, 0, ep.err);
   __syncthreads();
-  pass_trigger<T>();
+  pass_trigger<T, LOGN>();
   EpAcc<T> part;
   if (ok) part = row_ep_all<LOGN>(ep, bufs, ops, a.deapod, r0);
   row_ep_finish(ep, part, red);
@@ -1055,7 +1057,7 @@ __global__ void __launch_bounds__(GridHalf<T, LOGN>::NT, GridHalf<T, LOGN>::MINB
     for (int m = 0; m < E; ++m) s[t + m * TT] = v[m];
   }
   __syncthreads();
-  pass_trigger<T>();
+  pass_trigger<T, LOGN, 7>();
   for (int q = threadIdx.x; q < K; q += H::NT) {
     const int o = q & 1, m = q >> 1;
     C out[NC], col0 = cz<C>();
@@ -1161,7 +1163,7 @@ __global__ void __launch_bounds__(GridHalf<T, LOGN>::NT, GridHalf<T, LOGN>::MINB
   half_sync<TT>(half);
   half_fft<H, 1>(v, t, s, half, a.tws);
   if (odd) half_omega<H, 1>(v, t, a.tw);
-  pass_trigger<T>();
+  pass_trigger<T, LOGN, 7>();
   const int c = c0 + (half >> 1);
   half_join<H>(v, t, odd, bufs, half, a.B + (c == n ? size_t(0) : half_at(c, 0, n)));
 }

@@ -161,10 +161,10 @@ __device__ void ana_body(const AnaArgs<T>& A, const T* __restrict__ h, const T* 
     }
   }
   __syncthreads();
-  // FP64 levels are bound by the FP64 units: the next level's CTAs, started
+  // Large FP64 levels are bound by the FP64 units: the next level's CTAs, started
   // early, pile up on the SMs that finish first (Db8, 4 levels, n = 512: 87 us
   // against 75); after the last level whatever follows may start
-  if (sizeof(T) == 4 || A.last) pdl_trigger();
+  if (sizeof(T) == 4 || A.n <= 256 || A.last) pdl_trigger();
   Acc<T> part;
   const int r = threadIdx.x / kTH, c = threadIdx.x - r * kTH;
   const int R = r0 + r, Cc = c0 + c;
