@@ -82,7 +82,7 @@ int purify_op_create(const double* uv, int64_t M, int n, int oversample, int J,
 typedef struct {
   int tile;   /* uv tile side in grid cells: 8 (default) or 16 */
   int chunk;  /* visibilities per work item, 64..8192 (default by M: 128 below 2^20 --
-                 FP64 64 below 2^18 -- else 512) */
+                 FP64 64 below 2^14 -- else 512) */
 } purify_op_options;
 
 /* purify_op_create_ex -- purify_op_create with an explicit tile / chunk. */

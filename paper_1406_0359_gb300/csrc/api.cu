@@ -441,10 +441,11 @@ template <typename T> class OpImpl : public purify_op {
     // 33 at 256, 50 at 1024) and end a large one together (512^2 / 4M: 110 at
     // 256..1024, 149 at 2048; 1024^2 / 4M: 150..154 at 256..2048).  FP64 takes
     // about 10 us for each 32 visibilities of an item's walk: half as long below
-    // 2^18, where the items do not fill the chip (NUFFT-form Phi^H Phi at 32^2 /
-    // 512 points 99 us at 64, 146 at 128; 256^2 / 131072 262 / 280; 512^2 /
-    // 393217 728 / 720).
-    const int64_t half = sizeof(T) == 8 ? int64_t(1) << 18 : 0;
+    // 2^14, where the items do not fill the chip (NUFFT-form Phi^H Phi at 32^2 /
+    // 512 points 99 us at 64, 146 at 128; at 128^2 / 12000 Phi 44 / 63).  Above,
+    // a solve, whose branches fill the chip together, loses (an SDMM iteration at
+    // 256^2 / 65536 886 / 823) although Phi alone still gains.
+    const int64_t half = sizeof(T) == 8 ? int64_t(1) << 14 : 0;
     chunk = chunk_opt > 0 ? chunk_opt : (M < half ? 64 : (M < (int64_t(1) << 20) ? 128 : 512));
     if (!light) {  // a set-up operator runs only on the caller's stream
       // the ball block is the longer branch of an iteration: its kernels'

@@ -1,5 +1,5 @@
 """The default work-item length: FP64 items are half as long as FP32's below
-2^18 points (a warp walks an item alone, and in FP64 the walk is the time), and
+2^14 points (a warp walks an item alone, and in FP64 the walk is the time), and
 the operators agree with the oracle when one tile's items meet at its cells."""
 import numpy as np
 import pytest
