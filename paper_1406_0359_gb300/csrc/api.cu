@@ -1913,13 +1913,14 @@ int batch_solve(int count, purify_op* const* ops_in, const void* const* y, const
   auto cg_operator = [&](int i) -> int {
     OpImpl<T>* o = b.ops[i];
     if (o->khat) return PURIFY_OK;
+    int rc = o->ensure_solver();  // (its allocations wait for the stream: before the set-up, not behind it)
+    if (rc) return rc;
     const size_t need = o->toeplitz_scratch();
     for (; oldest < held.size() && in_flight + need > limit; ++oldest) {
       CK(cudaStreamWaitEvent(o->own, b.ops[held[oldest].first]->ev_out, 0));
       in_flight -= held[oldest].second;
     }
-    const int rc = o->ensure_toeplitz(o->own);
-    if (rc) return rc;
+    if ((rc = o->ensure_toeplitz(o->own))) return rc;
     CK(cudaEventRecord(o->ev_out, o->own));
     held.emplace_back(i, need);
     in_flight += need;
