@@ -135,8 +135,8 @@ PD bool warp_stage_patch(C* patch, uint64_t* bar, const CUtensorMap* map, int tu
 // Degridding: one lane per visibility, its kernel weights in registers, its
 // J x J cells gathered from the warp's staged patch; visibilities are sorted by
 // cell, so a warp's lanes read neighbouring cells.  Bound by the shared-memory
-// pipe -- 64 cells of 8 bytes at 128 bytes a clock are 4 cycles per visibility --
-// and instruction issue (14 warp instructions), both near 70%.  The form with
+// pipe: 64 cells of 8 bytes at 128 bytes a clock are 4 cycles per visibility, the
+// pipe is 85% busy and issue, with the taps as packed pairs, 53%.  The form with
 // four lanes per visibility staged every weight through shared memory and
 // summed by shuffles, 7.8 cycles: 141 us a launch against 80 (1024^2,
 // M = 4,194,304).
@@ -270,8 +270,8 @@ __global__ void __launch_bounds__(32 * kWItems) k_degrid_w(Src src, KbPoly<T> kb
 // stays the same, and adds the run to the group's own patch of plain cells in
 // shared memory (no atomics, nothing shared between groups) when it changes.
 // The patches are merged at the end, one vector atomic per two cells.  Two
-// visibilities take 4 shared-memory cycles and 8 FMAs a lane; bound by
-// instruction issue (72%) and the shared-memory pipe (60%).  One visibility at
+// visibilities take 8 FMAs a lane; bound by instruction issue (70%) and the
+// shared-memory pipe (69%, some 6 cycles a visibility).  One visibility at
 // a time on 32 lanes took 165 us a launch, this form 115 (1024^2, M =
 // 4,194,304, half grid); four groups of 8 lanes win where cells are full (512^2:
 // 128 against 149 us for Phi^H) but hold 16 warps an SM and lose elsewhere (187
